@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -1040,19 +1041,24 @@ static ts_status bfs_step(const ts_csr_desc* A, const ts_csr_desc* F, uint32_t* 
     TS_CUDA(launch_msbfs_step(dev(A), dev(F), (int)d, visited, levels, level, sc, newbits,
                               (long long*)F_next->rowptr, cfg, st, fbits, parents),
             fn);
-    long long tot = 0;
-    TS_CUDA(cudaMemcpyAsync(&tot, (long long*)F_next->rowptr + n, sizeof tot, cudaMemcpyDeviceToHost, st), fn);
-    unsigned long long err = 0;
-    TS_CUDA(cudaMemcpyAsync(&err, &sc.hdr->err, sizeof err, cudaMemcpyDeviceToHost, st), fn);
+    // queued before the count is read, so that the read-out does not wait for
+    // the host; it writes nothing when F_next is too small
+    TS_CUDA(launch_msbfs_emit(n, (int)d, newbits, (const long long*)F_next->rowptr, F_next->col,
+                              F_next_capacity, sc.hdr, st),
+            fn);
+    struct {
+        unsigned long long err;
+        long long total;
+    } got = {0, 0};
+    static_assert(offsetof(WsHeader, total) == offsetof(WsHeader, err) + sizeof got.err, "read in one copy");
+    TS_CUDA(cudaMemcpyAsync(&got, &sc.hdr->err, sizeof got, cudaMemcpyDeviceToHost, st), fn);
     TS_CUDA(cudaStreamSynchronize(st), fn);
-    if (err) return fail(TS_ERR_BAD_CSR, "%s: device checks failed (flags 0x%llx)", fn, err);
+    const long long tot = got.total;
+    if (got.err) return fail(TS_ERR_BAD_CSR, "%s: device checks failed (flags 0x%llx)", fn, got.err);
     *nnz_next_host = tot;
     if (tot > F_next_capacity)
         return fail(TS_ERR_CAPACITY, "%s: next frontier has %lld entries, capacity %lld", fn, tot,
                     (long long)F_next_capacity);
-    TS_CUDA(launch_msbfs_emit(n, (int)d, newbits, (const long long*)F_next->rowptr, F_next->col,
-                              F_next_capacity, sc.hdr, st),
-            fn);
     return ok();
 }
 

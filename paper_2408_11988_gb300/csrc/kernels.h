@@ -70,6 +70,10 @@ cudaError_t launch_symbolic(const DevCsr& A, const DevCsr& B, long long d, const
 
 // In-place inclusive scan of x[0..n) (int64) using partial[] as scratch.
 cudaError_t launch_scan_inplace(long long* x, long long n, long long* partial, cudaStream_t st);
+// The same when partial[t] already holds the sum of x over tile t of
+// scan_tile_rows() values (left by the kernel that wrote x).
+cudaError_t launch_scan_summed(long long* x, long long n, long long* partial, cudaStream_t st);
+int scan_tile_rows();
 
 // Column-tile offsets: tp[k*(T+1)+t] = first position of row k of B with
 // column >= t*W (t = 0..T; t = T gives the row end).

@@ -46,6 +46,7 @@ struct WsHeader {
     unsigned long long heavy_ctr;     // next heavy row (dynamic CTA scheduling)
     unsigned long long item_ctr;      // next split-row work item
     unsigned long long err;           // ERR_* bits
+    long long total;                  // multi-source BFS: entries of the next frontier (read with err)
     long long hist[NUM_CLASSES];      // rows per flops class
     long long cursor[NUM_CLASSES];    // scatter cursors per class
     long long scratch[8];             // [0] flops items, [1] split rows, [2] split items

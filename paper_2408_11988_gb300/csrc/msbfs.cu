@@ -2,9 +2,10 @@
 //   N = A * F over (or, select2nd);  F_next = N minus S;  S = S or N;
 // fused into one gather pass per row (the boolean TS-SpGEMM with a d-bit
 // accumulator), a scan for F_next's row pointers and a read-out of the new
-// bits.  Rows whose visited set is already full cannot gain bits and are not
-// scheduled at all; rows whose neighbours have empty frontier rows have no
-// products and are skipped by the flops binning.
+// bits.  For d <= 256 the frontier is expanded to a bitmap and rows pull from
+// it (the pull form below); above that the list form walks F's rows, heaviest
+// rows first, and skips rows whose visited set is full and rows whose
+// neighbours have empty frontier rows.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -63,6 +64,7 @@ struct BfsParams {
     const int* perm;
     WsHeader* hdr;
     int cta_class;
+    long long n;
 };
 
 // Given the OR of the neighbours' frontier rows in bm (dw words), keep the
@@ -147,46 +149,49 @@ __global__ void __launch_bounds__(1024) k_msbfs_expand(BfsParams p) {
     }
 }
 
-// F_next columns from the stored new bits; one thread per row, rows without
-// new bits (this level's count is 0) are skipped, so stale words of rows not
-// scheduled this level are never read.
-__global__ void k_msbfs_emit(long long n, int dw, const unsigned* __restrict__ newbits,
-                             const long long* __restrict__ rp, int* __restrict__ col, long long cap,
-                             unsigned long long* err) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    long long pos = rp[i];
-    const long long end = rp[i + 1];
-    if (end <= pos) return;
-    for (int w = 0; w < dw; ++w) {
-        unsigned word = newbits[i * dw + w];
-        while (word) {
-            const int b = __ffs(word) - 1;
-            word &= word - 1;
-            if (pos < end && pos < cap) col[pos] = 32 * w + b;
-            else atomicOr(err, ERR_CAPACITY);
-            ++pos;
-        }
-    }
-}
-
 // Initial frontier and visited/level state from d sources (distinct vertices;
-// a repeated vertex simply holds several columns).  Thread per vertex for the
-// row pointers (counting the sources at or below it), thread per source for
-// the columns.
-__global__ void k_msbfs_init_rows(long long n, int d, const int* __restrict__ src, long long* rp) {
-    const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v > n) return;
-    if (v == 0) {
-        rp[0] = 0;
-        return;
-    }
-    long long c = 0;  // rp[v] = number of (valid) sources at vertices < v
-    for (int s = 0; s < d; ++s) {
+// a repeated vertex simply holds several columns).  Row pointers: a block
+// takes 1024 vertices, counts the sources below them once and keeps those
+// among them in shared memory, where every vertex counts the ones at or
+// below it (a thread per vertex over all d sources took 39 us for 2^20
+// vertices and 128 sources).  Columns: a thread per source.
+constexpr int INIT_ROWS = 1024;
+__global__ void __launch_bounds__(256) k_msbfs_init_rows(long long n, int d, const int* __restrict__ src,
+                                                         long long* rp) {
+    __shared__ int s_here[INIT_ROWS];  // sources at each of the block's vertices, then their running sum
+    __shared__ int s_below, s_w[8];
+    const int tid = threadIdx.x, lane = lane_id(), warp = warp_id();
+    const long long base = (long long)blockIdx.x * INIT_ROWS;
+    for (int i = tid; i < INIT_ROWS; i += 256) s_here[i] = 0;
+    if (tid == 0) s_below = 0;
+    __syncthreads();
+    int below = 0;
+    for (int s = tid; s < d; s += 256) {
         const int u = __ldg(src + s);
-        c += (u >= 0 && (long long)u < v) ? 1 : 0;
+        if (u < 0) continue;
+        if ((long long)u < base) ++below;
+        else if ((long long)u < base + INIT_ROWS) atomicAdd(&s_here[u - (int)base], 1);
     }
-    rp[v] = c;
+    below = warp_sum(below);
+    if (lane == 0 && below) atomicAdd(&s_below, below);
+    __syncthreads();
+    // vertices 4 tid .. 4 tid + 3 of the block
+    int c[4], run = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        c[q] = run;
+        run += s_here[4 * tid + q];
+    }
+    const int incl = warp_incl_scan(run);
+    if (lane == 31) s_w[warp] = incl;
+    __syncthreads();
+    int before = s_below + incl - run;
+    for (int w = 0; w < warp; ++w) before += s_w[w];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {  // rp[v] = sources at vertices < v
+        const long long v = base + 4 * tid + q;
+        if (v <= n) rp[v] = before + c[q];
+    }
 }
 
 __global__ void k_msbfs_init_cols(long long n, int d, int dw, const int* __restrict__ src, int* col,
@@ -208,224 +213,668 @@ __global__ void k_msbfs_init_cols(long long n, int d, int dw, const int* __restr
 
 
 // ---------------------------------------------------------------------------
-// Pull expansion with the frontier as a bitmap (the dense-frontier form of
-// Alg. 3's N = A * F): F is first written as DWP words per row (d <= 256,
-// DWP = dw rounded up to a power of two), then row v ORs the bitmap rows of
-// its neighbours, one load of DWP words per entry of A, instead of gathering
-// each neighbour's list of frontier columns.  The cost per entry no longer
-// grows with the frontier's density.  The OR, the visited mask, the level
-// write and the new-bit words are those of the list form.
+// Pull form (d <= 256): the frontier as a bitmap of DWP words per vertex (dw
+// rounded up to a power of two), and row v of N = A * F the OR of its
+// neighbours' bitmap rows, one load of DWP words per entry of A whatever the
+// frontier's density.  A level is bound by those gathers (the bitmap stays in
+// L2: 16 MB for 2^20 vertices and 128 sources) and by the latency of long
+// rows, so:
+//  - rows are taken in their own order, 32 (fewer when there are few rows) to
+//    a warp, with no flops pass, classes or permutation before (these cost
+//    180 us a level at scale 20): a row of at most BFS_SHORT entries by its
+//    lane, a longer one by the whole warp, 64 or 128 entries at a time, and one
+//    above BFS_HEAVY by blocks of BFS_CHUNK entries in a kernel of its own
+//    (a hub's row in one warp took 0.8 - 1.1 ms of each of the first levels);
+//  - a row stops gathering once its unvisited sources are all found, which in
+//    the dense levels is after the first few neighbours, and a row whose
+//    sources are all found is not read (A's columns are range-checked as a
+//    stream beside the frontier's expansion, whatever the rows need of them);
+//  - while F holds fewer entries than n / BFS_SPARSE, a bit per vertex says
+//    whether its frontier row is empty, and empty ones are not gathered (the
+//    bits of 2^20 vertices are 128 KB and stay in L1).
+// The whole 128-source search of the scale-20 graph: 5.9 -> 2.4 ms; the BFS
+// trees of 50 sources over 300,007 vertices: 2.94 -> 1.19 ms.
 // ---------------------------------------------------------------------------
-template <int DWP>
-__global__ void __launch_bounds__(256) k_frontier_bits(long long n, int d, const long long* __restrict__ Fp,
-                                                       long long nnzF, const int* __restrict__ Fi,
-                                                       unsigned* __restrict__ fb, unsigned long long* err) {
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-         v += (long long)gridDim.x * blockDim.x) {
-        unsigned w[DWP];
-#pragma unroll
-        for (int m = 0; m < DWP; ++m) w[m] = 0u;
-        const long long s = clampll(__ldg(Fp + v), 0, nnzF), e = clampll(__ldg(Fp + v + 1), s, nnzF);
-        for (long long j = s; j < e; ++j) {
-            const int c = __ldg(Fi + j);
-            if ((unsigned)c < (unsigned)d) {
-#pragma unroll
-                for (int m = 0; m < DWP; ++m) w[m] |= (c >> 5) == m ? 1u << (c & 31) : 0u;
-            } else {
-                atomicOr(err, ERR_B_COL);
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < DWP; ++m) fb[v * DWP + m] = w[m];
-    }
-}
+constexpr int BFS_SHORT = 16;
+constexpr int BFS_HEAVY = 2048;
+constexpr int BFS_CHUNK = 4096;
+constexpr int BFS_SPARSE = 4;
 
-// OR of the frontier bitmap rows of entries [e0, e1) of A, lane-strided.
+// Bitmap rows of F and the bits of the non-empty ones; also clears what the
+// level accumulates (scan partials) and C's first row pointer.  A warp takes
+// 32 vertices, whose entries follow each other in F: 128 entries a step, four
+// per lane with one 16-byte load, the row of a lane's first entry by a search
+// of the warp's row starts in shared memory, and the bits of neighbouring
+// entries of one word gathered before one OR into the warp's words in shared
+// memory.  (A thread per row took 127 us for a frontier of 57 million entries
+// over 2^20 vertices, its lines thrown out of L1 before they were used up;
+// this way 106 us, the check of A's 31 million columns included.)
+//
+// The blocks behind the first nfront range-check A's columns, so that the
+// pull may leave out rows and ends of rows with nothing left to find: a
+// stream over A beside the decoding (30 us in all where the frontier is small).
+constexpr int CHECK_PER_BLOCK = 16384;
 template <int DWP>
-__device__ __forceinline__ void pull_or(const BfsParams& p, const unsigned* __restrict__ fb, long long e0,
-                                        long long e1, int t0, int nt, unsigned acc[DWP], unsigned long long* err) {
-    // unrolled so that several neighbours' rows are in flight per thread; a
-    // bad column reads row 0 and contributes nothing (keep = 0)
+__global__ void __launch_bounds__(256) k_bfs_frontier(long long n, int d, const long long* __restrict__ Fp,
+                                                      long long nnzF, const int* __restrict__ Fi,
+                                                      unsigned* __restrict__ fb, unsigned* __restrict__ nonempty,
+                                                      long long* partial, long long npartial, long long* rp_next,
+                                                      unsigned nfront, const long long* __restrict__ Ap,
+                                                      const int* __restrict__ Ai, long long nnzA,
+                                                      unsigned long long* err) {
+    const int lane = lane_id(), warp = warp_id();
+    if (blockIdx.x >= nfront) {
+        const long long lo = clampll(__ldg(Ap), 0, nnzA), hi = clampll(__ldg(Ap + n), lo, nnzA);
+        const long long b0 = (long long)(blockIdx.x - nfront) * CHECK_PER_BLOCK;
+        const long long first = b0 > lo ? b0 : lo;
+        const long long last = b0 + CHECK_PER_BLOCK < hi ? b0 + CHECK_PER_BLOCK : hi;
+        bool bad = false;
+        if (last - first == CHECK_PER_BLOCK && !(reinterpret_cast<uintptr_t>(Ai) & 15)) {
+            const int4* q = reinterpret_cast<const int4*>(Ai + first);  // first is a multiple of four
 #pragma unroll 4
-    for (long long e = e0 + t0; e < e1; e += nt) {
-        int u = __ldg(p.Ai + e);
-        unsigned keep = FULL;
-        if ((unsigned)u >= (unsigned)p.nF) {
-            atomicOr(err, ERR_A_COL);
-            u = 0;
-            keep = 0u;
-        }
-        const unsigned* r = fb + (long long)u * DWP;
-        if constexpr (DWP >= 4) {
-#pragma unroll
-            for (int m = 0; m < DWP; m += 4) {
-                const uint4 x = __ldg(reinterpret_cast<const uint4*>(r + m));
-                acc[m] |= x.x & keep;
-                acc[m + 1] |= x.y & keep;
-                acc[m + 2] |= x.z & keep;
-                acc[m + 3] |= x.w & keep;
+            for (int i = threadIdx.x; i < CHECK_PER_BLOCK / 4; i += 256) {
+                const int4 c = __ldg(q + i);
+                const unsigned x = max(max((unsigned)c.x, (unsigned)c.y), max((unsigned)c.z, (unsigned)c.w));
+                bad |= x >= (unsigned)n;
             }
         } else {
-#pragma unroll
-            for (int m = 0; m < DWP; ++m) acc[m] |= __ldg(r + m) & keep;
+            for (long long e = first + threadIdx.x; e < last; e += 256) bad |= (unsigned)__ldg(Ai + e) >= (unsigned)n;
         }
+        if (bad) atomicOr(err, ERR_A_COL);
+        return;
+    }
+    __shared__ unsigned s_bits[8][32 * DWP];
+    __shared__ int s_start[8][33];
+    const long long base = ((long long)blockIdx.x * 8 + warp) * 32, v = base + lane;
+    for (long long x = (long long)blockIdx.x * 256 + threadIdx.x; x < npartial; x += 256LL * nfront) partial[x] = 0;
+    if (v == 0) rp_next[0] = 0;
+    unsigned* bits = s_bits[warp];
+    int* start = s_start[warp];
+#pragma unroll
+    for (int m = 0; m < DWP; ++m) bits[32 * m + lane] = 0u;
+    if (base >= n) return;
+    const long long s = clampll(__ldg(Fp + (v < n ? v : n)), 0, nnzF);
+    const long long e0 = shfl64(s, 0);
+    const long long e1 = clampll(__ldg(Fp + (base + 32 < n ? base + 32 : n)), e0, nnzF);
+    const int total = (int)(e1 - e0 < (1LL << 30) ? e1 - e0 : 1LL << 30);  // at most 32 d in a well-formed F
+    start[lane] = (int)clampll(s - e0, 0, total);
+    if (lane == 0) start[32] = total;
+    __syncwarp();
+    const int* f = Fi + e0;
+    const int lead = (int)((reinterpret_cast<uintptr_t>(f) >> 2) & 3);  // entries of the first 16 bytes before f
+    bool bad = false;
+    for (int i0 = -lead; i0 < total; i0 += 128) {
+        const int i = i0 + 4 * lane;
+        if (i >= total) continue;
+        int c[4];
+        if (i >= 0 && i + 4 <= total) {
+            const int4 x = __ldg(reinterpret_cast<const int4*>(f + i));
+            c[0] = x.x;
+            c[1] = x.y;
+            c[2] = x.z;
+            c[3] = x.w;
+        } else {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) c[t] = i + t >= 0 && i + t < total ? __ldg(f + i + t) : 0;
+        }
+        int r = 0;  // last row starting at or before the lane's first entry
+        const int at = i > 0 ? i : 0;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1)
+            if (start[r + o] <= at) r += o;
+        int word = -1;
+        unsigned x = 0u;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (i + t < 0 || i + t >= total) continue;
+            while (r < 31 && i + t >= start[r + 1]) ++r;
+            if ((unsigned)c[t] >= (unsigned)d) {
+                bad = true;
+                continue;
+            }
+            const int w = r * DWP + (c[t] >> 5);
+            if (w != word) {
+                if (x) atomicOr(bits + word, x);
+                word = w;
+                x = 0u;
+            }
+            x |= 1u << (c[t] & 31);
+        }
+        if (x) atomicOr(bits + word, x);
+    }
+    __syncwarp();
+    unsigned any = 0u;
+#pragma unroll
+    for (int m = 0; m < DWP; ++m) any |= bits[lane * DWP + m];
+    const unsigned ne = __ballot_sync(FULL, any != 0u);
+    if (lane == 0) nonempty[base >> 5] = ne;
+    // the 32 rows' words, contiguous in fb
+#pragma unroll
+    for (int m = 0; m < DWP; ++m)
+        if (32 * m + lane < (n - base) * DWP) fb[base * DWP + 32 * m + lane] = bits[32 * m + lane];
+    if (bad) atomicOr(err, ERR_B_COL);
+}
+
+// Bitmap row of vertex u.
+template <int DWP>
+__device__ __forceinline__ void bfs_row(const unsigned* __restrict__ fb, int u, unsigned w[DWP]) {
+    const unsigned* r = fb + (long long)u * DWP;
+    if constexpr (DWP >= 4) {
+#pragma unroll
+        for (int m = 0; m < DWP; m += 4) {
+            const uint4 x = __ldg(reinterpret_cast<const uint4*>(r + m));
+            w[m] = x.x;
+            w[m + 1] = x.y;
+            w[m + 2] = x.z;
+            w[m + 3] = x.w;
+        }
+    } else if constexpr (DWP == 2) {
+        const uint2 x = __ldg(reinterpret_cast<const uint2*>(r));
+        w[0] = x.x;
+        w[1] = x.y;
+    } else {
+        w[0] = __ldg(r);
     }
 }
 
-// Settle row `row` from the OR of its neighbours (all lanes of the warp hold
-// the full OR): new = N and not S; S |= new; new bits stored for the
-// read-out; levels written, lane l taking bit l of every word.  Returns the
-// number of new bits (all lanes).
-template <int DWP>
-__device__ __forceinline__ int pull_settle(const BfsParams& p, long long row, const unsigned acc[DWP],
-                                           unsigned nws[DWP]) {
-    const int lane = lane_id();
-    int c = 0;
-#pragma unroll
-    for (int m = 0; m < DWP; ++m) {
-        nws[m] = 0u;
-        if (m >= p.dw) continue;
-        const int bits = p.d - 32 * m;
-        const unsigned valid = bits >= 32 ? FULL : ((1u << bits) - 1u);
-        const unsigned old = __ldg(p.S + row * p.dw + m);
-        const unsigned nw = acc[m] & ~old & valid;
-        nws[m] = nw;
-        if (lane == 0) {
-            p.newbits[row * p.dw + m] = nw;
-            if (nw) p.S[row * p.dw + m] = old | nw;
-        }
-        if ((nw >> lane) & 1u) p.levels[row * p.d + 32 * m + lane] = p.level;
-        c += __popc(nw);
+// A's columns as the pull reads them: load() gives the neighbour of entry e
+// (-1 for none, or for a column outside [0, n), which k_bfs_frontier's check
+// reports), hit() whether its frontier row is to be gathered.
+struct BfsCols {
+    const int* __restrict__ Ai;
+    const unsigned* __restrict__ nonempty;  // nullptr: gather every neighbour
+    int nF;
+    __device__ __forceinline__ int load(long long e, bool in) const {
+        const int u = in ? __ldg(Ai + e) : -1;
+        return (unsigned)u < (unsigned)nF ? u : -1;
     }
-    return c;
+    __device__ __forceinline__ bool hit(int u) const {
+        return u >= 0 && (!nonempty || ((__ldg(nonempty + (u >> 5)) >> (u & 31)) & 1u));
+    }
+};
+
+// Transpose of a 32 x 32 bit matrix over the warp: bit b of lane l becomes
+// bit l of lane b.
+__device__ __forceinline__ unsigned warp_transpose(unsigned x) {
+    const int lane = lane_id();
+    unsigned m = 0x0000FFFFu;
+#pragma unroll
+    for (int j = 16; j >= 1; j >>= 1) {
+        const unsigned t = __shfl_xor_sync(FULL, x, j);
+        x = (lane & j) ? ((t >> j) & m) | (x & ~m) : ((t << j) & ~m) | (x & m);
+        m ^= m << (j >> 1);
+    }
+    return x;
 }
 
-// Parents of the new bits of `row` (the (sel2nd, min) semiring of the
-// BFS-tree variant: the smallest neighbour in the frontier of each source).
-// A's row is ascending, so the neighbours are scanned 32 at a time in order
-// and each still-open bit goes to the first lane whose frontier row holds it
-// (an exclusive prefix OR over the lanes); the scan stops once every new bit
-// has its parent.  One warp, all lanes converged; rem is warp-uniform.
+// One word of the step of 32 neighbours (lane l: neighbour u, its bits `hit`
+// among the row's open ones): every bit's parent is the first lane that holds
+// it (A's rows ascend, so the smallest neighbour).  Returns the bits found.
+__device__ __forceinline__ unsigned bfs_first(unsigned hit, int u, int& parent, bool& found) {
+    const unsigned who = warp_transpose(hit);
+    found = who != 0u;
+    parent = __shfl_sync(FULL, u, found ? __ffs(who) - 1 : 0);
+    return __ballot_sync(FULL, found);
+}
+
+// Level writes of one row's new bits (warp-uniform words), lane l bit l.
 template <int DWP>
-__device__ __forceinline__ void pull_parents(const BfsParams& p, const unsigned* __restrict__ fb, long long row,
-                                             long long a0, long long a1, unsigned rem[DWP]) {
+__device__ __forceinline__ void bfs_write_levels(const BfsParams& p, long long row, const unsigned nw[DWP]) {
+    int* lv = p.levels + row * p.d + lane_id();
+#pragma unroll
+    for (int m = 0; m < DWP; ++m)
+        if ((nw[m] >> lane_id()) & 1u) lv[32 * m] = p.level;
+}
+
+template <int DWP, bool PARENTS>
+__global__ void __launch_bounds__(256, 4) k_bfs_pull(BfsParams p, const unsigned* __restrict__ fb,
+                                                     const unsigned* __restrict__ nonempty, int rows_per_warp,
+                                                     long long* items, long long item_cap, long long* done,
+                                                     long long* partial, int scan_tile) {
+    constexpr int U = DWP == 8 ? 2 : 4;  // neighbours in flight per lane
     const int lane = lane_id();
+    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long base = gw * rows_per_warp;
+    if (base >= p.n) return;
+    const BfsCols cols{p.Ai, nonempty, p.nF};
+    const long long v = base + lane;
+    const bool mine = lane < rows_per_warp && v < p.n;
+    long long a0 = 0, a1 = 0;
+    unsigned old[DWP], want[DWP], acc[DWP];
     unsigned open = 0u;
 #pragma unroll
-    for (int m = 0; m < DWP; ++m) open |= rem[m];
-    for (long long e0 = a0; e0 < a1 && open; e0 += 32) {
-        const long long e = e0 + lane;
-        int u = -1;
-        unsigned hit[DWP];
-#pragma unroll
-        for (int m = 0; m < DWP; ++m) hit[m] = 0u;
-        if (e < a1) {
-            u = __ldg(p.Ai + e);
-            if ((unsigned)u < (unsigned)p.nF) {
-#pragma unroll
-                for (int m = 0; m < DWP; ++m) hit[m] = __ldg(fb + (long long)u * DWP + m) & rem[m];
-            }
+    for (int m = 0; m < DWP; ++m) {
+        acc[m] = old[m] = want[m] = 0u;
+        if (mine && m < p.dw) {
+            const int bits = p.d - 32 * m;
+            old[m] = p.S[v * p.dw + m];
+            want[m] = ~old[m] & (bits >= 32 ? FULL : ((1u << bits) - 1u));
         }
-        open = 0u;
-#pragma unroll
-        for (int m = 0; m < DWP; ++m) {
-            unsigned incl = hit[m];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned t = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl |= t;
+        open |= want[m];
+    }
+    if (mine) {
+        a0 = clampll(__ldg(p.Ap + v), 0, p.nnzA);
+        a1 = clampll(__ldg(p.Ap + v + 1), a0, p.nnzA);
+    }
+    const long long len = open ? a1 - a0 : 0;  // nothing to find: the row is left out
+    const bool heavy = len > BFS_HEAVY;
+    // rows of many entries: queued for k_bfs_heavy in chunks
+    if (__any_sync(FULL, heavy)) {
+        const long long nc = heavy ? (len + BFS_CHUNK - 1) / BFS_CHUNK : 0;
+        const long long incl = warp_incl_scan(nc);
+        long long first = 0;
+        if (lane == 31) first = (long long)atomicAdd((unsigned long long*)&p.hdr->scratch[0], (unsigned long long)incl);
+        first = shfl64(first, 31) + incl - nc;
+        if (heavy) {
+            done[v] = 0;
+            for (int m = 0; m < p.dw; ++m) p.newbits[v * p.dw + m] = 0u;
+            for (long long c = 0; c < nc; ++c) {
+                if (first + c < item_cap) items[first + c] = (v << 24) | c;
+                else atomicOr(&p.hdr->err, ERR_CAPACITY);
             }
-            unsigned excl = __shfl_up_sync(FULL, incl, 1);
-            if (lane == 0) excl = 0u;
-            unsigned mine = hit[m] & ~excl;
-            while (mine) {
-                const int b = __ffs(mine) - 1;
-                mine &= mine - 1;
-                p.parents[row * p.d + 32 * m + b] = u;
-            }
-            rem[m] &= ~__shfl_sync(FULL, incl, 31);
-            open |= rem[m];
         }
     }
+    // short rows: a lane each, U neighbours in flight and the next U columns
+    // of A loaded ahead
+    const int slen = len <= BFS_SHORT ? (int)len : 0;
+    const int smax = (int)__reduce_max_sync(FULL, (unsigned)slen);
+    if (smax > 0) {
+        int u[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) u[t] = cols.load(a0 + t, t < slen);
+        for (int j = 0; j < smax; j += U) {
+            int un[U];
+            unsigned w[U][DWP];
+#pragma unroll
+            for (int t = 0; t < U; ++t) un[t] = cols.load(a0 + j + U + t, j + U + t < slen);
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+#pragma unroll
+                for (int m = 0; m < DWP; ++m) w[t][m] = 0u;
+                if (cols.hit(u[t])) bfs_row<DWP>(fb, u[t], w[t]);
+            }
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+#pragma unroll
+                for (int m = 0; m < DWP; ++m) {
+                    if constexpr (PARENTS) {
+                        unsigned h = w[t][m] & want[m] & ~acc[m];
+                        while (h) {
+                            const int b = __ffs(h) - 1;
+                            h &= h - 1;
+                            p.parents[v * p.d + 32 * m + b] = u[t];
+                        }
+                    }
+                    acc[m] |= w[t][m];
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < U; ++t) u[t] = un[t];
+        }
+    }
+    // longer rows: the warp takes one after another, 32 U neighbours at a
+    // time; the columns of the next step (the row's next, or the next row's
+    // first) are loaded before this step's frontier rows
+    unsigned rows = __ballot_sync(FULL, len > BFS_SHORT && !heavy);
+    if (rows) {
+        int r = __ffs(rows) - 1, j = 0;
+        long long e0 = shfl64(a0, r);
+        int nr = (int)shfl64(len, r);
+        int u[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) u[t] = cols.load(e0 + 32 * t + lane, 32 * t + lane < nr);
+        unsigned rem[DWP], got[DWP];  // the row's open bits; the bits this lane's neighbours (parents: the row) have
+#pragma unroll
+        for (int m = 0; m < DWP; ++m) {
+            rem[m] = __shfl_sync(FULL, want[m], r);
+            got[m] = 0u;
+        }
+        for (;;) {
+            const bool more = j + 32 * U < nr;  // of this row
+            const unsigned rest = rows & (rows - 1);
+            const int r2 = rest ? __ffs(rest) - 1 : r;  // the row after it
+            const long long e2 = shfl64(a0, r2);
+            const int n2 = rest ? (int)shfl64(len, r2) : 0;
+            const long long ne = more ? e0 + j + 32 * U : e2;
+            const int nn = more ? nr - j - 32 * U : n2;
+            int un[U];
+            unsigned w[U][DWP];
+#pragma unroll
+            for (int t = 0; t < U; ++t) un[t] = cols.load(ne + 32 * t + lane, 32 * t + lane < nn);
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+#pragma unroll
+                for (int m = 0; m < DWP; ++m) w[t][m] = 0u;
+                if (cols.hit(u[t])) bfs_row<DWP>(fb, u[t], w[t]);
+            }
+            unsigned live = 0u;
+            if constexpr (PARENTS) {
+#pragma unroll
+                for (int t = 0; t < U; ++t) {
+                    unsigned h = 0u;
+#pragma unroll
+                    for (int m = 0; m < DWP; ++m) h |= w[t][m] & rem[m];
+                    if (!__any_sync(FULL, h != 0u)) continue;
+#pragma unroll
+                    for (int m = 0; m < DWP; ++m) {
+                        int parent;
+                        bool found;
+                        const unsigned bits = bfs_first(w[t][m] & rem[m], u[t], parent, found);
+                        if (found) p.parents[(base + r) * p.d + 32 * m + lane] = parent;
+                        got[m] |= bits;
+                        rem[m] &= ~bits;
+                    }
+                }
+#pragma unroll
+                for (int m = 0; m < DWP; ++m) live |= rem[m];
+            } else {
+#pragma unroll
+                for (int m = 0; m < DWP; ++m) {
+#pragma unroll
+                    for (int t = 0; t < U; ++t) got[m] |= w[t][m];
+                    if (more) live |= rem[m] & ~__reduce_or_sync(FULL, got[m]);
+                }
+            }
+            if (more && live) {  // the row goes on
+                j += 32 * U;
+#pragma unroll
+                for (int t = 0; t < U; ++t) u[t] = un[t];
+                continue;
+            }
+#pragma unroll
+            for (int m = 0; m < DWP; ++m) {
+                const unsigned x = PARENTS ? got[m] : __reduce_or_sync(FULL, got[m]);
+                if (lane == r) acc[m] = x;
+                got[m] = 0u;
+            }
+            if (!rest) break;
+            rows = rest;
+            r = r2;
+            e0 = e2;
+            nr = n2;
+            j = 0;
+#pragma unroll
+            for (int t = 0; t < U; ++t)
+                u[t] = more ? cols.load(e0 + 32 * t + lane, 32 * t + lane < nr) : un[t];  // found early: not loaded yet
+#pragma unroll
+            for (int m = 0; m < DWP; ++m) rem[m] = __shfl_sync(FULL, want[m], r);
+        }
+    }
+    // settle: new = N and not S; S |= new; counts, new words, levels
+    int c = 0;
+    unsigned any = 0u;
+#pragma unroll
+    for (int m = 0; m < DWP; ++m) {
+        acc[m] &= want[m];
+        any |= acc[m];
+        c += __popc(acc[m]);
+    }
+    if (mine && !heavy) {
+        p.cnt_next[v] = c;
+        if (any) {
+#pragma unroll
+            for (int m = 0; m < DWP; ++m) {
+                if (m < p.dw) {
+                    p.newbits[v * p.dw + m] = acc[m];
+                    if (acc[m]) p.S[v * p.dw + m] = old[m] | acc[m];
+                }
+            }
+        }
+    }
+    for (unsigned rows = __ballot_sync(FULL, any != 0u); rows; rows &= rows - 1) {
+        const int r = __ffs(rows) - 1;
+        unsigned nw[DWP];
+#pragma unroll
+        for (int m = 0; m < DWP; ++m) nw[m] = __shfl_sync(FULL, acc[m], r);
+        bfs_write_levels<DWP>(p, base + r, nw);
+    }
+    // this warp's rows lie in one tile of the scan (rows_per_warp divides it)
+    c = warp_sum(c);
+    if (lane == 0 && c) atomicAdd((unsigned long long*)(partial + base / scan_tile), (unsigned long long)c);
 }
 
+// Rows above BFS_HEAVY: a block per chunk ORs its neighbours into the row's
+// new words (cleared when the row was queued); the block of the row's last
+// chunk settles the row.  A chunk that starts when the row has nothing left
+// to find is left out.
 template <int DWP>
-__global__ void __launch_bounds__(256, 6) k_msbfs_pull(BfsParams p, const unsigned* __restrict__ fb) {
-    __shared__ long long s_item, s_nheavy, s_nrows;
+__global__ void __launch_bounds__(256) k_bfs_heavy(BfsParams p, const unsigned* __restrict__ fb,
+                                                   const unsigned* __restrict__ nonempty,
+                                                   const long long* __restrict__ items, long long item_cap,
+                                                   long long* done, long long* partial, int scan_tile) {
     __shared__ unsigned s_or[DWP];
-    const int nw = blockDim.x >> 5, warp = warp_id(), lane = lane_id(), tid = threadIdx.x;
-    if (tid < 32) {  // one warp; its lanes store the same values
-        long long nh, nr;
-        sched_counts(p.hdr, p.cta_class, nh, nr);
-        s_nheavy = nh;
-        s_nrows = nr;
-    }
-    if (tid < DWP) s_or[tid] = 0u;
-    __syncthreads();
-    const long long nheavy = s_nheavy, nrows = s_nrows;
-    unsigned long long* err = &p.hdr->err;
-    // heavy rows: the block's threads split the row's entries
-    for (;;) {
-        if (tid == 0) s_item = (long long)atomicAdd(&p.hdr->heavy_ctr, 1ull);
-        __syncthreads();
-        const long long h = s_item;
-        __syncthreads();
-        if (h >= nheavy) break;
-        const int row = p.perm[h];
+    __shared__ int s_last;
+    const int lane = lane_id(), tid = threadIdx.x;
+    const long long nitems = min(p.hdr->scratch[0], item_cap);
+    const BfsCols cols{p.Ai, nonempty, p.nF};
+    for (long long it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const long long row = items[it] >> 24, c = items[it] & 0xFFFFFF;
         const long long a0 = clampll(__ldg(p.Ap + row), 0, p.nnzA);
         const long long a1 = clampll(__ldg(p.Ap + row + 1), a0, p.nnzA);
-        unsigned acc[DWP];
-#pragma unroll
-        for (int m = 0; m < DWP; ++m) acc[m] = 0u;
-        pull_or<DWP>(p, fb, a0, a1, tid, blockDim.x, acc, err);
+        const long long e0 = a0 + c * BFS_CHUNK;
+        const int n = (int)(a1 - e0 < BFS_CHUNK ? a1 - e0 : BFS_CHUNK);
+        if (tid < DWP) s_or[tid] = 0u;
+        unsigned want[DWP], got[DWP];
+        unsigned live = 0u;
 #pragma unroll
         for (int m = 0; m < DWP; ++m) {
-            const unsigned x = __reduce_or_sync(FULL, acc[m]);
+            want[m] = got[m] = 0u;
+            if (m < p.dw) {
+                const int bits = p.d - 32 * m;
+                want[m] = ~__ldcg(p.S + row * p.dw + m) & (bits >= 32 ? FULL : ((1u << bits) - 1u));
+                live |= want[m] & ~__ldcg(p.newbits + row * p.dw + m);
+            }
+        }
+        __syncthreads();
+        for (int j = tid; live && j < n; j += 4 * 256) {
+            int u[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) u[t] = cols.load(e0 + j + 256 * t, j + 256 * t < n);
+            unsigned w[DWP];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                if (cols.hit(u[t])) {
+                    bfs_row<DWP>(fb, u[t], w);
+#pragma unroll
+                    for (int m = 0; m < DWP; ++m) got[m] |= w[m];
+                }
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < DWP; ++m) {
+            const unsigned x = __reduce_or_sync(FULL, got[m] & want[m]);
             if (lane == 0 && x) atomicOr(&s_or[m], x);
         }
         __syncthreads();
-        if (warp == 0) {
-#pragma unroll
-            for (int m = 0; m < DWP; ++m) acc[m] = s_or[m];
-            unsigned nws[DWP];
-            const int c = pull_settle<DWP>(p, row, acc, nws);
-            if (lane == 0) p.cnt_next[row] = c;
-            if (p.parents) pull_parents<DWP>(p, fb, row, a0, a1, nws);
+        if (tid < p.dw && s_or[tid]) atomicOr(p.newbits + row * p.dw + tid, s_or[tid]);
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            const long long nc = (a1 - a0 + BFS_CHUNK - 1) / BFS_CHUNK;
+            s_last = (long long)atomicAdd((unsigned long long*)(done + row), 1ull) == nc - 1;
         }
         __syncthreads();
-        if (tid < DWP) s_or[tid] = 0u;
+        if (s_last && tid < 32) {
+            __threadfence();
+            unsigned nw[DWP];
+            int cnt = 0;
+#pragma unroll
+            for (int m = 0; m < DWP; ++m) {
+                nw[m] = m < p.dw ? __ldcg(p.newbits + row * p.dw + m) : 0u;
+                cnt += __popc(nw[m]);
+                if (lane == 0 && nw[m]) p.S[row * p.dw + m] |= nw[m];
+                // k_bfs_heavy_parents takes the minimum from here
+                if (p.parents && ((nw[m] >> lane) & 1u)) p.parents[row * p.d + 32 * m + lane] = 0x7FFFFFFF;
+            }
+            bfs_write_levels<DWP>(p, row, nw);
+            if (lane == 0) {
+                p.cnt_next[row] = cnt;
+                if (cnt) atomicAdd((unsigned long long*)(partial + row / scan_tile), (unsigned long long)cnt);
+            }
+        }
+        __syncthreads();
     }
-    // light rows: one warp per row
-    for (long long idx = nheavy + (long long)blockIdx.x * nw + warp; idx < nrows;
-         idx += (long long)gridDim.x * nw) {
-        const int row = p.perm[idx];
+}
+
+// Parents of the rows above BFS_HEAVY (the (sel2nd, min) semiring of the
+// BFS-tree variant): a block per chunk finds the first neighbour of the chunk
+// for every new bit whose parent so far lies behind the chunk's first column,
+// 256 neighbours at a time until every bit has one, and takes the minimum
+// into parents.  (A's rows ascend: once a chunk is reached, a parent at or
+// below its first column is final.)
+template <int DWP>
+__global__ void __launch_bounds__(256) k_bfs_heavy_parents(BfsParams p, const unsigned* __restrict__ fb,
+                                                           const unsigned* __restrict__ nonempty,
+                                                           const long long* __restrict__ items, long long item_cap) {
+    __shared__ unsigned s_rem[DWP];
+    __shared__ int s_first[32 * DWP];
+    const int lane = lane_id(), warp = warp_id(), tid = threadIdx.x;
+    const long long nitems = min(p.hdr->scratch[0], item_cap);
+    const BfsCols cols{p.Ai, nonempty, p.nF};
+    for (long long it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const long long row = items[it] >> 24, c = items[it] & 0xFFFFFF;
         const long long a0 = clampll(__ldg(p.Ap + row), 0, p.nnzA);
         const long long a1 = clampll(__ldg(p.Ap + row + 1), a0, p.nnzA);
-        unsigned acc[DWP];
+        const long long e0 = a0 + c * BFS_CHUNK;
+        const int n = (int)(a1 - e0 < BFS_CHUNK ? a1 - e0 : BFS_CHUNK);
+        const int u0 = __ldg(p.Ai + e0);
+        if (warp < DWP) {
+            bool need = false;
+            const int b = 32 * warp + lane;
+            if (warp < p.dw && ((__ldcg(p.newbits + row * p.dw + warp) >> lane) & 1u))
+                need = __ldcg(p.parents + row * p.d + b) > u0;
+            const unsigned r = __ballot_sync(FULL, need);
+            if (lane == 0) s_rem[warp] = r;
+            s_first[b] = 0x7FFFFFFF;
+        }
+        __syncthreads();
+        for (int j = 0; j < n; j += 256) {
+            unsigned rem[DWP];
+            unsigned live = 0u;
 #pragma unroll
-        for (int m = 0; m < DWP; ++m) acc[m] = 0u;
-        pull_or<DWP>(p, fb, a0, a1, lane, 32, acc, err);
+            for (int m = 0; m < DWP; ++m) {
+                rem[m] = s_rem[m];
+                live |= rem[m];
+            }
+            if (!live) break;  // the same for the whole block
+            const int u = cols.load(e0 + j + tid, j + tid < n);
+            unsigned w[DWP];
+            unsigned h = 0u;
 #pragma unroll
-        for (int m = 0; m < DWP; ++m) acc[m] = __reduce_or_sync(FULL, acc[m]);
-        unsigned nws[DWP];
-        const int c = pull_settle<DWP>(p, row, acc, nws);
-        if (lane == 0) p.cnt_next[row] = c;
-        if (p.parents) pull_parents<DWP>(p, fb, row, a0, a1, nws);
+            for (int m = 0; m < DWP; ++m) w[m] = 0u;
+            if (cols.hit(u)) bfs_row<DWP>(fb, u, w);
+#pragma unroll
+            for (int m = 0; m < DWP; ++m) h |= w[m] & rem[m];
+            if (__any_sync(FULL, h != 0u)) {
+#pragma unroll
+                for (int m = 0; m < DWP; ++m) {
+                    int parent;
+                    bool found;
+                    bfs_first(w[m] & rem[m], u, parent, found);
+                    if (found) atomicMin(&s_first[32 * m + lane], parent);
+                }
+            }
+            __syncthreads();
+            if (warp < DWP) {
+                const unsigned r = __ballot_sync(FULL, s_first[32 * warp + lane] != 0x7FFFFFFF);
+                if (lane == 0) s_rem[warp] &= ~r;
+            }
+            __syncthreads();
+        }
+        __syncthreads();
+        if (warp < p.dw && s_first[32 * warp + lane] != 0x7FFFFFFF)
+            atomicMin(p.parents + row * p.d + 32 * warp + lane, s_first[32 * warp + lane]);
+        __syncthreads();
+    }
+}
+
+// Columns of F_next from the new words, a warp per 32 rows: each row's bits
+// are written side by side, lane l bit l of every word.  Up to eight words a
+// row are loaded for all 32 rows at once (a load per row left each row to
+// wait for L2: 105 us for 57 million entries, so 90 us).  Nothing is written
+// when F_next does not fit (the caller repeats the read-out with more room);
+// hdr->total gets the number of entries.
+__global__ void __launch_bounds__(256) k_bfs_emit(long long n, int dw, const unsigned* __restrict__ newbits,
+                                                  const long long* __restrict__ rp, int* __restrict__ col,
+                                                  long long cap, WsHeader* hdr) {
+    const long long total = __ldg(rp + n);
+    if (blockIdx.x == 0 && threadIdx.x == 0) hdr->total = total;
+    if (total > cap) return;
+    const int lane = lane_id();
+    const unsigned lt = lanemask_lt();
+    const long long base = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32;
+    const long long v = base + lane;
+    long long pos = 0, end = 0;
+    if (v < n) {
+        pos = __ldg(rp + v);
+        end = __ldg(rp + v + 1);
+    }
+    const bool some = end > pos;
+    auto put = [&](unsigned word, int m, long long& at, long long last) {
+        if ((word >> lane) & 1u) {
+            const long long q = at + __popc(word & lt);
+            if (q < last && q < cap) col[q] = 32 * m + lane;
+            else atomicOr(&hdr->err, ERR_CAPACITY);
+        }
+        at += __popc(word);
+    };
+    if (dw <= 8) {
+        unsigned w[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) w[m] = some && m < dw ? __ldg(newbits + v * dw + m) : 0u;
+        for (unsigned rows = __ballot_sync(FULL, some); rows; rows &= rows - 1) {
+            const int r = __ffs(rows) - 1;
+            long long at = shfl64(pos, r);
+            const long long last = shfl64(end, r);
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+                if (m < dw) put(__shfl_sync(FULL, w[m], r), m, at, last);
+        }
+        return;
+    }
+    for (unsigned rows = __ballot_sync(FULL, some); rows; rows &= rows - 1) {
+        const int r = __ffs(rows) - 1;
+        long long at = shfl64(pos, r);
+        const long long last = shfl64(end, r);
+        for (int m0 = 0; m0 < dw; m0 += 32) {
+            const unsigned mine = m0 + lane < dw ? __ldg(newbits + (base + r) * dw + m0 + lane) : 0u;
+            for (int m = 0; m < 32 && m0 + m < dw; ++m) put(__shfl_sync(FULL, mine, m), m0 + m, at, last);
+        }
     }
 }
 
 template <int DWP>
-static cudaError_t launch_pull(const BfsParams& p, const DevCsr& F, unsigned* fb, const LaunchCfg& cfg,
-                               cudaStream_t st) {
+static cudaError_t launch_pull(BfsParams p, const DevCsr& F, unsigned* fb, const Sched& s, const LaunchCfg& cfg,
+                               long long* rp_next, long long item_cap, cudaStream_t st) {
     const long long n = F.nrows;
-    long long blocks = (n + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
+    unsigned* nonempty = reinterpret_cast<unsigned*>(s.blen);  // n / 32 words of the n the region holds
+    const unsigned nfront = (unsigned)((n + 255) / 256);
+    const unsigned ncheck = (unsigned)((p.nnzA + CHECK_PER_BLOCK - 1) / CHECK_PER_BLOCK);
     count_launch();
-    k_frontier_bits<DWP><<<(unsigned)blocks, 256, 0, st>>>(n, p.d, F.rowptr, F.nnz, F.col, fb, &p.hdr->err);
-    const int threads = 32 * cfg.warps_per_cta;
-    const int grid = persistent_grid((const void*)k_msbfs_pull<DWP>, threads, 0, cfg.sms);
+    k_bfs_frontier<DWP><<<nfront + ncheck, 256, 0, st>>>(n, p.d, F.rowptr, F.nnz, F.col, fb, nonempty, s.partial,
+                                                         (long long)scan_partial_count(n), rp_next, nfront, p.Ap,
+                                                         p.Ai, p.nnzA, &p.hdr->err);
+    // rows per warp: 32, or fewer (a power of two, at least 4) while that
+    // leaves less than 16 warps per SM
+    int rows = 32;
+    while (rows > 4 && n < (long long)cfg.sms * 16 * rows) rows /= 2;
+    const unsigned grid = (unsigned)((n + 8LL * rows - 1) / (8LL * rows));
+    const unsigned* ne = F.nnz < n / BFS_SPARSE ? nonempty : nullptr;
+    const int tile = scan_tile_rows();
     count_launch();
-    k_msbfs_pull<DWP><<<grid, threads, 0, st>>>(p, fb);
+    if (p.parents)
+        k_bfs_pull<DWP, true><<<grid, 256, 0, st>>>(p, fb, ne, rows, s.items, item_cap, s.flops, s.partial, tile);
+    else
+        k_bfs_pull<DWP, false><<<grid, 256, 0, st>>>(p, fb, ne, rows, s.items, item_cap, s.flops, s.partial, tile);
+    if (p.nnzA > BFS_HEAVY) {
+        const unsigned hg = (unsigned)(cfg.sms * 4);
+        count_launch();
+        k_bfs_heavy<DWP><<<hg, 256, 0, st>>>(p, fb, ne, s.items, item_cap, s.flops, s.partial, tile);
+        if (p.parents) {
+            count_launch();
+            k_bfs_heavy_parents<DWP><<<hg, 256, 0, st>>>(p, fb, ne, s.items, item_cap);
+        }
+    }
     return cudaGetLastError();
 }
 
@@ -460,7 +909,7 @@ cudaError_t launch_msbfs_init(long long n, int d, const int* src, unsigned* S, i
     if ((e = cudaMemsetAsync(S, 0, sizeof(unsigned) * (size_t)n * dw, st))) return e;
     if ((e = cudaMemsetAsync(levels, 0xFF, sizeof(int) * (size_t)n * d, st))) return e;
     count_launch();
-    k_msbfs_init_rows<<<(unsigned)((n + 1 + 255) / 256), 256, 0, st>>>(n, d, src, rp);
+    k_msbfs_init_rows<<<(unsigned)((n + 1 + INIT_ROWS - 1) / INIT_ROWS), 256, 0, st>>>(n, d, src, rp);
     count_launch();
     k_msbfs_init_cols<<<(d + 127) / 128, 128, 0, st>>>(n, d, dw, src, col, S, levels);
     return cudaGetLastError();
@@ -471,15 +920,13 @@ cudaError_t launch_msbfs_step(const DevCsr& A, const DevCsr& F, int d, unsigned*
                               cudaStream_t st, unsigned* fbits, int* parents) {
     cudaError_t e;
     const long long n = A.nrows;
-    if ((e = launch_row_flops(A, F, s, st))) return e;
-    if (n == 0) return cudaMemsetAsync(rp_next, 0, sizeof(long long), st);
     const int dw = (d + 31) / 32;
-    // prune rows that cannot gain bits, then histogram and order (rows left
-    // without products get their count 0 here)
-    count_launch();
-    k_mask_full_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, d, dw, S, s.flops);
-    if ((e = launch_reclassify(n, s, rp_next + 1, st))) return e;
-    if ((e = cudaMemsetAsync(rp_next, 0, sizeof(long long), st))) return e;
+    const int dwp = fbits ? msbfs_pull_words(d) : 0;
+    if (parents && !dwp) return cudaErrorInvalidValue;  // parents: pull form only
+    if (n == 0) {
+        if ((e = cudaMemsetAsync(s.hdr, 0, sizeof(WsHeader), st))) return e;
+        return cudaMemsetAsync(rp_next, 0, sizeof(long long), st);
+    }
     BfsParams p;
     p.Ap = A.rowptr;
     p.Ai = A.col;
@@ -498,18 +945,26 @@ cudaError_t launch_msbfs_step(const DevCsr& A, const DevCsr& F, int d, unsigned*
     p.perm = s.perm;
     p.hdr = s.hdr;
     p.cta_class = cfg.cta_class;
-    const int dwp = msbfs_pull_words(d);
-    if (parents && !(fbits && dwp)) return cudaErrorInvalidValue;  // parents: pull form only
-    if (fbits && dwp) {
+    p.n = n;
+    if (dwp) {
+        if ((e = cudaMemsetAsync(s.hdr, 0, sizeof(WsHeader), st))) return e;
+        const long long cap = flops_item_capacity(n, A.nnz);
         switch (dwp) {
-            case 1: e = launch_pull<1>(p, F, fbits, cfg, st); break;
-            case 2: e = launch_pull<2>(p, F, fbits, cfg, st); break;
-            case 4: e = launch_pull<4>(p, F, fbits, cfg, st); break;
-            default: e = launch_pull<8>(p, F, fbits, cfg, st); break;
+            case 1: e = launch_pull<1>(p, F, fbits, s, cfg, rp_next, cap, st); break;
+            case 2: e = launch_pull<2>(p, F, fbits, s, cfg, rp_next, cap, st); break;
+            case 4: e = launch_pull<4>(p, F, fbits, s, cfg, rp_next, cap, st); break;
+            default: e = launch_pull<8>(p, F, fbits, s, cfg, rp_next, cap, st); break;
         }
         if (e) return e;
-        return launch_scan_inplace(rp_next + 1, n, s.partial, st);
+        return launch_scan_summed(rp_next + 1, n, s.partial, st);
     }
+    if ((e = launch_row_flops(A, F, s, st))) return e;
+    // prune rows that cannot gain bits, then histogram and order (rows left
+    // without products get their count 0 here)
+    count_launch();
+    k_mask_full_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, d, dw, S, s.flops);
+    if ((e = launch_reclassify(n, s, rp_next + 1, st))) return e;
+    if ((e = cudaMemsetAsync(rp_next, 0, sizeof(long long), st))) return e;
     const int threads = 32 * cfg.warps_per_cta;
     const size_t smem = sizeof(unsigned) * (size_t)dw * cfg.warps_per_cta;
     if (smem > 48 * 1024 &&
@@ -527,8 +982,7 @@ cudaError_t launch_msbfs_emit(long long n, int d, const unsigned* newbits, const
                               long long cap, WsHeader* hdr, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     count_launch();
-    k_msbfs_emit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, (d + 31) / 32, newbits, rp, col, cap,
-                                                                &hdr->err);
+    k_bfs_emit<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, (d + 31) / 32, newbits, rp, col, cap, hdr);
     return cudaGetLastError();
 }
 

@@ -1023,6 +1023,14 @@ cudaError_t launch_scan_inplace(long long* x, long long n, long long* partial, c
     const long long nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     count_launch();
     k_scan_reduce<<<(unsigned)nb, SCAN_THREADS, 0, st>>>(x, n, partial);
+    return launch_scan_summed(x, n, partial, st);
+}
+
+int scan_tile_rows() { return SCAN_TILE; }
+
+cudaError_t launch_scan_summed(long long* x, long long n, long long* partial, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    const long long nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     count_launch();
     k_scan_partials<<<1, 1024, 0, st>>>(partial, nb);
     count_launch();
