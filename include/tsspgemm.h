@@ -364,6 +364,25 @@ TS_API ts_status msbfs_step_parents(const ts_csr_desc* A, const ts_csr_desc* F, 
 TS_API ts_status msbfs_init_parents(int64_t n, int64_t d, const int32_t* sources_dev, int32_t* parents,
                                     void* stream);
 
+/*
+ * A whole search (Alg. 3's loop, d <= 256) without the lists of frontiers
+ * that msbfs_step takes and gives: the levels start + 1 .. start + max_steps,
+ * or up to the first empty frontier.  start = 0 sets levels (int32[n*d]) and
+ * parents (int32[n*d], or NULL: levels only) up from the sources (device
+ * int32[d], as for msbfs_init); a search that has not ended when the call
+ * returns is resumed by calling again with the same arguments and ws and
+ * start = the steps made so far.  frontier_nnz[i] (host, max_steps entries) =
+ * nnz of the frontier that step i of this call found, *steps = the number of
+ * steps made (the last found nothing: the search has ended).  Synchronises
+ * the stream.  ws: msbfs_search_workspace_size bytes.  Errors as msbfs_step
+ * (a column of A outside [0, n) is TS_ERR_BAD_CSR); d above 256 is
+ * TS_ERR_UNSUPPORTED.
+ */
+TS_API ts_status msbfs_search_workspace_size(int64_t n, int64_t nnz_A, int64_t d, size_t* bytes);
+TS_API ts_status msbfs_search(const ts_csr_desc* A, int64_t d, const int32_t* sources_dev, int32_t* levels,
+                              int32_t* parents, int64_t start, int64_t max_steps, int64_t* frontier_nnz,
+                              int64_t* steps, void* ws, size_t ws_bytes, void* stream);
+
 /* Writes F_next->col from the state a TS_ERR_CAPACITY msbfs_step left in ws. */
 TS_API ts_status msbfs_emit(const ts_csr_desc* F_next, int64_t F_next_capacity, void* ws,
                      size_t ws_bytes, void* stream);

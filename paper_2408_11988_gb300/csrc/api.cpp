@@ -1091,6 +1091,43 @@ extern "C" ts_status msbfs_init_parents(int64_t n, int64_t d, const int32_t* sou
     return ok();
 }
 
+extern "C" ts_status msbfs_search_workspace_size(int64_t n, int64_t nnz_A, int64_t d, size_t* bytes) {
+    if (!bytes || n < 0 || nnz_A < 0 || d < 1)
+        return fail(TS_ERR_INVALID_ARG, "msbfs_search_workspace_size: bad argument");
+    if (d > 256) return fail(TS_ERR_UNSUPPORTED, "msbfs_search: d above 256");
+    *bytes = msbfs_search_bytes(n, nnz_A, (int)d);
+    return ok();
+}
+
+extern "C" ts_status msbfs_search(const ts_csr_desc* A, int64_t d, const int32_t* sources_dev, int32_t* levels,
+                                  int32_t* parents, int64_t start, int64_t max_steps, int64_t* frontier_nnz,
+                                  int64_t* steps, void* ws, size_t ws_bytes, void* stream) {
+    NvtxRange nvtx_range("msbfs_search");
+    const char* fn = "msbfs_search";
+    ts_status s;
+    if ((s = check_desc(A, "A", false)) != TS_OK) return s;
+    if (A->ncols != A->nrows) return fail(TS_ERR_INVALID_ARG, "%s: A must be n x n", fn);
+    if (d < 1 || !sources_dev || !levels || start < 0 || max_steps < 0 || !steps || (max_steps > 0 && !frontier_nnz))
+        return fail(TS_ERR_INVALID_ARG, "%s: NULL or negative argument", fn);
+    if (d > 256) return fail(TS_ERR_UNSUPPORTED, "%s: d above 256", fn);
+    if (start + max_steps > INT32_MAX) return fail(TS_ERR_OVERFLOW, "%s: levels are 32-bit", fn);
+    const size_t need = msbfs_search_bytes(A->nrows, A->nnz, (int)d);
+    if (!ws || ws_bytes < need)
+        return fail(TS_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes, %zu needed", fn, ws_bytes, need);
+    if (((uintptr_t)ws) & 255) return fail(TS_ERR_INVALID_ARG, "%s: workspace not 256-byte aligned", fn);
+    *steps = 0;
+    if (A->nrows == 0) return ok();
+    unsigned long long err = 0;
+    long long done = 0;
+    static_assert(sizeof(long long) == sizeof(int64_t), "counts");
+    TS_CUDA(launch_msbfs_search(dev(A), (int)d, sources_dev, levels, parents, start, max_steps,
+                                (long long*)frontier_nnz, &done, &err, sm_count(), ws, (cudaStream_t)stream),
+            fn);
+    if (err) return fail(TS_ERR_BAD_CSR, "%s: device checks failed (flags 0x%llx)", fn, err);
+    *steps = done;
+    return ok();
+}
+
 extern "C" ts_status msbfs_emit(const ts_csr_desc* F_next, int64_t F_next_capacity, void* ws,
                                 size_t ws_bytes, void* stream) {
     const char* fn = "msbfs_emit";

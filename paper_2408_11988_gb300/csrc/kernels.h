@@ -165,6 +165,15 @@ cudaError_t launch_msbfs_step(const DevCsr& A, const DevCsr& F, int d, unsigned*
                               const LaunchCfg& cfg, cudaStream_t st, unsigned* fbits = nullptr,
                               int* parents = nullptr);
 int msbfs_pull_words(int d);
+// A whole search with the frontier kept as a bitmap (d <= 256), levels start + 1
+// .. start + max_steps or up to an empty frontier: frontier[i] = entries found
+// by step i of this call, *steps = their number, *err = ERR_* bits.  start = 0
+// sets the search up; a later call with the same workspace resumes it.
+// Synchronises the stream.
+size_t msbfs_search_bytes(long long n, long long nnzA, int d);
+cudaError_t launch_msbfs_search(const DevCsr& A, int d, const int* src, int* levels, int* parents, long long start,
+                                long long max_steps, long long* frontier, long long* steps, unsigned long long* err,
+                                int sms, void* ws, cudaStream_t st);
 cudaError_t launch_msbfs_init_parents(long long n, int d, const int* src, int* parents, cudaStream_t st);
 cudaError_t launch_msbfs_emit(long long n, int d, const unsigned* newbits, const long long* rp,
                               int* col, long long cap, WsHeader* hdr, cudaStream_t st);

@@ -19,6 +19,26 @@ class BfsResult:
     parents: Optional[torch.Tensor] = None  # int32[n, d] BFS-tree parents (with parents=True)
 
 
+def _search(A: DeviceCSR, src: torch.Tensor, d: int, max_levels: int, stream, parents: bool) -> BfsResult:
+    """The search as one call of the library (resumed every 256 levels)."""
+    dev, n = A.rowptr.device, A.nrows
+    sz = ctypes.c_size_t()
+    N.call("msbfs_search_workspace_size", n, A.nnz, d, ctypes.byref(sz))
+    ws = torch.empty(max(int(sz.value), 256), dtype=torch.uint8, device=dev)
+    levels = torch.empty(n * d, dtype=torch.int32, device=dev)
+    par = torch.empty(n * d, dtype=torch.int32, device=dev) if parents else None
+    a = A.desc()
+    sizes, nnz, steps = [d], (ctypes.c_int64 * 256)(), ctypes.c_int64(0)
+    while True:
+        more = min(256, max_levels - (len(sizes) - 1))
+        N.call("msbfs_search", ctypes.byref(a), d, _ptr(src), _ptr(levels), _ptr(par), len(sizes) - 1, max(more, 0), nnz,
+               ctypes.byref(steps), _ptr(ws), ws.numel(), _stream(stream))
+        sizes.extend(nnz[:steps.value])
+        if steps.value < 256 or sizes[-1] == 0:
+            break
+    return BfsResult(levels.view(n, d), len(sizes) - 1, sizes, None if par is None else par.view(n, d))
+
+
 def msbfs(A: DeviceCSR, sources: torch.Tensor, max_levels: int = 1 << 20, stream=None,
           parents: bool = False) -> BfsResult:
     """Levels of every vertex from each of the d sources (columns); with
@@ -33,6 +53,8 @@ def msbfs(A: DeviceCSR, sources: torch.Tensor, max_levels: int = 1 << 20, stream
     s_host = src.cpu()
     if int(s_host.min()) < 0 or int(s_host.max()) >= n:
         raise ValueError("msbfs: source out of range")
+    if d <= 256:
+        return _search(A, src, d, max_levels, stream, parents)
     dw = (d + 31) // 32
     sz = ctypes.c_size_t()
     N.call("msbfs_workspace_size", n, A.nnz, d, ctypes.byref(sz))
