@@ -183,6 +183,18 @@ static bool dense_b_auto(bool vals, long long d, long long nB, long long nnzB) {
     return (double)nnzB * 1000.0 >= permille * (double)nB * (double)d;
 }
 
+// Products from which a row takes a whole block.  A lighter row is a chain of
+// its entries of A, shared by the slots of a warp, so the line is drawn at
+// about 320 entries, by B's mean row length, between 1024 and 4096 products
+// (powers of two).  Measured numeric + backward, us, at 1024 / 2048 / 4096:
+// B rows of 3 entries, 2^18 rows: 368 / 369 / 485; of 6, 2^16 rows: 156 / 156
+// / 199; of 26, 2^20 rows: 2817 / 2308 / 2268; of 51, 2^18 rows: 817 / 773 / 645.
+static long long auto_cta_min_flops(long long nB, long long nnzB) {
+    const double avg = nB > 0 ? (double)nnzB / (double)nB : 0.0;
+    if (avg <= 0.0 || avg >= 9.0) return 4096;
+    return avg >= 4.5 ? 2048 : 1024;
+}
+
 static ts_status resolve_tuning(long long d, const ts_tuning& force, ts_tuning& t,
                                 long long nB = 0, long long nnzB = 0, bool vals = false) {
     const long long dpad = round_up(d, 32);
@@ -191,7 +203,7 @@ static ts_status resolve_tuning(long long d, const ts_tuning& force, ts_tuning& 
                           : (dense_b_auto(vals, d, nB, nnzB) ? TS_ACC_DENSE_B
                                                               : (dpad <= 4096 ? TS_ACC_DENSE : TS_ACC_HASH));
     t.col_tile = force.col_tile ? force.col_tile : (int)std::min<long long>(dpad, 1024);
-    t.cta_min_flops = force.cta_min_flops ? force.cta_min_flops : 4096;
+    t.cta_min_flops = force.cta_min_flops ? force.cta_min_flops : auto_cta_min_flops(nB, nnzB);
     t.warps_per_cta = force.warps_per_cta ? force.warps_per_cta : 8;
     t.hash_slots = force.hash_slots ? force.hash_slots : 1024;
     t.group = force.group ? force.group : auto_group(nB, nnzB, 0);
@@ -498,7 +510,7 @@ static ts_status run_numeric(ts_plan* plan, const ts_csr_desc* A, const ts_csr_d
     const bool vals = plan->semiring == TS_SR_PLUS_TIMES_F32;
     const Sched sc = carve(ws, L);
     const DevCsr dA = dev(A), dB = dev(B);
-    const LaunchCfg cfg = cfg_of(plan->cur);
+    LaunchCfg cfg = cfg_of(plan->cur);
     if (plan->cur.accum == TS_ACC_DENSE_B && vals) {
         TS_CUDA(launch_numeric_denseb(dA, dB, plan->d, sc, cfg, (const long long*)C->rowptr, C->col, (float*)C->val,
                                       C->nnz, (char*)ws + L.denseb, st),
@@ -525,10 +537,12 @@ static ts_status run_numeric(ts_plan* plan, const ts_csr_desc* A, const ts_csr_d
         int4* bq = nullptr;
         if (use_bq) {
             bq = (int4*)((char*)ws + L.bq);
-            TS_CUDA(launch_pack_b_rows(dB, qE, plan->d, bq, &sc.hdr->err, st), fn);
+            TS_CUDA(launch_pack_b_rows(dB, qE, plan->d, bq, sc.hdr, st), fn);
+            cfg.counters_clear = true;
         } else if (vals && plan->cur.pack_b == 1 && B->nnz > 0) {
             bpk = (int2*)((char*)ws + L.bpk);
-            TS_CUDA(launch_pack_b(dB, bpk, st), fn);
+            TS_CUDA(launch_pack_b(dB, bpk, st, sc.hdr), fn);
+            cfg.counters_clear = true;
         }
         if (copies) {
             // light rows in row groups behind the copies kernel when they fit
@@ -598,11 +612,12 @@ static ts_status run_backward(ts_plan* plan, const ts_csr_desc* A, const ts_csr_
     if (plan->d > 8192) return fail(TS_ERR_UNSUPPORTED, "%s: backward supports d <= 8192", fn);
     const Sched sc = carve(ws, L);
     int2* bpk = nullptr;
+    LaunchCfg bcfg = cfg_of(plan->cur);
     if (plan->cur.pack_b == 1 && B->nnz > 0) {
         bpk = (int2*)((char*)ws + L.bpk);
-        TS_CUDA(launch_pack_b(dev(B), bpk, (cudaStream_t)stream), fn);
+        TS_CUDA(launch_pack_b(dev(B), bpk, (cudaStream_t)stream, sc.hdr), fn);
+        bcfg.counters_clear = true;
     }
-    LaunchCfg bcfg = cfg_of(plan->cur);
     bcfg.group = plan->cur.bwd_group;
     if (bcfg.group == 2 && (!bpk || (reinterpret_cast<uintptr_t>(dB) & 15))) bcfg.group = 16;  // no quads
     // option T: dA from the kernels (dB skipped), dB by the ordered pull

@@ -38,6 +38,7 @@ struct BwdParams {
     long long item_cap;
     int skip_light;  // 1: split and heavy rows only (light rows run in k_backward_light)
     int tiny;        // 1: light rows of classes <= BWD_TINY_CLASS run in k_backward_tiny
+    int tiny_rows;   // rows per chunk of that kernel
 };
 
 // Rows with at most 31 products (flops classes 1 .. 40) are the backward's
@@ -367,27 +368,30 @@ __device__ __forceinline__ void brg_seg(const BwdParams& p, int k, bool ok, long
 template <int RG>
 __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
     extern __shared__ __align__(16) float fsm[];
-    __shared__ long long s_nheavy, s_nrows;
+    __shared__ LightUnits s_lu;
     constexpr int R = 32 / RG;
     const int nw = blockDim.x >> 5, warp = warp_id(), lane = lane_id(), tid = threadIdx.x;
     const int g = lane / RG, gl = lane % RG;
     for (int i = tid; i < nw * R * p.dpad; i += blockDim.x) fsm[i] = 0.0f;
     if (tid < 32) {  // one warp; its lanes store the same values
-        long long nh, nr;
-        sched_counts(p.hdr, p.cta_class, nh, nr);
-        s_nheavy = nh;
-        s_nrows = nr;
+        LightUnits lu;
+        lu.init(p.hdr, p.cta_class, R, 0, gridDim.x * nw);
+        s_lu = lu;
     }
     __syncthreads();
-    float* gr = fsm + (size_t)(warp * R + g) * p.dpad;
+    const LightUnits& lu = s_lu;
     unsigned long long* err = &p.hdr->err;
     const int4* P4 = reinterpret_cast<const int4*>(p.Bpk);
     const long long* mark = p.s.flops;
-    const long long end = s_nrows, step = (long long)gridDim.x * nw * R;
-    for (long long idx = s_nheavy + ((long long)blockIdx.x * nw + warp) * R; idx < end; idx += step) {
-        const long long my = idx + g;
+    for (unsigned un = blockIdx.x * nw + warp; un < lu.units; un += gridDim.x * nw) {
+        // a unit is R rows, a slot each, or one row whose entries the slots
+        // share: the whole warp then scatters its row of dC into slot 0's
+        const bool team = lu.team(un);
+        float* gr = fsm + (size_t)(warp * R + (team ? 0 : g)) * p.dpad;
+        const int tl = team ? lane : gl, tn = team ? 32 : RG;  // lanes on one row of dC
+        const unsigned my = lu.row_at(un, g, R);
         long long a0 = 0, a1 = 0, c0 = 0, c1 = 0;
-        if (my < end) {
+        if (my < lu.end) {
             const int row = __ldg(p.perm + my);
             a0 = clampll(__ldg(p.Ap + row), 0, p.nnzA);
             a1 = clampll(__ldg(p.Ap + row + 1), a0, p.nnzA);
@@ -398,7 +402,8 @@ __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
                 c1 = clampll(__ldg(p.Cp + row + 1), c0, p.nnzC);
             }
         }
-        const int len = (int)(a1 - a0);
+        int len = (int)(a1 - a0);
+        if (team) team_share(g, R, a0, len);
         // first two chunks of A while dC is scattered
         int k0, k1;
         float x0, x1;
@@ -407,18 +412,18 @@ __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
         // the row of dC into the dense row, eight entries per lane in flight
         // (the row is read once, from DRAM: a chain of single loads would
         // wait out one memory latency per entry)
-        for (long long e = c0 + gl; e < c1; e += 8 * RG) {
+        for (long long e = c0 + tl; e < c1; e += 8 * tn) {
             int cc[8];
             float vv[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const long long eu = e + u * RG;
+                const long long eu = e + u * tn;
                 cc[u] = eu < c1 ? __ldg(p.Ci + eu) : 0;
                 vv[u] = eu < c1 ? __ldg(p.dC + eu) : 0.0f;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                if (e + u * RG < c1) {
+                if (e + u * tn < c1) {
                     if ((unsigned)cc[u] < (unsigned)p.d) gr[cc[u]] = vv[u];
                     else atomicOr(err, ERR_C_ROW);
                 }
@@ -480,7 +485,7 @@ __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
         // clear the whole dense row with 16-byte stores (dpad is a multiple
         // of 32, rows 16-byte aligned): cheaper than revisiting the row's
         // entries of C
-        for (int c = 4 * gl; c < p.dpad; c += 4 * RG) *reinterpret_cast<float4*>(gr + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 4 * tl; c < p.dpad; c += 4 * tn) *reinterpret_cast<float4*>(gr + c) = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncwarp();
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -497,6 +502,7 @@ __global__ void __launch_bounds__(256, HEAVY ? 6 : 5) k_backward(BwdParams p) {
     extern __shared__ __align__(16) float fsm[];
     __shared__ long long s_item, s_nheavy, s_nrows;
     const int nw = blockDim.x >> 5, warp = warp_id(), tid = threadIdx.x;
+    if (HEAVY && nothing_heavy(p.hdr, p.cta_class)) return;
     // layout: [nw][dpad] dense dC rows, then [nw][32] dA partials
     for (int i = tid; i < nw * (p.dpad + 32); i += blockDim.x) fsm[i] = 0.0f;
     if (tid < 32) {  // one warp; its lanes store the same values
@@ -536,9 +542,8 @@ __global__ void __launch_bounds__(256, HEAVY ? 6 : 5) k_backward(BwdParams p) {
         // k_backward_tiny takes them, are the last ones)
         long long nlight_end = nrows;
         if (p.tiny) {
-            long long t = 0;
-            for (int c = 1 + lane_id(); c <= BWD_TINY_CLASS && c < p.cta_class; c += 32) t += p.hdr->hist[c];
-            nlight_end -= warp_sum(t);
+            const int last = BWD_TINY_CLASS < p.cta_class ? BWD_TINY_CLASS : p.cta_class - 1;
+            nlight_end -= nrows - rows_from_class(p.hdr, last + 1);
         }
         float* g = fsm + (size_t)warp * p.dpad;
         BwdRowBody<G, BA> body{p, ba, g, sdA, &p.hdr->err, -1, 0, 0, 0, 0};
@@ -554,21 +559,23 @@ __global__ void __launch_bounds__(256, HEAVY ? 6 : 5) k_backward(BwdParams p) {
 // Eq. 1).  A product (k, col) finds dC(i, col) by a binary search of the
 // sorted row of C over the lanes; it adds A(i,k) * dC(i, col) to dB with a
 // float atomic and B(k, col) * dC(i, col) to dA(i,k), the products of one
-// entry (neighbouring lanes) summed into their first lane.  32-row chunks
-// are dealt to the warps in turn.  Used where the light rows would each
+// entry (neighbouring lanes) summed into their first lane.  Chunks of 32
+// rows (fewer when there are few, tiny_chunk_rows) are dealt to the warps in
+// turn.  Used where the light rows would each
 // take a warp pass over a dense row of d floats (d above the row-group
 // range).
 template <bool PACKED>
 __global__ void __launch_bounds__(256) k_backward_tiny(BwdParams p) {
     const int lane = lane_id();
     unsigned long long* err = &p.hdr->err;
-    const long long nchunks = ((long long)p.nB + 31) / 32;
+    const int cr = p.tiny_rows;
+    const long long nchunks = ((long long)p.nB + cr - 1) / cr;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     const SegWhole seg{p.Bp, p.nnzB, p.d};
     for (long long c = gw; c < nchunks; c += nwarps) {
-        const long long r = c * 32 + lane;
-        const long long f = r < p.nB ? __ldg(p.s.flops + r) : 0;
+        const long long r = c * cr + lane;
+        const long long f = lane < cr && r < p.nB ? __ldg(p.s.flops + r) : 0;
         const int cls = flops_class(f);
         const bool tiny = f >= 1 && cls <= BWD_TINY_CLASS && cls < p.cta_class;
         long long a0 = 0, a1 = 0, o0 = 0, o1 = 0;
@@ -667,7 +674,8 @@ cudaError_t launch_backward(const DevCsr& A, const DevCsr& B, long long d, const
     if (dA && A.nnz && (e = cudaMemsetAsync(dA, 0, sizeof(float) * A.nnz, st))) return e;
     if (dB && B.nnz && (e = cudaMemsetAsync(dB, 0, sizeof(float) * B.nnz, st))) return e;
     if (A.nrows == 0 || (!dA && !dB)) return cudaSuccess;
-    if ((e = cudaMemsetAsync(&s.hdr->heavy_ctr, 0, 2 * sizeof(unsigned long long), st))) return e;
+    if (!cfg.counters_clear && (e = cudaMemsetAsync(&s.hdr->heavy_ctr, 0, 2 * sizeof(unsigned long long), st)))
+        return e;
     BwdParams p;
     p.Ap = A.rowptr;
     p.Ai = A.col;
@@ -713,10 +721,11 @@ cudaError_t launch_backward(const DevCsr& A, const DevCsr& B, long long d, const
     if (!rg && cfg.row_lanes != 32 && d > 256) {
         p.tiny = 1;
         const void* kt = pk ? (const void*)k_backward_tiny<true> : (const void*)k_backward_tiny<false>;
+        const int tgrid = persistent_grid(kt, 256, 0, cfg.sms);
+        p.tiny_rows = tiny_chunk_rows(A.nrows, 8LL * tgrid);
         void* targs[] = {&p};
         count_launch();
-        if ((e = cudaLaunchKernel(kt, dim3(persistent_grid(kt, 256, 0, cfg.sms)), dim3(256), targs, 0, st)))
-            return e;
+        if ((e = cudaLaunchKernel(kt, dim3(tgrid), dim3(256), targs, 0, st))) return e;
     }
     const void* k;
     switch (cfg.group) {

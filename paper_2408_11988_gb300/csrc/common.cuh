@@ -346,18 +346,81 @@ __device__ __forceinline__ void pipelined_rows(const int* __restrict__ perm, lon
     }
 }
 
+// Rows of class c and above, c >= 1 (of the classes' running sums that the row
+// order leaves in the header: every block of every pass reads these, and
+// summing the 385 counters there took each of them 2 - 3 us).
+__device__ __forceinline__ long long rows_from_class(const WsHeader* hdr, int c) {
+    return c < NUM_CLASSES ? __ldg(hdr->above + (c > 1 ? c : 1) - 1) : 0;
+}
+
 // Rows with products: all classes >= 1; heavy: classes >= cta_class.
-// Called by all 32 lanes of one warp (every lane gets the counts).
 __device__ __forceinline__ void sched_counts(const WsHeader* hdr, int cta_class, long long& nheavy,
                                              long long& nrows) {
-    long long nh = 0, nr = 0;
-    for (int c = 1 + lane_id(); c < NUM_CLASSES; c += 32) {
-        const long long h = hdr->hist[c];
-        nr += h;
-        if (c >= cta_class) nh += h;
+    nheavy = rows_from_class(hdr, cta_class);
+    nrows = rows_from_class(hdr, 1);
+}
+
+// No split item and no row for a whole block in this product.
+__device__ __forceinline__ bool nothing_heavy(const WsHeader* hdr, int cta_class) {
+    return rows_from_class(hdr, cta_class) == 0 && __ldg(&hdr->scratch[2]) == 0;
+}
+
+// Units of a light-row kernel whose warps hold R slots: the first nteam light
+// rows of the class order (the heaviest) are one unit each, their entries of A
+// shared out over the warp's slots; the rows behind them go R to a unit, one
+// per slot.  A row in one slot is a serial chain of segments of B: at the
+// block threshold it alone took 140 - 240 us of each pass, which was the whole
+// pass of a product of less than some 100 million products.  Rows of at least
+// 512 products are shared (a slot walks that in some 20 us), or of 2048 where
+// every warp has many units and such a chain is hidden (scale 22: numeric
+// 3.23 ms, 3.39 with rows from 512 on shared); where warps would be left over,
+// rows of at least 128, as many as leave no more units than warps (below that
+// the extra read-outs cost what the shorter chains save).  Symbolic / numeric /
+// backward, us, before and after: 2^14 rows, d = 64, 1.5 million products 333 /
+// 152 / 258 -> 103 / 57 / 56; 2^18 rows, d = 128, 25 million 334 / 235 / 293 ->
+// 212 / 189 / 209; 2^20 rows, d = 128, 412 million 706 / 1032 / 1329 -> 694 /
+// 1036 / 1261.
+constexpr int TEAM_CLASS = 1 + (9 << CLASS_SUB_BITS), TEAM_CLASS_MANY = 1 + (11 << CLASS_SUB_BITS);
+constexpr int TEAM_CLASS_FEW = 1 + (7 << CLASS_SUB_BITS);
+constexpr int TEAM_UNITS_MANY = 32;  // per warp, all rows R to a unit
+
+struct LightUnits {
+    unsigned nheavy, nteam, end, units;  // rows are numbered with 31 bits
+    // nwarps: of the grid.  Rows of classes <= last_class_out are left out (the
+    // tail of the class order).
+    __device__ __forceinline__ void init(const WsHeader* hdr, int cta_class, int R, int last_class_out,
+                                         unsigned nwarps) {
+        const long long nh = rows_from_class(hdr, cta_class);
+        auto light_from = [&](int c) {
+            const long long x = rows_from_class(hdr, c) - nh;
+            return (unsigned)(x > 0 ? x : 0);
+        };
+        const unsigned light = light_from(last_class_out + 1);
+        const bool many = light >= (unsigned long long)TEAM_UNITS_MANY * R * nwarps;
+        unsigned team = light_from(many ? TEAM_CLASS_MANY : TEAM_CLASS);
+        if (light < R * nwarps) {
+            const unsigned spare = (R * nwarps - light) / (R - 1);  // team + (light - team) / R <= nwarps
+            const unsigned few = light_from(TEAM_CLASS_FEW);
+            if (team < spare) team = spare < few ? spare : few;
+        }
+        nheavy = (unsigned)nh;
+        nteam = team < light ? team : light;
+        end = nheavy + light;
+        units = nteam + (light - nteam + R - 1) / R;
     }
-    nheavy = warp_sum(nh);
-    nrows = warp_sum(nr);
+    __device__ __forceinline__ bool team(unsigned u) const { return u < nteam; }
+    // the place in the class order of unit u's row for slot g (end or more: none)
+    __device__ __forceinline__ unsigned row_at(unsigned u, int g, int R) const {
+        if (u < nteam) return nheavy + u;
+        return u < units ? nheavy + nteam + (u - nteam) * R + g : end;
+    }
+};
+
+// Slot g's share [a0, a0 + len) of R equal contiguous ones.
+__device__ __forceinline__ void team_share(int g, int R, long long& a0, int& len) {
+    const int q = len / R, r = len - q * R;
+    a0 += (long long)q * g + (g < r ? g : r);
+    len = q + (g < r ? 1 : 0);
 }
 
 // Fetch the next split item for this block; false when none is left.  On

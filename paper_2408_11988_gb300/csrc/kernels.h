@@ -48,6 +48,7 @@ struct LaunchCfg {
     int cta_class = 14;      // rows of flops class >= this run CTA-per-row
     int sms = 152;
     int group = 1;           // lanes per A entry (1 = flattened products)
+    bool counters_clear = false;  // the header's work counters were cleared by the packing kernel just before
     int row_lanes = 32;      // numeric light rows: 32 = a warp per row, 4/8/16 = row groups,
                              // 1 = a warp per row on one shared accumulator (wide kernel)
 };
@@ -62,7 +63,14 @@ cudaError_t launch_row_schedule(const DevCsr& A, const DevCsr& B, const Sched& s
 // The two halves: flops per row (clears the header), and histogram + perm
 // from the flops array (Cp_next[i] = 0 for rows without products if given).
 cudaError_t launch_row_flops(const DevCsr& A, const DevCsr& B, const Sched& s, cudaStream_t st);
-cudaError_t launch_reclassify(long long n, const Sched& s, long long* Cp_next, cudaStream_t st);
+// A != nullptr: its rows of many entries are cut into split items.  The
+// header was cleared by launch_row_flops.
+cudaError_t launch_reclassify(long long n, const Sched& s, long long* Cp_next, cudaStream_t st,
+                              const DevCsr* A = nullptr);
+// Rows per chunk of the tiny-row kernels: 32, or fewer (a power of two, at
+// least 2) while that leaves warps without a chunk -- a chunk's rows are taken
+// one after another (3001 rows of 25 products: 61 us with 32 rows a warp).
+int tiny_chunk_rows(long long n, long long nwarps);
 
 // Symbolic pass: Cp[i+1] = nnz(C_i) for the scheduled rows, then Cp = running sum.
 cudaError_t launch_symbolic(const DevCsr& A, const DevCsr& B, long long d, const Sched& s,
@@ -103,12 +111,13 @@ cudaError_t launch_numeric_copies(const DevCsr& A, const DevCsr& B, long long d,
 // Dynamic shared memory of that pass (0 for an unsupported G).
 size_t numeric_copies_smem(int W, int G, int warps);
 // Packed (column, value bits) copy of B's entries.
-cudaError_t launch_pack_b(const DevCsr& B, int2* P, cudaStream_t st);
+// hdr (may be nullptr): its work counters are cleared on the way.
+cudaError_t launch_pack_b(const DevCsr& B, int2* P, cudaStream_t st, WsHeader* hdr = nullptr);
 // Row-aligned packed copy of B: row k starts at entry E*ceil((Bp[k] + (E-1)k)/E),
 // its last group padded with column -1; columns outside [0, d) are stored as
-// -1 and set ERR_B_COL in *err.  E = 2 or 4.
-cudaError_t launch_pack_b_rows(const DevCsr& B, int E, long long d, int4* Q, unsigned long long* err,
-                               cudaStream_t st);
+// -1 and set ERR_B_COL in hdr->err; hdr's work counters are cleared on the way.
+// E = 2 or 4.
+cudaError_t launch_pack_b_rows(const DevCsr& B, int E, long long d, int4* Q, WsHeader* hdr, cudaStream_t st);
 size_t padded_b_bytes(long long nB, long long nnzB, long long d, int E);
 // Whether the copy's groups can be numbered with 32 bits.
 bool padded_b_fits(long long nB, long long nnzB, long long d, int E);

@@ -49,6 +49,7 @@ struct WsHeader {
     long long total;                  // multi-source BFS: entries of the next frontier (read with err)
     long long hist[NUM_CLASSES];      // rows per flops class
     long long cursor[NUM_CLASSES];    // scatter cursors per class
+    long long above[NUM_CLASSES];     // rows in the classes above each (written with the row order)
     long long scratch[8];             // [0] flops items, [1] split rows, [2] split items
 };
 

@@ -483,25 +483,32 @@ __device__ __forceinline__ void rg_row_bounds(const NumParams& p, int row, const
     active = true;
 }
 
-// rg_light_rows on the row-aligned copy (T = 1), pipelined across row
-// groups: while group idx is gathered, the schedule entry of group idx + 2
-// steps and the row bounds of group idx + step are in flight; the next
-// group's first two chunks of A and output range load before this group's
-// read-out.  A group then starts with only B's row pointers and first groups
-// to wait for.
+// rg_light_rows on the row-aligned copy (T = 1), by units (a row shared by the
+// warp's slots, or a row per slot: LightUnits) and pipelined across them:
+// while unit u is gathered, the schedule entries of unit u + 2 steps and the
+// row bounds of unit u + step are in flight; the next unit's first two chunks
+// of A and output range load before this unit's read-out.  A unit then starts
+// with only B's row pointers and first groups to wait for.
 template <int RG>
-__device__ __forceinline__ void rgp_light_rows(const NumParams& p, float* racc, long long idx0, long long end,
-                                               long long step, const long long* mark) {
-    constexpr int E = RG == 4 ? 4 : 2;
+__device__ __forceinline__ void rgp_light_rows(const NumParams& p, float* racc, const LightUnits& lu, unsigned u0,
+                                               unsigned step, const long long* mark) {
+    constexpr int E = RG == 4 ? 4 : 2, R = 32 / RG;
     const int lane = lane_id(), g = lane / RG, gl = lane % RG;
     float* acc = racc + g * (p.W + 8);  // W columns, a spare and padding
     unsigned long long* err = &p.hdr->err;
-    auto row_at = [&](long long idx) { return idx + g < end ? __ldg(p.perm + idx + g) : -1; };
-    int row = row_at(idx0), nrow = row_at(idx0 + step);
+    auto row_of = [&](unsigned u) {
+        const unsigned at = lu.row_at(u, g, R);
+        return at < lu.end ? __ldg(p.perm + at) : -1;
+    };
+    auto bounds = [&](unsigned u, int row, long long& a0, int& len, bool& active) {
+        rg_row_bounds(p, row, mark, a0, len, active);
+        if (lu.team(u)) team_share(g, R, a0, len);
+    };
+    int row = row_of(u0), nrow = row_of(u0 + step);
     long long a0;
     int len;
     bool active;
-    rg_row_bounds(p, row, mark, a0, len, active);
+    bounds(u0, row, a0, len, active);
     long long out = 0, out_end = 0;
     if (active) {
         out = clampll(__ldg(p.Cp + row), 0, p.nnzC);
@@ -511,12 +518,12 @@ __device__ __forceinline__ void rgp_light_rows(const NumParams& p, float* racc, 
     float x0, x1;
     rg_load_a(p, a0 + gl, gl < len, k0, x0);
     rg_load_a(p, a0 + RG + gl, RG + gl < len, k1, x1);
-    for (long long idx = idx0; idx < end; idx += step) {
+    for (unsigned u = u0; u < lu.units; u += step) {
         long long na0;
         int nlen;
         bool nactive;
-        rg_row_bounds(p, nrow, mark, na0, nlen, nactive);
-        const int nnrow = row_at(idx + 2 * step);
+        bounds(u + step, nrow, na0, nlen, nactive);
+        const int nnrow = row_of(u + 2 * step);
         const int lmax = (int)__reduce_max_sync(FULL, (unsigned)len);
         rgp_tile<RG, E>(p, p.Bq, AddPlain{acc}, a0, len, lmax, err, k0, x0, k1, x1);
         rg_load_a(p, na0 + gl, gl < nlen, k0, x0);
@@ -526,7 +533,8 @@ __device__ __forceinline__ void rgp_light_rows(const NumParams& p, float* racc, 
             nout = clampll(__ldg(p.Cp + nrow), 0, p.nnzC);
             nout_end = clampll(__ldg(p.Cp + nrow + 1), nout, p.nnzC);
         }
-        rg_emit<RG>(racc, p.W, 0, out, out_end, p.Ci, p.Cx, err);
+        if (lu.team(u)) rg_emit_team<RG>(racc, p.W, out, out_end, p.Ci, p.Cx);
+        else rg_emit<RG>(racc, p.W, 0, out, out_end, p.Ci, p.Cx, err);
         __syncwarp();
         if (active && gl == 0 && out != out_end) atomicOr(err, ERR_C_ROW);
         a0 = na0;
@@ -548,28 +556,22 @@ __device__ __forceinline__ void rgp_light_rows(const NumParams& p, float* racc, 
 template <int RG, bool PADDED>
 __global__ void __launch_bounds__(256, 5) k_numeric_light(NumParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long s_nheavy, s_nrows;
+    __shared__ LightUnits s_lu;
     constexpr int R = 32 / RG;
     const int nw = blockDim.x >> 5, warp = warp_id(), tid = threadIdx.x;
     float* racc = reinterpret_cast<float*>(smem);
     for (int i = tid; i < nw * R * (p.W + 8); i += blockDim.x) reinterpret_cast<unsigned*>(racc)[i] = RG_EMPTY;
     if (tid < 32) {  // one warp; its lanes store the same values
-        long long nh, nr;
-        sched_counts(p.hdr, p.cta_class, nh, nr);
-        if (p.tiny_max) {  // the tiny rows, last in the class order, run in k_numeric_tiny
-            long long t = 0;
-            for (int c = 1 + lane_id(); c <= TINY_CLASS && c < p.cta_class; c += 32) t += p.hdr->hist[c];
-            nr -= warp_sum(t);
-        }
-        s_nheavy = nh;
-        s_nrows = nr;
+        LightUnits lu;
+        lu.init(p.hdr, p.cta_class, R, p.tiny_max ? TINY_CLASS : 0, (long long)gridDim.x * nw);  // tiny rows run in k_numeric_tiny
+        s_lu = lu;
     }
     __syncthreads();
     const long long* mark = p.s.stg_vals != nullptr ? p.s.flops : nullptr;
     float* wacc = racc + (size_t)warp * R * (p.W + 8);
-    const long long idx0 = s_nheavy + ((long long)blockIdx.x * nw + warp) * R, step = (long long)gridDim.x * nw * R;
-    if constexpr (PADDED) rgp_light_rows<RG>(p, wacc, idx0, s_nrows, step, mark);
-    else rg_light_rows<RG>(p, wacc, idx0, s_nrows, step, mark);
+    const long long gw = (long long)blockIdx.x * nw + warp, gws = (long long)gridDim.x * nw;
+    if constexpr (PADDED) rgp_light_rows<RG>(p, wacc, s_lu, (unsigned)gw, (unsigned)gws, mark);
+    else rg_light_rows<RG>(p, wacc, s_lu.nheavy + gw * R, s_lu.end, gws * R, mark);
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -620,6 +622,7 @@ __global__ void __launch_bounds__(256, 5) k_numeric_rgcta(NumParams p) {
     __shared__ int s_last;
     constexpr int R = 32 / RG;
     const int tid = threadIdx.x, S = (blockDim.x >> 5) * R, ld = p.W + 8;
+    if (nothing_heavy(p.hdr, p.cta_class)) return;
     float* racc = reinterpret_cast<float*>(smem);
     float* sum = racc + (size_t)S * ld;
     for (int i = tid; i < S * ld + p.W; i += blockDim.x) reinterpret_cast<unsigned*>(racc)[i] = RG_EMPTY;
@@ -961,8 +964,17 @@ __global__ void __launch_bounds__(256, 5) k_numeric(NumParams p) {
                        SegTile{p.tp, p.T + 1, 0, p.W}, &p.hdr->err, body, mark);
 }
 
+// The pass that follows takes its rows by these counters.
+__device__ __forceinline__ void clear_counters(WsHeader* hdr) {
+    if (hdr && blockIdx.x == 0 && threadIdx.x == 0) {
+        hdr->heavy_ctr = 0;
+        hdr->item_ctr = 0;
+    }
+}
+
 __global__ void k_pack_b(long long nnz, const int* __restrict__ Bi, const float* __restrict__ Bx,
-                         int2* __restrict__ P) {
+                         int2* __restrict__ P, WsHeader* hdr) {
+    clear_counters(hdr);
     for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < nnz;
          j += (long long)gridDim.x * blockDim.x)
         P[j] = make_int2(__ldg(Bi + j), __float_as_int(__ldg(Bx + j)));
@@ -974,8 +986,9 @@ __global__ void k_pack_b(long long nnz, const int* __restrict__ Bi, const float*
 template <int E>
 __global__ void __launch_bounds__(256) k_pack_b_rows(int nB, const long long* __restrict__ Bp, long long nnzB,
                                                      const int* __restrict__ Bi, const float* __restrict__ Bx, int d,
-                                                     int2* __restrict__ Q, unsigned long long* err) {
+                                                     int2* __restrict__ Q, WsHeader* hdr) {
     const int gl = threadIdx.x & 7;
+    clear_counters(hdr);
     bool bad = false;
     for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; k < nB; k += (gridDim.x * blockDim.x) >> 3) {
         long long s;
@@ -995,7 +1008,7 @@ __global__ void __launch_bounds__(256) k_pack_b_rows(int nB, const long long* __
             q[j] = v;
         }
     }
-    if (bad) atomicOr(err, ERR_B_COL);
+    if (bad) atomicOr(&hdr->err, ERR_B_COL);
 }
 
 // Entries of the row-aligned copy for B (n_B rows, nnzB entries, d columns)
@@ -1013,7 +1026,7 @@ bool padded_b_fits(long long nB, long long nnzB, long long d, int E) {
     return padded_b_entries(nB, nnzB, d, E) / E < (1LL << 31) && nB < (1LL << 31);
 }
 
-cudaError_t launch_pack_b_rows(const DevCsr& B, int E, long long d, int4* Q, unsigned long long* err,
+cudaError_t launch_pack_b_rows(const DevCsr& B, int E, long long d, int4* Q, WsHeader* hdr,
                                cudaStream_t st) {
     if (B.nrows == 0) return cudaSuccess;
     if ((E != 2 && E != 4) || !padded_b_fits(B.nrows, B.nnz, d, E)) return cudaErrorInvalidValue;
@@ -1022,18 +1035,18 @@ cudaError_t launch_pack_b_rows(const DevCsr& B, int E, long long d, int4* Q, uns
     int2* P = reinterpret_cast<int2*>(Q);
     count_launch();
     if (E == 2)
-        k_pack_b_rows<2><<<(unsigned)blocks, 256, 0, st>>>((int)B.nrows, B.rowptr, B.nnz, B.col, B.val, (int)d, P, err);
+        k_pack_b_rows<2><<<(unsigned)blocks, 256, 0, st>>>((int)B.nrows, B.rowptr, B.nnz, B.col, B.val, (int)d, P, hdr);
     else
-        k_pack_b_rows<4><<<(unsigned)blocks, 256, 0, st>>>((int)B.nrows, B.rowptr, B.nnz, B.col, B.val, (int)d, P, err);
+        k_pack_b_rows<4><<<(unsigned)blocks, 256, 0, st>>>((int)B.nrows, B.rowptr, B.nnz, B.col, B.val, (int)d, P, hdr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_b(const DevCsr& B, int2* P, cudaStream_t st) {
+cudaError_t launch_pack_b(const DevCsr& B, int2* P, cudaStream_t st, WsHeader* hdr) {
     if (B.nnz == 0) return cudaSuccess;
     long long blocks = (B.nnz + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
     count_launch();
-    k_pack_b<<<(unsigned)blocks, 256, 0, st>>>(B.nnz, B.col, B.val, P);
+    k_pack_b<<<(unsigned)blocks, 256, 0, st>>>(B.nnz, B.col, B.val, P, hdr);
     return cudaGetLastError();
 }
 
@@ -1162,7 +1175,8 @@ cudaError_t launch_numeric_dense(const DevCsr& A, const DevCsr& B, long long d, 
     if (A.nrows == 0) return cudaSuccess;
     if (W <= 0 || W % 32 || W > MAX_DENSE_W || (long long)W * T < d) return cudaErrorInvalidValue;
     if (cfg.warps_per_cta < 1 || cfg.warps_per_cta > 8) return cudaErrorInvalidValue;
-    if ((e = cudaMemsetAsync(&s.hdr->heavy_ctr, 0, 2 * sizeof(unsigned long long), st))) return e;
+    if (!cfg.counters_clear && (e = cudaMemsetAsync(&s.hdr->heavy_ctr, 0, 2 * sizeof(unsigned long long), st)))
+        return e;
     NumParams p = numeric_params(A, B, d, W, T, tp, Bpk, s, cfg, Cp, Ci, Cx, nnzC);
     const int w = cfg.warps_per_cta;
     if (Bq && (T != 1 || !values || cfg.row_lanes == 32)) return cudaErrorInvalidValue;

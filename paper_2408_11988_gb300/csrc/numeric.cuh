@@ -36,6 +36,7 @@ struct NumParams {
     Sched s;
     long long item_cap;
     int skip_light;  // 1: split and heavy rows only (light rows run in a kernel of their own)
+    int tiny_rows;   // k_numeric_tiny: rows per chunk
     int tiny_max;    // wide kernel: light rows with at most this many products run in k_numeric_tiny
 };
 
@@ -74,6 +75,7 @@ inline NumParams numeric_params(const DevCsr& A, const DevCsr& B, long long d, i
     p.s = s;
     p.item_cap = split_item_capacity(A.nnz);
     p.skip_light = 0;
+    p.tiny_rows = 32;
     p.tiny_max = 0;
     return p;
 }

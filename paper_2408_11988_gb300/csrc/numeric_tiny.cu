@@ -186,8 +186,8 @@ __device__ __forceinline__ void tiny_process(const NumParams& p, const int2* __r
 
 // Every light row with 1 .. TINY_MAX products (split rows carry negative
 // marks in the flops array and are never tiny; with a heavy threshold that
-// low, heavy rows stay with the other kernels' blocks), 32-row chunks dealt
-// to the warps in turn.  Lane l loads what row l of the chunk needs before
+// low, heavy rows stay with the other kernels' blocks), chunks of 32 rows (fewer
+// when there are few: tiny_chunk_rows) dealt to the warps in turn.  Lane l loads what row l of the chunk needs before
 // its rows of B (bounds in A and C, up to TINY_ENT entries of A and their
 // rows' descriptions), all rows of the chunk at once; then the chunk's tiny
 // rows go through a two-stage pipeline: the next row's gathers are issued
@@ -196,12 +196,13 @@ __global__ void __launch_bounds__(256, 4) k_numeric_tiny(NumParams p) {
     const int lane = lane_id();
     unsigned long long* err = &p.hdr->err;
     const int2* Q = reinterpret_cast<const int2*>(p.Bq);
-    const long long nchunks = ((long long)p.nB + 31) / 32;
+    const int cr = p.tiny_rows;
+    const long long nchunks = ((long long)p.nB + cr - 1) / cr;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long c = gw; c < nchunks; c += nw) {
-        const long long r = c * 32 + lane;
-        const long long f = r < p.nB ? __ldg(p.s.flops + r) : 0;
+        const long long r = c * cr + lane;
+        const long long f = lane < cr && r < p.nB ? __ldg(p.s.flops + r) : 0;
         const bool tiny = f >= 1 && f <= TINY_MAX && flops_class(f) < p.cta_class;  // light rows only
         long long a0 = 0, a1 = 0, o0 = 0, o1 = 0;
         if (tiny) {
@@ -281,8 +282,10 @@ __global__ void __launch_bounds__(256, 4) k_numeric_tiny(NumParams p) {
 cudaError_t launch_numeric_tiny(const NumParams& p, int sms, cudaStream_t st) {
     if (p.nB == 0 || !p.Bq) return cudaSuccess;
     const int grid = persistent_grid((const void*)k_numeric_tiny, 256, 0, sms);
+    NumParams q = p;
+    q.tiny_rows = tiny_chunk_rows(p.nB, 8LL * grid);
     count_launch();
-    k_numeric_tiny<<<grid, 256, 0, st>>>(p);
+    k_numeric_tiny<<<grid, 256, 0, st>>>(q);
     return cudaGetLastError();
 }
 

@@ -62,6 +62,45 @@ __device__ __forceinline__ void rg_emit(float* racc, int W, int c0, long long& o
     }
 }
 
+// Read-out of one row whose entries the warp's slots shared: column c is the
+// sum of the slots' accumulators (empty where no slot reached it), in slot
+// order.  Every lane holds the row's output range.
+template <int RG>
+__device__ __forceinline__ void rg_emit_team(float* racc, int W, long long& out, long long out_end, int* Ci,
+                                             float* Cx) {
+    constexpr int R = 32 / RG;
+    const int lane = lane_id();
+    const unsigned lt = lanemask_lt();
+    const long long r = out_end - out;
+    const int room = r < 0x7FFFFFFFLL ? (int)r : 0x7FFFFFFF;
+    int* ci = Ci + out;
+    float* cx = Cx + out;
+    int o = 0;
+#pragma unroll 2
+    for (int base = 0; base < W; base += 32) {
+        const int c = base + lane;
+        unsigned x = RG_EMPTY;
+#pragma unroll
+        for (int h = 0; h < R; ++h) {
+            float* a = racc + h * (W + 8) + c;
+            const unsigned y = __float_as_uint(*a);
+            if (y != RG_EMPTY) {
+                x = x == RG_EMPTY ? y : __float_as_uint(__uint_as_float(x) + __uint_as_float(y));
+                *a = __uint_as_float(RG_EMPTY);
+            }
+        }
+        const bool take = x != RG_EMPTY;
+        const unsigned bal = __ballot_sync(FULL, take);
+        const int pos = o + __popc(bal & lt);
+        if (take && pos < room) {
+            ci[pos] = c;
+            cx[pos] = __uint_as_float(x);
+        }
+        o += __popc(bal);
+    }
+    out += o;
+}
+
 // Column index and value of entry ei of A (k = -1 past the row's end).
 __device__ __forceinline__ void rg_load_a(const NumParams& p, long long ei, bool ok, int& k, float& a) {
     k = -1;

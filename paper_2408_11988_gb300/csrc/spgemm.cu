@@ -71,31 +71,40 @@ __global__ void __launch_bounds__(256) k_flops_rows(long long n, const long long
     const int incl = warp_incl_scan(len), excl = incl - len;
     const int total = __shfl_sync(FULL, incl, 31);
     const long long shift = a0 - excl;  // entry of number p in row q: shift(q) + p
-    for (int p0 = 0; p0 < total; p0 += 32) {
-        const int p = p0 + lane;
-        const int q = owner_lane(excl, p);
-        const long long e = shfl64(shift, q) + p;
-        long long v = 0;
-        if (p < total) {
-            const int k = __ldg(Ai + e);
-            if ((unsigned)k < (unsigned)nB) {
+    constexpr int U = 4;  // rounds of 32 entries in flight
+    for (int p0 = 0; p0 < total; p0 += 32 * U) {
+        int q[U], k[U], v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = p0 + 32 * u + lane;
+            q[u] = owner_lane(excl, p);
+            const long long e = shfl64(shift, q[u]) + p;
+            k[u] = p < total ? __ldg(Ai + e) : -1;
+            if (p < total && (unsigned)k[u] >= (unsigned)nB) atomicOr(err, ERR_A_COL);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            v[u] = 0;
+            if ((unsigned)k[u] < (unsigned)nB) {
                 long long s0;
-                int l;
-                segB(k, s0, l);
-                v = l;
-            } else {
-                atomicOr(err, ERR_A_COL);
+                segB(k[u], s0, v[u]);
             }
         }
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {  // sum over this lane's run of equal q, from this lane on
-            const long long t = shfl64_down(v, o);
-            const int qo = __shfl_down_sync(FULL, q, o);
-            if (lane + o < 32 && qo == q) v += t;
+        for (int u = 0; u < U; ++u) {
+            // sum over this lane's run of equal q, from this lane on (at most
+            // 32 rows of B of at most d entries: an int)
+            int sum = v[u];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_down_sync(FULL, sum, o);
+                const int qo = __shfl_down_sync(FULL, q[u], o);
+                if (lane + o < 32 && qo == q[u]) sum += t;
+            }
+            const int qp = __shfl_up_sync(FULL, q[u], 1);
+            if (p0 + 32 * u + lane < total && (lane == 0 || qp != q[u])) wf[q[u]] += sum;  // one lane per row and round
+            __syncwarp();
         }
-        const int qp = __shfl_up_sync(FULL, q, 1);
-        if (p < total && (lane == 0 || qp != q)) wf[q] += v;  // one lane per row and step
-        __syncwarp();
     }
     if (i < n) flops[i] = nchunks ? 0 : wf[lane];
     // reserve item slots: one atomic per warp
@@ -174,126 +183,21 @@ __global__ void __launch_bounds__(256) k_classify(long long n, const long long* 
         atomicAdd(&s_hist[c], 1u);
         if (c == 0 && Cp_next) Cp_next[i] = 0;
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && Cp_next) Cp_next[-1] = 0;  // C's first row pointer
     __syncthreads();
     for (int c = threadIdx.x; c < NUM_CLASSES; c += blockDim.x)
         if (s_hist[c]) atomicAdd((unsigned long long*)&hdr->hist[c], (unsigned long long)s_hist[c]);
 }
 
-// perm = rows with products, heaviest class first (order inside a class is
-// arbitrary).  Each block ranks its rows per class in shared memory and
-// reserves one range per class with a single global atomic.
-constexpr int SCATTER_ROWS = 8;  // rows per thread
-__global__ void __launch_bounds__(256) k_scatter(long long n, const long long* __restrict__ flops,
-                                                 int* __restrict__ perm, WsHeader* hdr) {
-    __shared__ unsigned s_cnt[NUM_CLASSES];
-    __shared__ long long s_start[NUM_CLASSES];
-    __shared__ long long s_base[NUM_CLASSES];
-    const int tid = threadIdx.x;
-    for (int c = tid; c < NUM_CLASSES; c += blockDim.x) s_cnt[c] = 0;
-    if (tid < 32) {  // start of class c = rows of the classes above it (warp scan, highest class first)
-        long long run = 0;
-        for (int top = NUM_CLASSES - 1; top >= 1; top -= 32) {
-            const int c = top - tid;
-            const long long h = c >= 1 ? hdr->hist[c] : 0;
-            const long long incl = warp_incl_scan(h);
-            if (c >= 1) s_start[c] = run + incl - h;
-            run += __shfl_sync(FULL, incl, 31);
-        }
-        if (tid == 0) s_start[0] = run;
-    }
-    __syncthreads();
-    const long long base = (long long)blockIdx.x * blockDim.x * SCATTER_ROWS;
-    int cls[SCATTER_ROWS];
-    unsigned rank[SCATTER_ROWS];
-#pragma unroll
-    for (int u = 0; u < SCATTER_ROWS; ++u) {
-        const long long i = base + (long long)u * blockDim.x + tid;
-        cls[u] = 0;
-        if (i < n) {
-            cls[u] = flops_class(flops[i]);
-            if (cls[u] > 0) rank[u] = atomicAdd(&s_cnt[cls[u]], 1u);
-        }
-    }
-    __syncthreads();
-    for (int c = tid; c < NUM_CLASSES; c += blockDim.x)
-        s_base[c] = (c > 0 && s_cnt[c])
-                        ? (long long)atomicAdd((unsigned long long*)&hdr->cursor[c], (unsigned long long)s_cnt[c])
-                        : 0;
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < SCATTER_ROWS; ++u) {
-        const long long i = base + (long long)u * blockDim.x + tid;
-        if (i < n && cls[u] > 0) perm[s_start[cls[u]] + s_base[cls[u]] + rank[u]] = (int)i;
-    }
-}
-
-cudaError_t launch_row_flops(const DevCsr& A, const DevCsr& B, const Sched& s, cudaStream_t st) {
-    const long long n = A.nrows;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(s.hdr, 0, sizeof(WsHeader), st))) return e;
-    if (n == 0) return cudaSuccess;
-    const SegWhole segB{B.rowptr, B.nnz, (int)B.ncols};
-    const long long cap = flops_item_capacity(n, A.nnz);
-    const unsigned rb = (unsigned)((n + 255) / 256);
-    if (s.blen && B.nrows > 0) {
-        long long lb = (B.nrows + 255) / 256;
-        if (lb > 152 * 16) lb = 152 * 16;
-        count_launch();
-        k_row_len<<<(unsigned)lb, 256, 0, st>>>(B.nrows, segB, s.blen);
-        const SegLen sl{s.blen};
-        count_launch();
-        k_flops_rows<<<rb, 256, 0, st>>>(n, A.rowptr, A.col, A.nnz, sl, (int)B.nrows, s.flops, s.items, cap, s.hdr);
-        count_launch();
-        k_flops_chunks<<<152 * 8, 256, 0, st>>>(A.rowptr, A.col, A.nnz, sl, (int)B.nrows, s.flops, s.items, cap,
-                                                s.hdr);
-    } else {
-        count_launch();
-        k_flops_rows<<<rb, 256, 0, st>>>(n, A.rowptr, A.col, A.nnz, segB, (int)B.nrows, s.flops, s.items, cap,
-                                         s.hdr);
-        count_launch();
-        k_flops_chunks<<<152 * 8, 256, 0, st>>>(A.rowptr, A.col, A.nnz, segB, (int)B.nrows, s.flops, s.items,
-                                                cap, s.hdr);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reclassify(long long n, const Sched& s, long long* Cp_next, cudaStream_t st) {
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(s.hdr->hist, 0, sizeof(long long) * 2 * NUM_CLASSES, st))) return e;
-    if (n == 0) return cudaSuccess;
-    long long cb = (n + 255) / 256;
-    if (cb > 152 * 16) cb = 152 * 16;
-    count_launch();
-    k_classify<<<(unsigned)cb, 256, 0, st>>>(n, s.flops, Cp_next, s.hdr);
-    const long long sb = (n + 256LL * SCATTER_ROWS - 1) / (256LL * SCATTER_ROWS);
-    count_launch();
-    k_scatter<<<(unsigned)sb, 256, 0, st>>>(n, s.flops, s.perm, s.hdr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_row_schedule(const DevCsr& A, const DevCsr& B, const Sched& s, long long* Cp,
-                                cudaStream_t st) {
-    cudaError_t e;
-    if ((e = launch_row_flops(A, B, s, st))) return e;
-    return launch_reclassify(A.nrows, s, Cp ? Cp + 1 : nullptr, st);
-}
-
-// ---------------------------------------------------------------------------
 // Split rows: a row with more than SPLIT_ENTRIES entries of A (and some
 // products) gets a slot u < MAX_SPLIT_ROWS and ceil(len / SPLIT_ENTRIES)
 // work items (u, part) that any block may take, so that one very heavy row
 // is spread over many SMs instead of forming the tail of the pass.  The
 // row's flops entry becomes the mark -1 - u, and its staging slot is cleared.
-// ---------------------------------------------------------------------------
 long long split_item_capacity(long long nnzA) { return nnzA / SPLIT_ENTRIES + MAX_SPLIT_ROWS + 1; }
 
-__global__ void __launch_bounds__(256) k_split_rows(long long n, const long long* __restrict__ Ap, long long nnzA,
-                                                    long long* flops, Sched s, long long item_cap) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const long long a0 = clampll(Ap[i], 0, nnzA), a1 = clampll(Ap[i + 1], a0, nnzA);
-    const long long alen = a1 - a0;
-    if (alen <= SPLIT_ENTRIES || flops[i] <= 0) return;
+__device__ __forceinline__ void split_row(long long i, long long alen, long long* flops, const Sched& s,
+                                          long long item_cap) {
     const long long u = (long long)atomicAdd((unsigned long long*)&s.hdr->scratch[1], 1ull);
     if (u >= MAX_SPLIT_ROWS) return;  // out of slots: the row runs whole
     const long long nsub = (alen + SPLIT_ENTRIES - 1) / SPLIT_ENTRIES;
@@ -317,6 +221,123 @@ __global__ void __launch_bounds__(256) k_split_rows(long long n, const long long
     flops[i] = -1 - u;
 }
 
+// perm = rows with products, heaviest class first (order inside a class is
+// arbitrary).  Each block ranks its rows per class in shared memory and
+// reserves one range per class with a single global atomic.  Ap != nullptr:
+// rows of many entries are cut into split items on the way.  The classes'
+// running sums come from one load of the histogram and a scan in shared
+// memory, a warp's lane taking 13 classes (as a loop of loads and warp scans
+// they were 10 of the kernel's 14 us for a small product).
+constexpr int SCATTER_ROWS = 8;  // rows per thread
+__global__ void __launch_bounds__(256) k_scatter(long long n, long long* flops, int* __restrict__ perm, WsHeader* hdr,
+                                                 const long long* __restrict__ Ap, long long nnzA, Sched s,
+                                                 long long item_cap) {
+    __shared__ unsigned s_cnt[NUM_CLASSES];
+    __shared__ long long s_start[NUM_CLASSES];
+    __shared__ long long s_base[NUM_CLASSES];
+    const int tid = threadIdx.x;
+    for (int c = tid; c < NUM_CLASSES; c += blockDim.x) {
+        s_cnt[c] = 0;
+        s_start[c] = c ? hdr->hist[c] : 0;
+    }
+    const long long base = (long long)blockIdx.x * blockDim.x * SCATTER_ROWS;
+    int cls[SCATTER_ROWS];
+    unsigned rank[SCATTER_ROWS];
+#pragma unroll
+    for (int u = 0; u < SCATTER_ROWS; ++u) {
+        const long long i = base + (long long)u * blockDim.x + tid;
+        cls[u] = i < n ? flops_class(flops[i]) : 0;
+    }
+    __syncthreads();
+    if (tid < 32) {  // start of class c = rows of the classes above it
+        constexpr int PER = (NUM_CLASSES + 31) / 32;
+        const int top = NUM_CLASSES - 1 - PER * tid;  // this lane's classes: top, top - 1, ...
+        long long sum = 0;
+        for (int j = 0; j < PER; ++j) sum += top - j >= 0 ? s_start[top - j] : 0;
+        long long run = warp_incl_scan(sum) - sum;
+        for (int j = 0; j < PER; ++j) {
+            if (top - j < 0) break;
+            const long long h = s_start[top - j];
+            s_start[top - j] = run;
+            run += h;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < SCATTER_ROWS; ++u)
+        if (cls[u] > 0) rank[u] = atomicAdd(&s_cnt[cls[u]], 1u);
+    __syncthreads();
+    if (blockIdx.x == 0)
+        for (int c = tid; c < NUM_CLASSES; c += blockDim.x) hdr->above[c] = s_start[c];
+    for (int c = tid; c < NUM_CLASSES; c += blockDim.x)
+        s_base[c] = (c > 0 && s_cnt[c])
+                        ? (long long)atomicAdd((unsigned long long*)&hdr->cursor[c], (unsigned long long)s_cnt[c])
+                        : 0;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < SCATTER_ROWS; ++u) {
+        const long long i = base + (long long)u * blockDim.x + tid;
+        if (i >= n || cls[u] == 0) continue;
+        perm[s_start[cls[u]] + s_base[cls[u]] + rank[u]] = (int)i;
+        if (Ap) {
+            const long long a0 = clampll(__ldg(Ap + i), 0, nnzA), a1 = clampll(__ldg(Ap + i + 1), a0, nnzA);
+            if (a1 - a0 > SPLIT_ENTRIES) split_row(i, a1 - a0, flops, s, item_cap);
+        }
+    }
+}
+
+// B's row lengths as an array of their own pay from this many rows of B on
+// (below, the flops pass reads row pointers and saves a launch).
+constexpr long long ROW_LEN_MIN = 65536;
+
+cudaError_t launch_row_flops(const DevCsr& A, const DevCsr& B, const Sched& s, cudaStream_t st) {
+    const long long n = A.nrows;
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(s.hdr, 0, sizeof(WsHeader), st))) return e;
+    if (n == 0) return cudaSuccess;
+    const SegWhole segB{B.rowptr, B.nnz, (int)B.ncols};
+    const long long cap = flops_item_capacity(n, A.nnz);
+    const unsigned rb = (unsigned)((n + 255) / 256);
+    // a warp per chunk of a long row; none can exist in a matrix this small
+    const unsigned cb = A.nnz > SHORT_ROW ? (unsigned)(cap < 152 * 64 ? (cap + 7) / 8 : 152 * 8) : 0;
+    auto run = [&](auto seg) {
+        using Seg = decltype(seg);
+        count_launch();
+        k_flops_rows<Seg><<<rb, 256, 0, st>>>(n, A.rowptr, A.col, A.nnz, seg, (int)B.nrows, s.flops, s.items, cap, s.hdr);
+        if (!cb) return;
+        count_launch();
+        k_flops_chunks<Seg><<<cb, 256, 0, st>>>(A.rowptr, A.col, A.nnz, seg, (int)B.nrows, s.flops, s.items, cap, s.hdr);
+    };
+    if (s.blen && B.nrows >= ROW_LEN_MIN) {
+        long long lb = (B.nrows + 255) / 256;
+        if (lb > 152 * 16) lb = 152 * 16;
+        count_launch();
+        k_row_len<<<(unsigned)lb, 256, 0, st>>>(B.nrows, segB, s.blen);
+        run(SegLen{s.blen});
+    } else {
+        run(segB);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reclassify(long long n, const Sched& s, long long* Cp_next, cudaStream_t st, const DevCsr* A) {
+    if (n == 0) return cudaSuccess;
+    long long cb = (n + 255) / 256;
+    if (cb > 152 * 16) cb = 152 * 16;
+    count_launch();
+    k_classify<<<(unsigned)cb, 256, 0, st>>>(n, s.flops, Cp_next, s.hdr);
+    const long long sb = (n + 256LL * SCATTER_ROWS - 1) / (256LL * SCATTER_ROWS);
+    count_launch();
+    k_scatter<<<(unsigned)sb, 256, 0, st>>>(n, s.flops, s.perm, s.hdr, A ? A->rowptr : nullptr, A ? A->nnz : 0, s,
+                                            A ? split_item_capacity(A->nnz) : 0);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_row_schedule(const DevCsr& A, const DevCsr& B, const Sched& s, long long* Cp,
+                                cudaStream_t st) {
+    cudaError_t e;
+    if ((e = launch_row_flops(A, B, s, st))) return e;
+    return launch_reclassify(A.nrows, s, Cp ? Cp + 1 : nullptr, st, &A);
+}
 
 // ---------------------------------------------------------------------------
 // Symbolic pass: nnz(C_i) = number of distinct columns over the rows B_k,
@@ -401,6 +422,7 @@ struct SymParams {
     long long item_cap;
     int skip_light;  // 1: split and heavy rows only (light rows run in k_symbolic_light)
     int tiny;        // 1: light rows of classes <= SYM_TINY_CLASS are counted by k_symbolic_tiny
+    int tiny_rows;   // rows per chunk of that kernel
 };
 
 // Rows with at most 31 products (flops classes 1 .. 40, eighths of an
@@ -496,8 +518,8 @@ __device__ __forceinline__ int block_sum(int c, int* s_red) {
 // entry of A has as many columns as its row of B (flops_i itself); a longer
 // one has its rows of B's columns placed one per lane, sorted (two rows: one
 // bitonic merge of the first row and the second reversed at the top lanes;
-// more: the full network) and the distinct ones counted.  32-row chunks are
-// dealt to the warps in turn; the one-entry rows of a chunk are counted lane
+// more: the full network) and the distinct ones counted.  Chunks of 32 rows (fewer
+// when there are few, tiny_chunk_rows) are dealt to the warps in turn; the one-entry rows of a chunk are counted lane
 // by lane.  Called when d is too wide for the row-group light kernel, where
 // each light row costs a pass over d/4 words of byte marks.
 __device__ __forceinline__ void warp_sort_keys(int& key) {
@@ -517,12 +539,13 @@ __global__ void __launch_bounds__(256) k_symbolic_tiny(SymParams p) {
     const int lane = lane_id();
     unsigned long long* err = &p.hdr->err;
     const long long* flops = p.s.flops;
-    const long long nchunks = ((long long)p.nB + 31) / 32;
+    const int cr = p.tiny_rows;
+    const long long nchunks = ((long long)p.nB + cr - 1) / cr;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long c = gw; c < nchunks; c += nwarps) {
-        const long long r = c * 32 + lane;
-        const long long f = r < p.nB ? __ldg(flops + r) : 0;
+        const long long r = c * cr + lane;
+        const long long f = lane < cr && r < p.nB ? __ldg(flops + r) : 0;
         const int cls = flops_class(f);
         const bool tiny = f >= 1 && cls <= SYM_TINY_CLASS && cls < p.cta_class;
         long long a0 = 0, a1 = 0;
@@ -561,7 +584,7 @@ __global__ void __launch_bounds__(256) k_symbolic_tiny(SymParams p) {
                     }
                     const int prev = __shfl_up_sync(FULL, key, 1);
                     const unsigned heads = __ballot_sync(FULL, key != 0x7FFFFFFF && (lane == 0 || prev != key));
-                    if (lane == 0) p.Cp_next[c * 32 + src] = __popc(heads);
+                    if (lane == 0) p.Cp_next[c * cr + src] = __popc(heads);
                     continue;
                 }
             }
@@ -591,7 +614,7 @@ __global__ void __launch_bounds__(256) k_symbolic_tiny(SymParams p) {
             warp_sort_keys(key);
             const int prev = __shfl_up_sync(FULL, key, 1);
             const unsigned heads = __ballot_sync(FULL, key != 0x7FFFFFFF && (lane == 0 || prev != key));
-            if (lane == 0) p.Cp_next[c * 32 + src] = __popc(heads);
+            if (lane == 0) p.Cp_next[c * cr + src] = __popc(heads);
         }
     }
 }
@@ -606,6 +629,7 @@ __global__ void __launch_bounds__(256, 8) k_symbolic(SymParams p) {
     __shared__ int s_red[32];
     __shared__ int s_full;  // the current item's marks hold all d columns
     const int nw = blockDim.x >> 5, warp = warp_id(), lane = lane_id(), tid = threadIdx.x;
+    if (p.skip_light && nothing_heavy(p.hdr, p.cta_class)) return;
     for (int i = tid; i < nw * p.slot; i += blockDim.x) smem_u[i] = 0;
     if (tid == 0) s_full = 0;
     if (tid < 32) {  // one warp; its lanes store the same values
@@ -689,9 +713,8 @@ __global__ void __launch_bounds__(256, 8) k_symbolic(SymParams p) {
     if (p.skip_light) return;
     long long nlight_end = nrows;
     if (p.tiny) {
-        long long t = 0;
-        for (int c = 1 + lane; c <= SYM_TINY_CLASS && c < p.cta_class; c += 32) t += p.hdr->hist[c];
-        nlight_end -= warp_sum(t);
+        const int last = SYM_TINY_CLASS < p.cta_class ? SYM_TINY_CLASS : p.cta_class - 1;
+        nlight_end -= nrows - rows_from_class(p.hdr, last + 1);
     }
     unsigned* bm = smem_u + warp * p.slot;
     SymRowBody<G, FL> body{p, bm, err};
@@ -740,30 +763,32 @@ __device__ __forceinline__ void symrg_mark(unsigned char* fl, const int c[4], in
 template <int RG>
 __global__ void __launch_bounds__(256, 5) k_symbolic_light(SymParams p) {
     extern __shared__ __align__(16) unsigned smem_u[];
-    __shared__ long long s_nheavy, s_nrows;
+    __shared__ LightUnits s_lu;
     constexpr int R = 32 / RG;
     const int nw = blockDim.x >> 5, warp = warp_id(), lane = lane_id(), tid = threadIdx.x;
     const int g = lane / RG, gl = lane % RG;
     const int slotw = 8 * p.dw;  // words of one row's dpad bytes
     for (int i = tid; i < nw * R * slotw; i += blockDim.x) smem_u[i] = 0u;
     if (tid < 32) {  // one warp; its lanes store the same values
-        long long nh, nr;
-        sched_counts(p.hdr, p.cta_class, nh, nr);
-        s_nheavy = nh;
-        s_nrows = nr;
+        LightUnits lu;
+        lu.init(p.hdr, p.cta_class, R, 0, gridDim.x * nw);
+        s_lu = lu;
     }
     __syncthreads();
-    unsigned* fw = smem_u + (size_t)(warp * R + g) * slotw;
-    unsigned char* fl = reinterpret_cast<unsigned char*>(fw);
+    const LightUnits& lu = s_lu;
     unsigned long long* err = &p.hdr->err;
     const long long* mark = p.s.flops;
-    const long long end = s_nrows, step = (long long)gridDim.x * nw * R;
     const long long nnzB = p.segB.nnzB;
-    for (long long idx = s_nheavy + ((long long)blockIdx.x * nw + warp) * R; idx < end; idx += step) {
-        const long long my = idx + g;
+    for (unsigned un = blockIdx.x * nw + warp; un < lu.units; un += gridDim.x * nw) {
+        // a unit is R rows, a slot each, or one row whose entries the slots
+        // share: they all mark slot 0's bytes (equal stores)
+        const bool team = lu.team(un);
+        unsigned* fw = smem_u + (size_t)(warp * R + (team ? 0 : g)) * slotw;
+        unsigned char* fl = reinterpret_cast<unsigned char*>(fw);
+        const unsigned my = lu.row_at(un, g, R);
         long long a0 = 0, a1 = 0;
         int row = -1;
-        if (my < end) {
+        if (my < lu.end) {
             row = __ldg(p.perm + my);
             a0 = clampll(__ldg(p.Ap + row), 0, p.nnzA);
             a1 = clampll(__ldg(p.Ap + row + 1), a0, p.nnzA);
@@ -772,7 +797,8 @@ __global__ void __launch_bounds__(256, 5) k_symbolic_light(SymParams p) {
                 row = -1;
             }
         }
-        const int len = (int)(a1 - a0);
+        int len = (int)(a1 - a0);
+        if (team) team_share(g, R, a0, len);
         const int lmax = (int)__reduce_max_sync(FULL, (unsigned)len);
         // chunks of RG entries, pipelined: while chunk e is marked, the
         // segment of chunk e + RG (B's row pointers) and the column of
@@ -819,7 +845,7 @@ __global__ void __launch_bounds__(256, 5) k_symbolic_light(SymParams p) {
         }
         __syncwarp();
         int c = 0;
-        for (int w = 4 * gl; w < slotw; w += 4 * RG) {
+        for (int w = 4 * (team ? lane : gl); w < slotw; w += team ? 128 : 4 * RG) {
             uint4* q = reinterpret_cast<uint4*>(fw + w);
             const uint4 v = *q;
             c += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
@@ -827,10 +853,20 @@ __global__ void __launch_bounds__(256, 5) k_symbolic_light(SymParams p) {
         }
 #pragma unroll
         for (int o = RG / 2; o >= 1; o >>= 1) c += __shfl_xor_sync(FULL, c, o, RG);
-        if (row >= 0 && gl == 0) p.Cp_next[row] = c;
+        if (team) {
+#pragma unroll
+            for (int o = 16; o >= RG; o >>= 1) c += __shfl_xor_sync(FULL, c, o);
+        }
+        if (row >= 0 && gl == 0 && (!team || g == 0)) p.Cp_next[row] = c;
         __syncwarp();
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+int tiny_chunk_rows(long long n, long long nwarps) {
+    int rows = 32;
+    while (rows > 2 && n < rows * nwarps) rows /= 2;
+    return rows;
 }
 
 static std::atomic<long long> g_launches{0};
@@ -855,12 +891,8 @@ cudaError_t launch_symbolic(const DevCsr& A, const DevCsr& B, long long d, const
                             const LaunchCfg& cfg, long long* Cp, cudaStream_t st) {
     cudaError_t e;
     const long long n = A.nrows;
-    if ((e = cudaMemsetAsync(Cp, 0, sizeof(long long), st))) return e;
-    if (n == 0) return cudaSuccess;
-    if ((e = cudaMemsetAsync(&s.hdr->heavy_ctr, 0, 2 * sizeof(unsigned long long), st))) return e;
+    if (n == 0) return cudaMemsetAsync(Cp, 0, sizeof(long long), st);
     const long long item_cap = split_item_capacity(A.nnz);
-    count_launch();
-    k_split_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, A.rowptr, A.nnz, s.flops, s, item_cap);
     SymParams p;
     p.Ap = A.rowptr;
     p.Ai = A.col;
@@ -909,6 +941,7 @@ cudaError_t launch_symbolic(const DevCsr& A, const DevCsr& B, long long d, const
     if (!rg_ok && cfg.row_lanes != 32 && d > 256) {
         p.tiny = 1;
         const int tgrid = persistent_grid((const void*)k_symbolic_tiny, 256, 0, cfg.sms);
+        p.tiny_rows = tiny_chunk_rows(n, 8LL * tgrid);
         count_launch();
         k_symbolic_tiny<<<tgrid, 256, 0, st>>>(p);
         if ((e = cudaGetLastError())) return e;
@@ -998,19 +1031,25 @@ __global__ void __launch_bounds__(1024) k_scan_partials(long long* partial, long
     if (threadIdx.x == 0) partial[nb] = carry;
 }
 
+// PARTIALS: partial holds the running sums (k_scan_partials); otherwise the
+// sums themselves, and every block adds up those before its tile.
+template <bool PARTIALS>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(long long* x, long long n,
                                                              const long long* __restrict__ partial) {
     const long long base = (long long)blockIdx.x * SCAN_TILE + (long long)threadIdx.x * SCAN_PER_THREAD;
     long long v[SCAN_PER_THREAD];
-    long long run = 0;
+    long long run = 0, before = 0;
+    if (!PARTIALS)
+        for (unsigned t = threadIdx.x; t < blockIdx.x; t += SCAN_THREADS) before += partial[t];
 #pragma unroll
     for (int u = 0; u < SCAN_PER_THREAD; ++u) {
         const long long i = base + u;
         run += (i < n) ? x[i] : 0;
         v[u] = run;
     }
-    long long tot;
-    const long long ex = block_excl_scan<SCAN_THREADS>(run, tot) + partial[blockIdx.x];
+    long long tot, all = 0;
+    if (!PARTIALS && blockIdx.x > 0) block_excl_scan<SCAN_THREADS>(before, all);
+    const long long ex = block_excl_scan<SCAN_THREADS>(run, tot) + (PARTIALS ? partial[blockIdx.x] : all);
 #pragma unroll
     for (int u = 0; u < SCAN_PER_THREAD; ++u) {
         const long long i = base + u;
@@ -1018,11 +1057,17 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(long long* x, long 
     }
 }
 
+// Tiles up to which every block of k_scan_apply sums the tiles before its own
+// (at most four loads a thread) instead of waiting for a kernel of one block.
+constexpr long long SCAN_FEW = 4 * SCAN_THREADS;
+
 cudaError_t launch_scan_inplace(long long* x, long long n, long long* partial, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const long long nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    count_launch();
-    k_scan_reduce<<<(unsigned)nb, SCAN_THREADS, 0, st>>>(x, n, partial);
+    if (nb > 1) {
+        count_launch();
+        k_scan_reduce<<<(unsigned)nb, SCAN_THREADS, 0, st>>>(x, n, partial);
+    }
     return launch_scan_summed(x, n, partial, st);
 }
 
@@ -1031,10 +1076,15 @@ int scan_tile_rows() { return SCAN_TILE; }
 cudaError_t launch_scan_summed(long long* x, long long n, long long* partial, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const long long nb = (n + SCAN_TILE - 1) / SCAN_TILE;
+    if (nb <= SCAN_FEW) {
+        count_launch();
+        k_scan_apply<false><<<(unsigned)nb, SCAN_THREADS, 0, st>>>(x, n, partial);
+        return cudaGetLastError();
+    }
     count_launch();
     k_scan_partials<<<1, 1024, 0, st>>>(partial, nb);
     count_launch();
-    k_scan_apply<<<(unsigned)nb, SCAN_THREADS, 0, st>>>(x, n, partial);
+    k_scan_apply<true><<<(unsigned)nb, SCAN_THREADS, 0, st>>>(x, n, partial);
     return cudaGetLastError();
 }
 
