@@ -1,260 +1,329 @@
-// Sparse Force2Vec minibatch step around the TS-SpGEMM (paper Sec. IV,
-// "Distributed sparse embedding"), for the rows [r0, r0 + b) of a sparse
-// embedding Z (n x d, exactly k stored entries per row, row i at [k*i, k*i+k)):
+// Sparse Force2Vec minibatch step (paper Sec. IV, "Distributed sparse
+// embedding"), for the rows [r0, r0 + b) of a sparse embedding Z (n x d,
+// exactly k stored entries per row, row i at [k*i, k*i+k)):
 //
-//   1. W's pattern: row r of the batch merges the neighbours of vertex r0 + r
-//      in A (weight class +1) with its s negative samples (class -1); a column
-//      met several times keeps its counts of both classes (k_f2v_newmask,
-//      k_f2v_rowlen, k_f2v_fill_a, k_f2v_fill_n: a thread per sample or per
-//      entry, so that hub rows add no tail);
-//   2. weights (a sampled product on W's pattern): x = z_i . z_j by a merge
-//      of the two rows of Z, w = npos * (1 - sigmoid(x)) - nneg * sigmoid(x)
-//      (k_f2v_weights, a thread per entry of W);
-//   3. G = W * Z, the plus-times TS-SpGEMM of this library (symbolic and
-//      numeric passes, run by the C ABI layer);
-//   4. U = Z_batch + lr * G, then the k entries of each row of U of largest
-//      magnitude (ties: smaller column) in ascending column order, by a
-//      radix select on the magnitude's bit pattern (k_f2v_update);
-//   5. the new rows replace the batch rows of Z (k_f2v_commit), after every
-//      row of the batch was computed from the old Z (synchronous SGD).
+//   U_i = z_i + lr * (sum over the neighbours j of vertex i in A of
+//           (1 - sigmoid(z_i . z_j)) z_j  -  sum over i's s negative samples j
+//           of sigmoid(z_i . z_j) z_j),
+//
+// then the k entries of U_i of largest magnitude (ties: smaller column) in
+// ascending column order, by a radix select on the magnitude's bit pattern.
+// A column met several times (a neighbour that is also a sample, a sample
+// drawn twice) is as many terms: the product W * Z of the weight matrix with
+// Z, row by row, without forming W.
+//
+// One kernel does all of it for a row: its warp holds z_i and the sum densely
+// in shared memory and, for each term, loads z_j once, takes the dot product,
+// the weight, and adds w * z_j (columns of one row of Z are distinct: plain
+// adds).  The path is bound by the latency of those gathers (a minibatch of
+// 4096 rows and 5 samples reads 150,000 rows of 208 bytes, from L2 mostly), so
+// four terms are in flight per warp and the next four load meanwhile.  A row
+// of more than F2V_CHUNK terms (a hub) is cut into chunks taken by any warp,
+// their sums added into a row of scratch; the warp of its last chunk finishes
+// the row.  The new rows replace the batch rows of Z at the end (k_f2v_commit),
+// after every row was computed from the old Z (synchronous SGD).
+//
+// As passes of their own (W's pattern, its weights, the row schedule and two
+// passes of the general product with a packed copy of all of Z, the update: 24
+// launches) a minibatch of 4096 rows, d = 128, took 364 us; now 104 us, of which
+// the two kernels take 31 us each.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace ts {
 
-constexpr int F2V_MAX_NEG = 32;
+// Terms per chunk: a chunk is a serial chain of some 300 ns a term pair, and the
+// batch is done when its longest one is (minibatch at 128 / 64 / 32 terms: 150 /
+// 122 / 104 us).  Terms in flight: eight instead of four hide nothing more
+// (114 us) and cost a block per SM.
+constexpr int F2V_CHUNK = 32;
+constexpr int F2V_FLIGHT = 4;
+constexpr unsigned F2V_EMPTY = 0x80000000u;  // -0.0: a column no term reached (x + -0.0 is x)
 
-// Entry-parallel construction of W's pattern (no thread walks a whole row,
-// so hub rows add no tail).  A negative sample of row r is "new" when it is
-// the first occurrence of its vertex among the row's samples and not a
-// neighbour; W's row r is A's row with the new negatives inserted in column
-// order, each column carrying its count of neighbour (0/1) and negative
-// occurrences.
+// Layout of the workspace for a batch of b rows with at most `terms` terms.
+struct F2vWs {
+    F2vCtl* ctl;
+    long long* items;  // (row of the batch, chunk) of the long rows
+    int* done;         // chunks finished, per row
+    float* G;          // sums of the long rows, [b][d]
+    int* Sc;
+    float* Sv;
+};
 
-// First position in the ascending A(i, :) whose column is >= c.
-__device__ __forceinline__ long long f2v_lower(const int* __restrict__ Ai, long long a0, long long a1, int c) {
-    long long lo = a0, hi = a1;
-    while (lo < hi) {
-        const long long mid = (lo + hi) >> 1;
-        if (__ldg(Ai + mid) < c) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
+// Chunks of the long rows: a row of t > F2V_CHUNK terms has at most
+// 2 t / F2V_CHUNK.
+static long long f2v_item_capacity(long long terms) { return 2 * (terms / F2V_CHUNK) + 1; }
+
+static size_t f2v_ws(char* base, long long d, long long nnzA, long long b, long long s, long long k, F2vWs* out) {
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* p = base + off;
+        off += (bytes + 255) & ~(size_t)255;
+        return p;
+    };
+    F2vWs w;
+    w.ctl = (F2vCtl*)take(sizeof(F2vCtl));
+    w.items = (long long*)take(sizeof(long long) * (size_t)f2v_item_capacity(nnzA + b * s));
+    w.done = (int*)take(sizeof(int) * (size_t)b);
+    w.G = (float*)take(sizeof(float) * (size_t)(b * d));
+    w.Sc = (int*)take(sizeof(int) * (size_t)(b * k));
+    w.Sv = (float*)take(sizeof(float) * (size_t)(b * k));
+    if (out) *out = w;
+    return off;
 }
 
-// Thread per (row, sample): the row's mask of new samples.
-__global__ void __launch_bounds__(256) k_f2v_newmask(const long long* __restrict__ Ap, const int* __restrict__ Ai,
-                                                     long long nnzA, int n, long long r0, long long b,
-                                                     const int* __restrict__ neg, int s, unsigned* newmask,
-                                                     unsigned long long* err) {
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= b * s) return;
-    const long long r = q / s;
-    const int t = (int)(q - r * s);
-    const int v = __ldg(neg + q);
-    if ((unsigned)v >= (unsigned)n) {
-        atomicOr(err, ERR_A_COL);
-        return;
-    }
-    for (int u = 0; u < t; ++u)
-        if (__ldg(neg + r * s + u) == v) return;  // not the first occurrence
-    const long long i = r0 + r;
-    const long long a0 = clampll(__ldg(Ap + i), 0, nnzA), a1 = clampll(__ldg(Ap + i + 1), a0, nnzA);
-    const long long p = f2v_lower(Ai, a0, a1, v);
-    if (p < a1 && __ldg(Ai + p) == v) return;  // a neighbour
-    atomicOr(newmask + r, 1u << t);
+size_t f2v_bytes(long long d, long long nnzA, long long b, long long s, long long k) {
+    return f2v_ws(nullptr, d, nnzA, b, s, k, nullptr);
 }
 
-// Thread per row: W's row length (into Wp + 1, scanned afterwards).
-__global__ void __launch_bounds__(256) k_f2v_rowlen(const long long* __restrict__ Ap, long long nnzA, long long r0,
-                                                    long long b, const unsigned* __restrict__ newmask, long long* cnt) {
-    const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= b) return;
-    const long long a0 = clampll(__ldg(Ap + r0 + r), 0, nnzA), a1 = clampll(__ldg(Ap + r0 + r + 1), a0, nnzA);
-    cnt[r] = (a1 - a0) + __popc(newmask[r]);
-}
+struct F2vParams {
+    const long long* Ap;
+    const int* Ai;
+    long long nnzA;
+    int n;
+    long long r0, b;
+    const int* neg;
+    int s;
+    const long long* Zp;
+    const int* Zc;
+    const float* Zv;
+    int k, d, dpad;
+    float lr;
+    float* U_out;
+    F2vWs ws;
+    long long item_cap;
+};
 
-// Among row r's samples: how many new ones have a column below c, and how
-// many samples (all occurrences) equal c.
-__device__ __forceinline__ void f2v_negstats(const int* __restrict__ neg, long long r, int s, unsigned mask, int c,
-                                             int& below, int& eq) {
-    below = 0;
-    eq = 0;
-    for (int t = 0; t < s; ++t) {
-        const int v = __ldg(neg + r * s + t);
-        below += ((mask >> t) & 1u) && v < c;
-        eq += v == c;
-    }
-}
-
-// Thread per entry of A in the batch rows: its place in W.
-__global__ void __launch_bounds__(256) k_f2v_fill_a(const long long* __restrict__ Ap, const int* __restrict__ Ai,
-                                                    long long nnzA, long long r0, long long b,
-                                                    const int* __restrict__ neg, int s,
-                                                    const unsigned* __restrict__ newmask, const long long* Wp,
-                                                    int* Wcol, int* Wmult, int* Wrow) {
-    const long long base = clampll(__ldg(Ap + r0), 0, nnzA), top = clampll(__ldg(Ap + r0 + b), base, nnzA);
-    for (long long e = base + (long long)blockIdx.x * blockDim.x + threadIdx.x; e < top;
-         e += (long long)gridDim.x * blockDim.x) {
-        long long lo = 0, hi = b;  // row: the last r with Ap[r0 + r] <= e
-        while (hi - lo > 1) {
-            const long long mid = (lo + hi) >> 1;
-            if (__ldg(Ap + r0 + mid) <= e) lo = mid;
-            else hi = mid;
-        }
-        const long long r = lo;
-        const int c = __ldg(Ai + e);
-        int below, eq;
-        f2v_negstats(neg, r, s, newmask[r], c, below, eq);
-        const long long pos = Wp[r] + (e - __ldg(Ap + r0 + r)) + below;
-        if (pos < Wp[r + 1]) {
-            Wcol[pos] = c;
-            Wmult[pos] = 1 | (eq << 16);
-            Wrow[pos] = (int)r;
-        }
+// Row i of Z scattered into the dense shared row g (cleared before).
+__device__ __forceinline__ void f2v_scatter(const F2vParams& p, long long i, float* g) {
+    for (int t = lane_id(); t < p.k; t += 32) {
+        const int c = __ldg(p.Zc + i * p.k + t);
+        if ((unsigned)c < (unsigned)p.d) g[c] = __ldg(p.Zv + i * p.k + t);
+        else atomicOr(&p.ws.ctl->err, ERR_B_COL);
     }
 }
 
-// Thread per (row, new sample): its place in W.
-__global__ void __launch_bounds__(256) k_f2v_fill_n(const long long* __restrict__ Ap, const int* __restrict__ Ai,
-                                                    long long nnzA, long long r0, long long b,
-                                                    const int* __restrict__ neg, int s,
-                                                    const unsigned* __restrict__ newmask, const long long* Wp,
-                                                    int* Wcol, int* Wmult, int* Wrow) {
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= b * s) return;
-    const long long r = q / s;
-    const int t = (int)(q - r * s);
-    const unsigned mask = newmask[r];
-    if (!((mask >> t) & 1u)) return;
-    const int c = __ldg(neg + q);
-    const long long i = r0 + r;
-    const long long a0 = clampll(__ldg(Ap + i), 0, nnzA), a1 = clampll(__ldg(Ap + i + 1), a0, nnzA);
-    int below, eq;
-    f2v_negstats(neg, r, s, mask, c, below, eq);
-    const long long pos = Wp[r] + (f2v_lower(Ai, a0, a1, c) - a0) + below;
-    if (pos < Wp[r + 1]) {
-        Wcol[pos] = c;
-        Wmult[pos] = eq << 16;
-        Wrow[pos] = (int)r;
-    }
-}
-
-// Z must hold exactly k entries per row: Zp[i] = k * i (else ERR_CAPACITY).
-__global__ void __launch_bounds__(256) k_f2v_check_rows(const long long* __restrict__ Zp, long long n, int k,
-                                                        unsigned long long* err) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i <= n && __ldg(Zp + i) != (long long)k * i) atomicOr(err, ERR_CAPACITY);
-}
-
-// Row i of Z scattered into the dense shared row g (or cleared again).
-__device__ __forceinline__ void f2v_scatter(const int* __restrict__ Zc, const float* __restrict__ Zv, long long i,
-                                            int k, int d, float* g, bool clear) {
-    for (int t = lane_id(); t < k; t += 32) {
-        const int c = __ldg(Zc + i * k + t);
-        if ((unsigned)c < (unsigned)d) g[c] = clear ? 0.0f : __ldg(Zv + i * k + t);
-    }
-}
-
-// Thread per entry of W: x = z_i . z_j by a merge of the two ascending rows
-// of Z, then the entry's weight.
-__global__ void __launch_bounds__(256) k_f2v_weights(const int* __restrict__ Zc, const float* __restrict__ Zv,
-                                                     long long n, int k, long long r0, const long long* __restrict__ Wp,
-                                                     long long b, const int* __restrict__ Wcol,
-                                                     const int* __restrict__ Wmult, const int* __restrict__ Wrow,
-                                                     float* Wval) {
-    const long long nW = Wp[b];
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nW;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long i = r0 + __ldg(Wrow + e), j = __ldg(Wcol + e);
-        if ((unsigned long long)j >= (unsigned long long)n || (unsigned long long)i >= (unsigned long long)n) {
-            Wval[e] = 0.0f;  // a bad column of A: flagged by the product pass
-            continue;
-        }
-        const int* ci = Zc + i * k;
-        const int* cj = Zc + j * k;
-        float x = 0.0f;
-        int p = 0, q = 0;
-        int a = __ldg(ci), c = __ldg(cj);
-        while (p < k && q < k) {
-            if (a == c) x += __ldg(Zv + i * k + p) * __ldg(Zv + j * k + q);
-            const bool adv_p = a <= c, adv_q = c <= a;
-            if (adv_p && ++p < k) a = __ldg(ci + p);
-            if (adv_q && ++q < k) c = __ldg(cj + q);
-        }
-        const int m = __ldg(Wmult + e);
-        const float sg = 1.0f / (1.0f + expf(-x));
-        Wval[e] = (float)(m & 0xFFFF) * (1.0f - sg) - (float)(m >> 16) * sg;
-    }
-}
-
-// U = Z_batch + lr * G per row (dense in shared memory), optional dense copy
-// to U_out, then the k entries of largest magnitude into the staging rows.
-__global__ void __launch_bounds__(256) k_f2v_update(const int* __restrict__ Zc, const float* __restrict__ Zv,
-                                                    int d, int k, long long r0, long long b,
-                                                    const long long* __restrict__ Gp, const int* __restrict__ Gc,
-                                                    const float* __restrict__ Gv, float lr, float* U_out,
-                                                    int* Sc, float* Sv, unsigned long long* err) {
-    extern __shared__ __align__(16) float fsm[];
-    const int nw = blockDim.x >> 5, warp = warp_id(), lane = lane_id();
-    const int dpad = (d + 31) & ~31;
-    const int mb = dpad >> 5;
-    const unsigned lt = lanemask_lt();
-    float* u = fsm + (size_t)warp * dpad;
-    for (int c = lane; c < dpad; c += 32) u[c] = 0.0f;
-    __syncwarp();
-    for (long long r = (long long)blockIdx.x * nw + warp; r < b; r += (long long)gridDim.x * nw) {
-        const long long i = r0 + r;
-        f2v_scatter(Zc, Zv, i, k, d, u, false);
-        __syncwarp();
-        for (long long e = Gp[r] + lane; e < Gp[r + 1]; e += 32) {
-            const int c = __ldg(Gc + e);
-            if ((unsigned)c < (unsigned)d) u[c] += lr * __ldg(Gv + e);  // G's columns are distinct
-            else atomicOr(err, ERR_C_ROW);
-        }
-        __syncwarp();
-        if (U_out)
-            for (int c = lane; c < d; c += 32) U_out[r * d + c] = u[c];
-        // T = the k-th largest magnitude key (bits of |u|; monotone in |u|)
-        unsigned T = 0u;
-        for (int bit = 31; bit >= 0; --bit) {
-            const unsigned cand = T | (1u << bit);
-            int cnt = 0;
-            for (int m = 0; m < mb; ++m) {
-                const int c = 32 * m + lane;
-                cnt += (c < d && (__float_as_uint(u[c]) & 0x7FFFFFFFu) >= cand) ? 1 : 0;
+// Up to KL entries per lane of row j of Z (column -1: none, as for j < 0 and
+// for a column outside [0, d), which is reported through `bad`).
+template <int KL>
+struct ZRow {
+    int c[KL];
+    float v[KL];
+    __device__ __forceinline__ void load(const F2vParams& p, int j) {
+#pragma unroll
+        for (int q = 0; q < KL; ++q) {
+            const int t = lane_id() + 32 * q;
+            c[q] = -1;
+            v[q] = 0.0f;
+            if (j >= 0 && t < p.k) {
+                c[q] = __ldg(p.Zc + (long long)j * p.k + t);
+                v[q] = __ldg(p.Zv + (long long)j * p.k + t);
             }
-            if (warp_sum(cnt) >= k) T = cand;
         }
-        int gt = 0;
-        for (int m = 0; m < mb; ++m) {
-            const int c = 32 * m + lane;
-            gt += (c < d && (__float_as_uint(u[c]) & 0x7FFFFFFFu) > T) ? 1 : 0;
+    }
+    __device__ __forceinline__ float dot(const F2vParams& p, const float* z, bool held, bool& bad) {
+        float x = 0.0f;
+#pragma unroll
+        for (int q = 0; q < KL; ++q) {
+            if ((unsigned)c[q] < (unsigned)p.d) {
+                x = fmaf(z[c[q]], v[q], x);
+            } else {
+                bad |= held && lane_id() + 32 * q < p.k;
+                c[q] = -1;
+            }
         }
-        const int need = k - warp_sum(gt);  // keys equal to T to keep, smallest columns first
-        int eq_before = 0, out = 0;
-        for (int m = 0; m < mb; ++m) {
-            const int c = 32 * m + lane;
-            const float v = c < d ? u[c] : 0.0f;
-            const unsigned key = __float_as_uint(v) & 0x7FFFFFFFu;
-            const bool valid = c < d;
-            const bool eq = valid && key == T;
-            const unsigned beq = __ballot_sync(FULL, eq);
-            const bool keep = (valid && key > T) || (eq && eq_before + __popc(beq & lt) < need);
-            const unsigned bk = __ballot_sync(FULL, keep);
-            if (keep) {
-                const int pos = out + __popc(bk & lt);
-                if (pos < k) {
-                    Sc[r * k + pos] = c;
-                    Sv[r * k + pos] = v;
+        return x;
+    }
+    __device__ __forceinline__ void add(float w, float* g) const {
+#pragma unroll
+        for (int q = 0; q < KL; ++q)
+            if (c[q] >= 0) g[c[q]] += w * v[q];
+    }
+};
+
+__device__ __forceinline__ float f2v_weight(float x, bool sample) {
+    const float sg = 1.0f / (1.0f + expf(-x));
+    return sample ? -sg : 1.0f - sg;
+}
+
+// Terms [t0, t1) of batch row r: term t < len is neighbour t of the vertex,
+// the others its samples.  KL entries of a row of Z per lane (KL = 0: more
+// than 64 entries a row, read twice).
+template <int KL>
+__device__ __forceinline__ void f2v_terms(const F2vParams& p, long long r, long long a0, long long len, long long t0,
+                                          long long t1, const float* z, float* g) {
+    constexpr int U = KL == 2 ? F2V_FLIGHT / 2 : F2V_FLIGHT;  // terms in flight
+    const int lane = lane_id();
+    bool bad_a = false, bad_z = false;
+    for (long long tb = t0; tb < t1; tb += 32) {
+        const long long t = tb + lane;
+        const int m = (int)(t1 - tb < 32 ? t1 - tb : 32);
+        int j = -1;
+        if (lane < m) {
+            j = t < len ? __ldg(p.Ai + a0 + t) : __ldg(p.neg + r * p.s + (t - len));
+            if ((unsigned)j >= (unsigned)p.n) {
+                bad_a = true;
+                j = -1;
+            }
+        }
+        const unsigned sample = __ballot_sync(FULL, t >= len);
+        if constexpr (KL > 0) {
+            ZRow<KL> cur[U], nxt[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) cur[u].load(p, __shfl_sync(FULL, j, u));
+            for (int q = 0; q < m; q += U) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int jn = __shfl_sync(FULL, j, (q + U + u) & 31);
+                    nxt[u].load(p, q + U + u < m ? jn : -1);
+                }
+                float w[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    w[u] = cur[u].dot(p, z, __shfl_sync(FULL, j, (q + u) & 31) >= 0 && q + u < m, bad_z);
+#pragma unroll
+                for (int u = 0; u < U; ++u) w[u] = f2v_weight(warp_sum(w[u]), (sample >> ((q + u) & 31)) & 1u);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    cur[u].add(w[u], g);  // a term past the end holds no entries
+                    __syncwarp();         // the next row's columns may be this one's
+                    cur[u] = nxt[u];
                 }
             }
-            eq_before += __popc(beq);
-            out += __popc(bk);
+        } else {
+            for (int q = 0; q < m; ++q) {
+                const int jq = __shfl_sync(FULL, j, q);
+                if (jq < 0) continue;
+                const int* zc = p.Zc + (long long)jq * p.k;
+                const float* zv = p.Zv + (long long)jq * p.k;
+                float x = 0.0f;
+                for (int e = lane; e < p.k; e += 32) {
+                    const int c = __ldg(zc + e);
+                    if ((unsigned)c < (unsigned)p.d) x = fmaf(z[c], __ldg(zv + e), x);
+                    else bad_z = true;
+                }
+                const float w = f2v_weight(warp_sum(x), (sample >> q) & 1u);
+                for (int e = lane; e < p.k; e += 32) {
+                    const int c = __ldg(zc + e);
+                    if ((unsigned)c < (unsigned)p.d) g[c] += w * __ldg(zv + e);
+                }
+                __syncwarp();
+            }
+        }
+    }
+    if (bad_a) atomicOr(&p.ws.ctl->err, ERR_A_COL);
+    if (bad_z) atomicOr(&p.ws.ctl->err, ERR_B_COL);
+}
+
+// Row r from z (its old row) and its sum g: u = z + lr * g in place of z, the
+// optional dense copy, then the k entries of largest magnitude to the staging
+// rows.  Columns c, c + 32, ... belong to lane c % 32.
+__device__ __forceinline__ void f2v_finish(const F2vParams& p, long long r, float* u, const float* g) {
+    const int lane = lane_id(), mb = p.dpad >> 5;
+    const unsigned lt = lanemask_lt();
+    for (int c = lane; c < p.d; c += 32) {
+        const float s = g[c];
+        if (__float_as_uint(s) != F2V_EMPTY) u[c] += p.lr * s;
+        if (p.U_out) p.U_out[r * p.d + c] = u[c];
+    }
+    __syncwarp();
+    auto key_of = [&](int m) {  // 0 past the row's end: never above a candidate
+        const int c = 32 * m + lane;
+        return c < p.d ? __float_as_uint(u[c]) & 0x7FFFFFFFu : 0u;
+    };
+    // T = the k-th largest magnitude key (bits of |u|; monotone in |u|)
+    unsigned T = 0u;
+    for (int bit = 30; bit >= 0; --bit) {
+        const unsigned cand = T | (1u << bit);
+        int cnt = 0;
+        for (int m = 0; m < mb; ++m) cnt += __popc(__ballot_sync(FULL, key_of(m) >= cand));
+        if (cnt >= p.k) T = cand;
+    }
+    int gt = 0;
+    for (int m = 0; m < mb; ++m) gt += __popc(__ballot_sync(FULL, key_of(m) > T));
+    const int need = p.k - gt;  // keys equal to T to keep, smallest columns first
+    int eq_before = 0, out = 0;
+    for (int m = 0; m < mb; ++m) {
+        const int c = 32 * m + lane;
+        const unsigned key = key_of(m);
+        const bool valid = c < p.d;
+        const bool eq = valid && key == T;
+        const unsigned beq = __ballot_sync(FULL, eq);
+        const bool keep = (valid && key > T) || (eq && eq_before + __popc(beq & lt) < need);
+        const unsigned bk = __ballot_sync(FULL, keep);
+        if (keep) {
+            const int pos = out + __popc(bk & lt);
+            if (pos < p.k) {
+                p.ws.Sc[r * p.k + pos] = c;
+                p.ws.Sv[r * p.k + pos] = u[c];
+            }
+        }
+        eq_before += __popc(beq);
+        out += __popc(bk);
+    }
+    __syncwarp();
+}
+
+// LONG = false: a warp per batch row; rows of more than F2V_CHUNK terms are
+// queued.  LONG = true: a warp per queued chunk.  Shared memory: z and g, dpad
+// floats each, per warp.  The check that Z holds exactly k entries per row
+// (Zp[i] = k * i) is spread over the first kernel's threads.
+template <int KL, bool LONG>
+__global__ void __launch_bounds__(256) k_f2v_rows(F2vParams p) {
+    extern __shared__ __align__(16) float fsm[];
+    const int nw = blockDim.x >> 5, warp = warp_id(), lane = lane_id();
+    float* z = fsm + (size_t)warp * 2 * p.dpad;
+    float* g = z + p.dpad;
+    const long long gw = (long long)blockIdx.x * nw + warp, gws = (long long)gridDim.x * nw;
+    F2vCtl* ctl = p.ws.ctl;
+    if (!LONG) {
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i <= p.n;
+             i += (long long)gridDim.x * blockDim.x)
+            if (__ldg(p.Zp + i) != (long long)p.k * i) atomicOr(&ctl->err, ERR_CAPACITY);
+    }
+    const long long units = LONG ? min((long long)__ldcg(&ctl->items), p.item_cap) : p.b;
+    for (long long x = gw; x < units; x += gws) {
+        const long long r = LONG ? p.ws.items[x] >> 24 : x;
+        const long long i = p.r0 + r;
+        const long long a0 = clampll(__ldg(p.Ap + i), 0, p.nnzA), a1 = clampll(__ldg(p.Ap + i + 1), a0, p.nnzA);
+        const long long len = a1 - a0, terms = len + p.s;
+        const int nch = (int)((terms + F2V_CHUNK - 1) / F2V_CHUNK);
+        if (!LONG && nch > 1) {  // queued; its sum starts empty
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(&ctl->items, (unsigned long long)nch);
+            at = __shfl_sync(FULL, at, 0);
+            for (int c = lane; c < nch; c += 32) {
+                if ((long long)at + c < p.item_cap) p.ws.items[at + c] = (r << 24) | c;
+                else atomicOr(&ctl->err, ERR_CAPACITY);
+            }
+            for (int c = lane; c < p.d; c += 32) p.ws.G[r * p.d + c] = __uint_as_float(F2V_EMPTY);
+            if (lane == 0) p.ws.done[r] = 0;
+            continue;
+        }
+        for (int c = lane; c < p.dpad; c += 32) {
+            z[c] = 0.0f;
+            g[c] = __uint_as_float(F2V_EMPTY);
         }
         __syncwarp();
-        for (int c = lane; c < dpad; c += 32) u[c] = 0.0f;
+        f2v_scatter(p, i, z);
         __syncwarp();
+        const long long t0 = LONG ? (p.ws.items[x] & 0xFFFFFF) * (long long)F2V_CHUNK : 0;
+        f2v_terms<KL>(p, r, a0, len, t0, t0 + F2V_CHUNK < terms ? t0 + F2V_CHUNK : terms, z, g);
+        __syncwarp();
+        if (LONG) {
+            float* G = p.ws.G + r * p.d;
+            for (int c = lane; c < p.d; c += 32)
+                if (__float_as_uint(g[c]) != F2V_EMPTY) atomicAdd(G + c, g[c]);
+            __threadfence();
+            __syncwarp();
+            int before = 0;
+            if (lane == 0) before = atomicAdd(p.ws.done + r, 1);
+            if (__shfl_sync(FULL, before, 0) != nch - 1) continue;
+            __threadfence();
+            for (int c = lane; c < p.d; c += 32) g[c] = __ldcg(G + c);
+            __syncwarp();
+        }
+        f2v_finish(p, r, z, g);
     }
 }
 
@@ -267,78 +336,63 @@ __global__ void __launch_bounds__(256) k_f2v_commit(long long r0, long long b, i
     }
 }
 
-static unsigned f2v_blocks_exact(long long m) { return (unsigned)((m + 255) / 256 > 0 ? (m + 255) / 256 : 1); }
-
-static unsigned f2v_blocks(long long m) {
-    long long g = (m + 255) / 256;
-    if (g < 1) g = 1;
-    if (g > 152 * 16) g = 152 * 16;
-    return (unsigned)g;
-}
-
-cudaError_t launch_f2v_pattern(const DevCsr& A, long long r0, long long b, const int* neg, int s, long long* Wp,
-                               unsigned* newmask, long long* partial, WsHeader* hdr, cudaStream_t st) {
+template <int KL>
+static cudaError_t launch_rows(const F2vParams& p, int sms, cudaStream_t st) {
+    const void* rows = (const void*)k_f2v_rows<KL, false>;
+    const void* chunks = (const void*)k_f2v_rows<KL, true>;
+    const size_t per_warp = 2 * sizeof(float) * (size_t)p.dpad;  // at most 32 KB
+    int warps = 8;
+    while (warps > 1 && warps * per_warp > 100 * 1024) warps /= 2;
+    const size_t smem = warps * per_warp;
     cudaError_t e;
-    if (s < 0 || s > F2V_MAX_NEG) return cudaErrorInvalidValue;
-    if ((e = cudaMemsetAsync(Wp, 0, sizeof(long long), st))) return e;
-    if (b == 0) return cudaSuccess;
-    if ((e = cudaMemsetAsync(newmask, 0, sizeof(unsigned) * (size_t)b, st))) return e;
-    if (s > 0) {
-        count_launch();
-        k_f2v_newmask<<<f2v_blocks_exact(b * s), 256, 0, st>>>(A.rowptr, A.col, A.nnz, (int)A.nrows, r0, b, neg, s,
-                                                               newmask, &hdr->err);
-    }
+    for (const void* k : {rows, chunks})
+        if (smem > 48 * 1024 && (e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+            return e;
+    F2vParams q = p;
+    void* args[] = {&q};
+    const long long need = (p.b + warps - 1) / warps;
+    const int full = persistent_grid(rows, 32 * warps, smem, sms);
     count_launch();
-    k_f2v_rowlen<<<f2v_blocks_exact(b), 256, 0, st>>>(A.rowptr, A.nnz, r0, b, newmask, Wp + 1);
-    if ((e = cudaGetLastError())) return e;
-    return launch_scan_inplace(Wp + 1, b, partial, st);
-}
-
-cudaError_t launch_f2v_fill(const DevCsr& A, long long r0, long long b, const int* neg, int s, const long long* Wp,
-                            const unsigned* newmask, int* Wcol, int* Wmult, int* Wrow, cudaStream_t st) {
-    if (b == 0) return cudaSuccess;
-    count_launch();
-    k_f2v_fill_a<<<152 * 8, 256, 0, st>>>(A.rowptr, A.col, A.nnz, r0, b, neg, s, newmask, Wp, Wcol, Wmult, Wrow);
-    if (s > 0) {
-        count_launch();
-        k_f2v_fill_n<<<f2v_blocks_exact(b * s), 256, 0, st>>>(A.rowptr, A.col, A.nnz, r0, b, neg, s, newmask, Wp,
-                                                              Wcol, Wmult, Wrow);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_f2v_check(const DevCsr& Z, int k, WsHeader* hdr, cudaStream_t st) {
-    count_launch();
-    k_f2v_check_rows<<<(unsigned)((Z.nrows + 1 + 255) / 256), 256, 0, st>>>(Z.rowptr, Z.nrows, k, &hdr->err);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_f2v_weights(const DevCsr& Z, int k, long long r0, long long b, const long long* Wp,
-                               const int* Wcol, const int* Wmult, const int* Wrow, float* Wval, cudaStream_t st) {
-    if (b == 0) return cudaSuccess;
-    count_launch();
-    k_f2v_weights<<<152 * 16, 256, 0, st>>>(Z.col, Z.val, Z.nrows, k, r0, Wp, b, Wcol, Wmult, Wrow, Wval);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_f2v_update(const DevCsr& Z, int k, long long r0, long long b, const long long* Gp, const int* Gc,
-                              const float* Gv, float lr, float* U_out, int* Sc, float* Sv, int sms, WsHeader* hdr,
-                              cudaStream_t st) {
-    if (b == 0) return cudaSuccess;
-    const int d = (int)Z.ncols, dpad = (d + 31) & ~31;
-    const size_t smem = sizeof(float) * (size_t)dpad * 8;
-    cudaError_t e;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute((const void*)k_f2v_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)))
+    if ((e = cudaLaunchKernel(rows, dim3((unsigned)(need < full ? need : full)), dim3(32 * warps), args, smem, st)))
         return e;
-    const int grid = persistent_grid((const void*)k_f2v_update, 256, smem, sms);
     count_launch();
-    k_f2v_update<<<grid, 256, smem, st>>>(Z.col, Z.val, d, k, r0, b, Gp, Gc, Gv, lr, U_out, Sc, Sv, &hdr->err);
-    if ((e = cudaGetLastError())) return e;
+    const long long most = (p.item_cap + warps - 1) / warps;
+    const int cgrid = persistent_grid(chunks, 32 * warps, smem, sms);
+    return cudaLaunchKernel(chunks, dim3((unsigned)(most < cgrid ? most : cgrid)), dim3(32 * warps), args, smem, st);
+}
+
+cudaError_t launch_f2v_step(const DevCsr& A, const DevCsr& Z, int k, long long r0, long long b, const int* neg, int s,
+                            float lr, float* U_out, int sms, void* ws, cudaStream_t st) {
+    cudaError_t e;
+    F2vParams p = {};
+    p.Ap = A.rowptr;
+    p.Ai = A.col;
+    p.nnzA = A.nnz;
+    p.n = (int)A.nrows;
+    p.r0 = r0;
+    p.b = b;
+    p.neg = neg;
+    p.s = s;
+    p.Zp = Z.rowptr;
+    p.Zc = Z.col;
+    p.Zv = Z.val;
+    p.k = k;
+    p.d = (int)Z.ncols;
+    p.dpad = (p.d + 31) & ~31;
+    p.lr = lr;
+    p.U_out = U_out;
+    f2v_ws((char*)ws, p.d, A.nnz, b, s, k, &p.ws);
+    p.item_cap = f2v_item_capacity(A.nnz + b * s);
+    if ((e = cudaMemsetAsync(p.ws.ctl, 0, sizeof(F2vCtl), st))) return e;
+    if (k <= 32) e = launch_rows<1>(p, sms, st);
+    else if (k <= 64) e = launch_rows<2>(p, sms, st);
+    else e = launch_rows<0>(p, sms, st);
+    if (e) return e;
+    long long blocks = (b * k + 255) / 256;
+    if (blocks > 152 * 16) blocks = 152 * 16;
     count_launch();
-    k_f2v_commit<<<f2v_blocks(b * k), 256, 0, st>>>(r0, b, k, Sc, Sv, const_cast<int*>(Z.col),
-                                                     const_cast<float*>(Z.val));
+    k_f2v_commit<<<(unsigned)blocks, 256, 0, st>>>(r0, b, k, p.ws.Sc, p.ws.Sv, const_cast<int*>(Z.col),
+                                                   const_cast<float*>(Z.val));
     return cudaGetLastError();
 }
 

@@ -243,19 +243,16 @@ cudaError_t launch_bat_backward(const InstDesc* inst, int count, long long g0, l
 cudaError_t launch_batch_bounds(const InstDesc* inst, int count, const long long* flops, long long* bound,
                                 cudaStream_t st);
 
-// Sparse Force2Vec step (force2vec.cu): W's pattern (count + scan, fill),
-// the Z layout check, the weights on W's pattern, and update + top-k +
-// commit into Z's batch rows.
-cudaError_t launch_f2v_pattern(const DevCsr& A, long long r0, long long b, const int* neg, int s, long long* Wp,
-                               unsigned* newmask, long long* partial, WsHeader* hdr, cudaStream_t st);
-cudaError_t launch_f2v_fill(const DevCsr& A, long long r0, long long b, const int* neg, int s, const long long* Wp,
-                            const unsigned* newmask, int* Wcol, int* Wmult, int* Wrow, cudaStream_t st);
-cudaError_t launch_f2v_check(const DevCsr& Z, int k, WsHeader* hdr, cudaStream_t st);
-cudaError_t launch_f2v_weights(const DevCsr& Z, int k, long long r0, long long b, const long long* Wp,
-                               const int* Wcol, const int* Wmult, const int* Wrow, float* Wval, cudaStream_t st);
-cudaError_t launch_f2v_update(const DevCsr& Z, int k, long long r0, long long b, const long long* Gp, const int* Gc,
-                              const float* Gv, float lr, float* U_out, int* Sc, float* Sv, int sms, WsHeader* hdr,
-                              cudaStream_t st);
+// Sparse Force2Vec step (force2vec.cu): the new rows computed, then written
+// into Z's batch rows.  ws: f2v_bytes, 256-byte aligned, beginning with an
+// F2vCtl that the step clears.
+struct F2vCtl {
+    unsigned long long err;    // ERR_* bits
+    unsigned long long items;  // chunks of long rows queued
+};
+size_t f2v_bytes(long long d, long long nnzA, long long b, long long s, long long k);
+cudaError_t launch_f2v_step(const DevCsr& A, const DevCsr& Z, int k, long long r0, long long b, const int* neg, int s,
+                            float lr, float* U_out, int sms, void* ws, cudaStream_t st);
 
 // CSR validation; writes the first bad row (or -1) into *bad (device).
 cudaError_t launch_validate(const DevCsr& M, long long* bad, cudaStream_t st);

@@ -123,3 +123,32 @@ def test_f2v_argument_errors():
     bad = DeviceCSR(Zd.nrows, Zd.ncols, Zd.rowptr, Zd.col[:-1], Zd.val[:-1])  # not k per row
     with pytest.raises(TSError):
         Force2Vec(Ad, bad, 8, negatives=2, batch=16).step(0, torch.zeros(32, dtype=torch.int32))
+
+
+@pytest.mark.parametrize("d,k", [(1, 1), (40, 33), (128, 64), (200, 65), (700, 200), (4096, 30)])
+def test_f2v_row_widths_and_long_rows(d, k):
+    # rows of Z of one, two and more entries per lane; a hub of several chunks
+    # of terms (128 each) beside rows of one chunk exactly and one term more
+    n, s, b, r0 = 700, 4, 60, 13
+    rng = np.random.default_rng(d + k)
+    lens = rng.integers(0, 9, n)
+    lens[r0:r0 + 8] = [0, 124, 125, 123, 252, 253, n, 300]
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(lens, out=rowptr[1:])
+    A = CSR(n, n, rowptr, np.concatenate([np.sort(rng.choice(n, m, replace=False)) for m in lens]).astype(np.int32))
+    Z = synth.sparse_embedding(n, d, k, 120 + d, scale=0.3)
+    _check_step(A, Z, r0, b, s, 0.2, k, synth.negatives(b, s, n, 121))
+
+
+@pytest.mark.parametrize("k", [20, 40, 70])
+def test_f2v_bad_columns_are_reported(k):
+    A = synth.rmat(8, 8, 130, symmetrize=True)
+    Z = synth.sparse_embedding(A.nrows, 96, k, 131)
+    neg = synth.negatives(A.nrows, 3, A.nrows, 132)
+    for what in ("A", "Z", "neg"):
+        a, z, m = A.col.copy(), Z.col.copy(), neg.copy()
+        {"A": a, "Z": z, "neg": m}[what][-1] = 1 << 20
+        Ad = DeviceCSR.from_host(CSR(A.nrows, A.ncols, A.rowptr, a), with_values=False)
+        Zd = DeviceCSR.from_host(CSR(Z.nrows, Z.ncols, Z.rowptr, z, Z.val))
+        with pytest.raises(TSError):
+            Force2Vec(Ad, Zd, k, negatives=3, batch=A.nrows).step(0, torch.as_tensor(m))
