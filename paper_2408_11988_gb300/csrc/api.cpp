@@ -567,6 +567,11 @@ static ts_status run_numeric(ts_plan* plan, const ts_csr_desc* A, const ts_csr_d
                                          (const long long*)C->rowptr, C->col, (float*)C->val, C->nnz, st, bq),
                     fn);
         }
+    } else if (plan->force.accum != TS_ACC_HASH && numeric_rank_fits(plan->d)) {
+        // the hash accumulator chosen, not asked for: ranked columns where they fit
+        TS_CUDA(launch_numeric_rank(dA, dB, plan->d, vals, sc, cfg, (const long long*)C->rowptr, C->col,
+                                    (float*)C->val, C->nnz, st),
+                fn);
     } else {
         TS_CUDA(launch_numeric_hash(dA, dB, plan->d, plan->cur.hash_slots, vals, sc, cfg,
                                     (const long long*)C->rowptr, C->col, (float*)C->val, C->nnz, st),

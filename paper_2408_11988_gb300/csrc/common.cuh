@@ -350,7 +350,7 @@ __device__ __forceinline__ void pipelined_rows(const int* __restrict__ perm, lon
 // order leaves in the header: every block of every pass reads these, and
 // summing the 385 counters there took each of them 2 - 3 us).
 __device__ __forceinline__ long long rows_from_class(const WsHeader* hdr, int c) {
-    return c < NUM_CLASSES ? __ldg(hdr->above + (c > 1 ? c : 1) - 1) : 0;
+    return c < NUM_CLASSES ? __ldg(hdr->hist + (c > 1 ? c : 1) - 1) : 0;
 }
 
 // Rows with products: all classes >= 1; heavy: classes >= cta_class.

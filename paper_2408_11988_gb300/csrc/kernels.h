@@ -127,6 +127,12 @@ cudaError_t launch_numeric_hash(const DevCsr& A, const DevCsr& B, long long d, i
                                 bool values, const Sched& s, const LaunchCfg& cfg,
                                 const long long* Cp, int* Ci, float* Cx, long long nnzC,
                                 cudaStream_t st);
+// Numeric pass by ranked columns (numeric_rank.cu), 4096 < d <= RANK_MAX_D.
+constexpr long long RANK_MAX_D = 32768;
+bool numeric_rank_fits(long long d);
+cudaError_t launch_numeric_rank(const DevCsr& A, const DevCsr& B, long long d, bool values, const Sched& s,
+                                const LaunchCfg& cfg, const long long* Cp, int* Ci, float* Cx, long long nnzC,
+                                cudaStream_t st);
 size_t numeric_dense_smem(int W, int warps, bool values);
 // Light rows only, in row groups of cfg.row_lanes lanes (4, 8 or 16; packed
 // B), launched with programmatic dependent launch behind a numeric kernel

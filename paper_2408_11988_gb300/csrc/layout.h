@@ -47,10 +47,9 @@ struct WsHeader {
     unsigned long long item_ctr;      // next split-row work item
     unsigned long long err;           // ERR_* bits
     long long total;                  // multi-source BFS: entries of the next frontier (read with err)
-    long long hist[NUM_CLASSES];      // rows per flops class
+    long long hist[NUM_CLASSES];      // rows per flops class; once the row order is written, rows in the classes above each
     long long cursor[NUM_CLASSES];    // scatter cursors per class
-    long long above[NUM_CLASSES];     // rows in the classes above each (written with the row order)
-    long long scratch[8];             // [0] flops items, [1] split rows, [2] split items
+    long long scratch[8];             // [0] flops items, [1] split rows, [2] split items, [3] blocks of the row order done
 };
 
 }  // namespace ts

@@ -47,10 +47,11 @@ __global__ void __launch_bounds__(256) k_flops_rows(long long n, const long long
                                                     const int* __restrict__ Ai, long long nnzA,
                                                     Seg segB, int nB, long long* __restrict__ flops,
                                                     long long* __restrict__ items, long long item_cap,
-                                                    WsHeader* hdr) {
+                                                    WsHeader* hdr, int rows) {
     __shared__ long long s_f[256];
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = lane_id();
+    // rows per warp: 32, or fewer where there are too few for every warp
+    const long long i = lane < rows ? ((long long)blockIdx.x * 8 + warp_id()) * rows + lane : n;
     unsigned long long* err = &hdr->err;
     long long nchunks = 0;
     long long a0 = 0;
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(256) k_flops_rows(long long n, const long long
     long long* wf = s_f + (threadIdx.x & ~31);
     wf[lane] = 0;
     __syncwarp();
-    // The short rows of the warp's 32 rows hold consecutive entries of A: they
+    // The short rows of the warp's rows hold consecutive entries of A: they
     // are numbered across the rows and read 32 at a time (coalesced); each
     // entry's B row length goes to its row by a segmented sum over the lanes
     // (the row of entry p is the last lane whose first number is <= p).
@@ -242,11 +243,23 @@ __global__ void __launch_bounds__(256) k_scatter(long long n, long long* flops, 
     }
     const long long base = (long long)blockIdx.x * blockDim.x * SCATTER_ROWS;
     int cls[SCATTER_ROWS];
-    unsigned rank[SCATTER_ROWS];
+    unsigned rank[SCATTER_ROWS], cut = 0;  // cut: bit u, row u has many entries
+    {
+        // every load of the block's rows before any is used
+        long long f[SCATTER_ROWS], a0[SCATTER_ROWS], a1[SCATTER_ROWS];
 #pragma unroll
-    for (int u = 0; u < SCATTER_ROWS; ++u) {
-        const long long i = base + (long long)u * blockDim.x + tid;
-        cls[u] = i < n ? flops_class(flops[i]) : 0;
+        for (int u = 0; u < SCATTER_ROWS; ++u) {
+            const long long i = base + (long long)u * blockDim.x + tid;
+            f[u] = i < n ? flops[i] : 0;
+            a0[u] = Ap && i < n ? __ldg(Ap + i) : 0;
+            a1[u] = Ap && i < n ? __ldg(Ap + i + 1) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < SCATTER_ROWS; ++u) {
+            cls[u] = flops_class(f[u]);
+            const long long s0 = clampll(a0[u], 0, nnzA);
+            if (clampll(a1[u], s0, nnzA) - s0 > SPLIT_ENTRIES) cut |= 1u << u;
+        }
     }
     __syncthreads();
     if (tid < 32) {  // start of class c = rows of the classes above it
@@ -266,8 +279,6 @@ __global__ void __launch_bounds__(256) k_scatter(long long n, long long* flops, 
     for (int u = 0; u < SCATTER_ROWS; ++u)
         if (cls[u] > 0) rank[u] = atomicAdd(&s_cnt[cls[u]], 1u);
     __syncthreads();
-    if (blockIdx.x == 0)
-        for (int c = tid; c < NUM_CLASSES; c += blockDim.x) hdr->above[c] = s_start[c];
     for (int c = tid; c < NUM_CLASSES; c += blockDim.x)
         s_base[c] = (c > 0 && s_cnt[c])
                         ? (long long)atomicAdd((unsigned long long*)&hdr->cursor[c], (unsigned long long)s_cnt[c])
@@ -278,11 +289,21 @@ __global__ void __launch_bounds__(256) k_scatter(long long n, long long* flops, 
         const long long i = base + (long long)u * blockDim.x + tid;
         if (i >= n || cls[u] == 0) continue;
         perm[s_start[cls[u]] + s_base[cls[u]] + rank[u]] = (int)i;
-        if (Ap) {
+        if ((cut >> u) & 1u) {
             const long long a0 = clampll(__ldg(Ap + i), 0, nnzA), a1 = clampll(__ldg(Ap + i + 1), a0, nnzA);
-            if (a1 - a0 > SPLIT_ENTRIES) split_row(i, a1 - a0, flops, s, item_cap);
+            split_row(i, a1 - a0, flops, s, item_cap);
         }
     }
+    // every block has read the histogram when the last one gets here: the
+    // running sums take its place for the passes
+    __shared__ int s_last;
+    if (tid == 0) {
+        __threadfence();
+        s_last = atomicAdd((unsigned long long*)&hdr->scratch[3], 1ull) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last)
+        for (int c = tid; c < NUM_CLASSES; c += blockDim.x) hdr->hist[c] = s_start[c];
 }
 
 // B's row lengths as an array of their own pay from this many rows of B on
@@ -296,13 +317,15 @@ cudaError_t launch_row_flops(const DevCsr& A, const DevCsr& B, const Sched& s, c
     if (n == 0) return cudaSuccess;
     const SegWhole segB{B.rowptr, B.nnz, (int)B.ncols};
     const long long cap = flops_item_capacity(n, A.nnz);
-    const unsigned rb = (unsigned)((n + 255) / 256);
+    const int rows = tiny_chunk_rows(n, 152 * 48);
+    const unsigned rb = (unsigned)((n + 8LL * rows - 1) / (8LL * rows));
     // a warp per chunk of a long row; none can exist in a matrix this small
     const unsigned cb = A.nnz > SHORT_ROW ? (unsigned)(cap < 152 * 64 ? (cap + 7) / 8 : 152 * 8) : 0;
     auto run = [&](auto seg) {
         using Seg = decltype(seg);
         count_launch();
-        k_flops_rows<Seg><<<rb, 256, 0, st>>>(n, A.rowptr, A.col, A.nnz, seg, (int)B.nrows, s.flops, s.items, cap, s.hdr);
+        k_flops_rows<Seg><<<rb, 256, 0, st>>>(n, A.rowptr, A.col, A.nnz, seg, (int)B.nrows, s.flops, s.items, cap, s.hdr,
+                                               rows);
         if (!cb) return;
         count_launch();
         k_flops_chunks<Seg><<<cb, 256, 0, st>>>(A.rowptr, A.col, A.nnz, seg, (int)B.nrows, s.flops, s.items, cap, s.hdr);
