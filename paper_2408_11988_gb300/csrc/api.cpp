@@ -632,7 +632,9 @@ static ts_status run_backward(ts_plan* plan, const ts_csr_desc* A, const ts_csr_
             fn);
     if (det)
         TS_CUDA(launch_backward_t(dev(A), dev(B), plan->d, (const long long*)C->rowptr, C->col, C->nnz, dC, dB,
-                                  (char*)ws + L.bt, sc.hdr, (cudaStream_t)stream),
+                                  (char*)ws + L.bt, L.bq ? (char*)ws + L.bq : nullptr,
+                                  L.bq ? padded_b_bytes(plan->n, B->nnz, plan->d, 4) : 0, sc.hdr,
+                                  (cudaStream_t)stream),
                 fn);
     return ok();
 }

@@ -49,7 +49,8 @@ struct WsHeader {
     long long total;                  // multi-source BFS: entries of the next frontier (read with err)
     long long hist[NUM_CLASSES];      // rows per flops class; once the row order is written, rows in the classes above each
     long long cursor[NUM_CLASSES];    // scatter cursors per class
-    long long scratch[8];             // [0] flops items, [1] split rows, [2] split items, [3] blocks of the row order done
+    long long scratch[8];             // [0] flops items, [1] split rows, [2] split items, [3] blocks of the row order done,
+                                      // [4], [5] the repeatable dB's queue
 };
 
 }  // namespace ts

@@ -6,6 +6,7 @@
 // it (the pull form below); above that the list form walks F's rows, heaviest
 // rows first, and skips rows whose visited set is full and rows whose
 // neighbours have empty frontier rows.
+#include "bitrows.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -291,13 +292,7 @@ __device__ __forceinline__ void check_columns(unsigned block, long long n, const
 
 // Bitmap rows of F and the bits of the non-empty ones; also clears what the
 // level accumulates (scan partials) and C's first row pointer.  A warp takes
-// 32 vertices, whose entries follow each other in F: 128 entries a step, four
-// per lane with one 16-byte load, the row of a lane's first entry by a search
-// of the warp's row starts in shared memory, and the bits of neighbouring
-// entries of one word gathered before one OR into the warp's words in shared
-// memory.  (A thread per row took 127 us for a frontier of 57 million entries
-// over 2^20 vertices, its lines thrown out of L1 before they were used up;
-// this way 106 us, the check of A's 31 million columns included.)
+// 32 vertices (rows_to_bits).
 //
 // The blocks behind the first nfront range-check A's columns, so that the
 // pull may leave out rows and ends of rows with nothing left to find: a
@@ -321,60 +316,8 @@ __global__ void __launch_bounds__(256) k_bfs_frontier(long long n, int d, const 
     for (long long x = (long long)blockIdx.x * 256 + threadIdx.x; x < npartial; x += 256LL * nfront) partial[x] = 0;
     if (v == 0) rp_next[0] = 0;
     unsigned* bits = s_bits[warp];
-    int* start = s_start[warp];
-#pragma unroll
-    for (int m = 0; m < DWP; ++m) bits[32 * m + lane] = 0u;
     if (base >= n) return;
-    const long long s = clampll(__ldg(Fp + (v < n ? v : n)), 0, nnzF);
-    const long long e0 = shfl64(s, 0);
-    const long long e1 = clampll(__ldg(Fp + (base + 32 < n ? base + 32 : n)), e0, nnzF);
-    const int total = (int)(e1 - e0 < (1LL << 30) ? e1 - e0 : 1LL << 30);  // at most 32 d in a well-formed F
-    start[lane] = (int)clampll(s - e0, 0, total);
-    if (lane == 0) start[32] = total;
-    __syncwarp();
-    const int* f = Fi + e0;
-    const int lead = (int)((reinterpret_cast<uintptr_t>(f) >> 2) & 3);  // entries of the first 16 bytes before f
-    bool bad = false;
-    for (int i0 = -lead; i0 < total; i0 += 128) {
-        const int i = i0 + 4 * lane;
-        if (i >= total) continue;
-        int c[4];
-        if (i >= 0 && i + 4 <= total) {
-            const int4 x = __ldg(reinterpret_cast<const int4*>(f + i));
-            c[0] = x.x;
-            c[1] = x.y;
-            c[2] = x.z;
-            c[3] = x.w;
-        } else {
-#pragma unroll
-            for (int t = 0; t < 4; ++t) c[t] = i + t >= 0 && i + t < total ? __ldg(f + i + t) : 0;
-        }
-        int r = 0;  // last row starting at or before the lane's first entry
-        const int at = i > 0 ? i : 0;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1)
-            if (start[r + o] <= at) r += o;
-        int word = -1;
-        unsigned x = 0u;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            if (i + t < 0 || i + t >= total) continue;
-            while (r < 31 && i + t >= start[r + 1]) ++r;
-            if ((unsigned)c[t] >= (unsigned)d) {
-                bad = true;
-                continue;
-            }
-            const int w = r * DWP + (c[t] >> 5);
-            if (w != word) {
-                if (x) atomicOr(bits + word, x);
-                word = w;
-                x = 0u;
-            }
-            x |= 1u << (c[t] & 31);
-        }
-        if (x) atomicOr(bits + word, x);
-    }
-    __syncwarp();
+    const bool bad = rows_to_bits<DWP>(n, d, Fp, nnzF, Fi, base, bits, s_start[warp]);
     unsigned any = 0u;
 #pragma unroll
     for (int m = 0; m < DWP; ++m) any |= bits[lane * DWP + m];
@@ -385,28 +328,6 @@ __global__ void __launch_bounds__(256) k_bfs_frontier(long long n, int d, const 
     for (int m = 0; m < DWP; ++m)
         if (32 * m + lane < (n - base) * DWP) fb[base * DWP + 32 * m + lane] = bits[32 * m + lane];
     if (bad) atomicOr(err, ERR_B_COL);
-}
-
-// Bitmap row of vertex u.
-template <int DWP>
-__device__ __forceinline__ void bfs_row(const unsigned* __restrict__ fb, int u, unsigned w[DWP]) {
-    const unsigned* r = fb + (long long)u * DWP;
-    if constexpr (DWP >= 4) {
-#pragma unroll
-        for (int m = 0; m < DWP; m += 4) {
-            const uint4 x = __ldg(reinterpret_cast<const uint4*>(r + m));
-            w[m] = x.x;
-            w[m + 1] = x.y;
-            w[m + 2] = x.z;
-            w[m + 3] = x.w;
-        }
-    } else if constexpr (DWP == 2) {
-        const uint2 x = __ldg(reinterpret_cast<const uint2*>(r));
-        w[0] = x.x;
-        w[1] = x.y;
-    } else {
-        w[0] = __ldg(r);
-    }
 }
 
 // A row of `words` <= DWP words read or written; VEC: of DWP words, aligned to
@@ -560,7 +481,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1024 / PULL_THREADS)
             for (int t = 0; t < U; ++t) {
 #pragma unroll
                 for (int m = 0; m < DWP; ++m) w[t][m] = 0u;
-                if (cols.hit(u[t])) bfs_row<DWP>(fb, u[t], w[t]);
+                if (cols.hit(u[t])) load_bit_row<DWP>(fb, u[t], w[t]);
             }
 #pragma unroll
             for (int t = 0; t < U; ++t) {
@@ -614,7 +535,7 @@ __global__ void __launch_bounds__(PULL_THREADS, 1024 / PULL_THREADS)
             for (int t = 0; t < U; ++t) {
 #pragma unroll
                 for (int m = 0; m < DWP; ++m) w[t][m] = 0u;
-                if (cols.hit(u[t])) bfs_row<DWP>(fb, u[t], w[t]);
+                if (cols.hit(u[t])) load_bit_row<DWP>(fb, u[t], w[t]);
             }
             unsigned live = 0u;
             if constexpr (PARENTS) {
@@ -751,7 +672,7 @@ __global__ void __launch_bounds__(256) k_bfs_heavy(BfsParams p, const unsigned* 
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 if (cols.hit(u[t])) {
-                    bfs_row<DWP>(fb, u[t], w);
+                    load_bit_row<DWP>(fb, u[t], w);
 #pragma unroll
                     for (int m = 0; m < DWP; ++m) got[m] |= w[m];
                 }
@@ -842,7 +763,7 @@ __global__ void __launch_bounds__(256) k_bfs_heavy_parents(BfsParams p, const un
             unsigned h = 0u;
 #pragma unroll
             for (int m = 0; m < DWP; ++m) w[m] = 0u;
-            if (cols.hit(u)) bfs_row<DWP>(fb, u, w);
+            if (cols.hit(u)) load_bit_row<DWP>(fb, u, w);
 #pragma unroll
             for (int m = 0; m < DWP; ++m) h |= w[m] & rem[m];
             if (__any_sync(FULL, h != 0u)) {
