@@ -1110,7 +1110,8 @@ struct ts_batched_plan {
 };
 
 struct BLayout {
-    size_t inst = 0, bound = 0, ctl = 0, flops = 0, heavy = 0, total = 0;
+    size_t inst = 0, bound = 0, ctl = 0, flops = 0, heavy = 0, items = 0, total = 0;
+    long long item_cap = 0;  // parts of very long rows
     std::vector<size_t> q, dense;  // per instance: packed copy, dense copy (0: none)
 };
 
@@ -1126,9 +1127,11 @@ static BLayout batched_layout(const ts_batched_plan* p) {
     };
     L.inst = take(sizeof(InstDesc) * (size_t)p->count);
     L.bound = take(sizeof(long long) * (size_t)p->count);
-    L.ctl = take(sizeof(BatchCtl));
+    L.ctl = take(sizeof(BatchCtl) + sizeof(unsigned long long) * (size_t)bat_tiles(p->NC, p->count));  // and the scan's sums
     L.flops = take(sizeof(long long) * (size_t)std::max<long long>(p->N, 1));
     L.heavy = take(sizeof(int) * (size_t)std::max<long long>(p->N, 1));
+    for (long long a : p->annz) L.item_cap += bat_long_capacity(a);
+    L.items = take(sizeof(long long) * (size_t)L.item_cap);
     L.q.assign((size_t)p->count, 0);
     L.dense.assign((size_t)p->count, 0);
     for (int b = 0; b < p->count; ++b) {
@@ -1302,11 +1305,13 @@ static ts_status bat_forward(ts_batched_plan* plan, char* w, const BLayout& L, i
     const long long c0 = plan->chunk_off[b0];
     const long long c1 = plan->chunk_off[b0 + nb - 1] + (plan->n[b0 + nb - 1] + 31) / 32;
     const int sms = sm_count();
-    TS_CUDA(cudaMemsetAsync(ctl, 0, sizeof(BatchCtl), st), fn);
-    TS_CUDA(launch_bat_prepare(inst, nb, c0, c1, flops, heavy, ctl, sms, st), fn);
+    unsigned long long* part = (unsigned long long*)(ctl + 1);
+    TS_CUDA(cudaMemsetAsync(ctl, 0, sizeof(BatchCtl) + sizeof *part * (size_t)bat_tiles(plan->NC, plan->count), st), fn);
+    TS_CUDA(launch_bat_prepare(inst, nb, c0, c1, flops, heavy, ctl, (long long*)(w + L.items), L.item_cap, sms, st), fn);
     if (!numeric) return TS_OK;
-    TS_CUDA(launch_bat_symbolic(inst, nb, c0, c1, 0, flops, heavy, ctl, plan->Wmax, sms, st), fn);
-    TS_CUDA(launch_bat_scan(inst, nb, ctl, st), fn);
+    TS_CUDA(launch_bat_symbolic(inst, nb, c0, c1, 0, flops, heavy, ctl, part, plan->Wmax, sms, st), fn);
+    TS_CUDA(launch_bat_scan(inst, nb, *std::max_element(plan->n.begin() + b0, plan->n.begin() + b0 + nb), ctl, part, st),
+            fn);
     TS_CUDA(launch_bat_numeric(inst, nb, c0, c1, bat_vals(plan) ? 1 : 0, flops, heavy, ctl, plan->Wmax, sms, st),
             fn);
     return TS_OK;

@@ -12,15 +12,19 @@
 // occupancy bits, or the dense-B form for a dense enough B_b) and its
 // heavy-row threshold.
 //
-// Forward (four launches): prepare (row flops, the row-aligned packed copy
+// Forward (five launches): prepare (row flops, the row-aligned packed copy
 // of each B_b and, for dense-B instances, the dense copy; rows at or above
-// their instance's threshold go on the heavy list), symbolic (row counts
+// their instance's threshold go on the heavy list), the flops of very long
+// rows, symbolic (row counts
 // into each C_b's row pointers: heavy rows one block each from the list,
-// light rows one warp each in row order), scan (one block per instance),
-// numeric (as the symbolic pass, writing each C_b).  Backward (two
+// light rows by warps in row order), scan (one block per 4096 rows, from the
+// sums that the symbolic pass leaves), numeric (as the symbolic pass, writing
+// each C_b).  Backward (two
 // launches): the gradients are cleared, then dA by rows and dB by float
 // atomics.  Nothing waits on another block: the only coordination is
 // atomic counters over the heavy list.
+#include <climits>
+
 #include "common.cuh"
 #include "denseb.cuh"
 #include "kernels.h"
@@ -72,9 +76,29 @@ __device__ __forceinline__ int inst_of_chunk(const InstDesc* __restrict__ inst, 
     return lo;
 }
 
-// This warp's next 32-row chunk from queue q: chunks are dealt c0, c0 + 1,
+// Units of the passes' queues: a 32-row chunk, or a half, quarter or eighth of
+// one (rows = 16, 8 or 4) where the batch has too few chunks for every warp to
+// take two: a warp takes a unit's rows one group after another.
+struct BatUnits {
+    long long u0, u1;  // units
+    int rows, shift;   // rows of a unit; units of a chunk, as a shift
+    __device__ __forceinline__ long long chunk(long long u) const { return u >> shift; }
+    // first row of unit u in its instance
+    __device__ __forceinline__ long long row0(const InstDesc& I, long long u) const {
+        return (chunk(u) - I.chunk_off) * 32 + (u & ((1 << shift) - 1)) * rows;
+    }
+};
+
+// Sums of C's row counts over 4096 rows of an instance, for the scan: where row
+// i of instance b keeps its sum.
+constexpr int BAT_TILE = 4096;
+__device__ __forceinline__ long long bat_tile(const InstDesc& I, int b, long long i) {
+    return (I.chunk_off >> 7) + b + i / BAT_TILE;  // instances' tiles do not meet: 128 chunks a tile, one spare each
+}
+
+// This warp's next unit from queue q: units are dealt c0, c0 + 1,
 // ... in order as warps ask for them (>= the caller's end when none is
-// left), so a warp that drew heavy chunks takes fewer of them.
+// left), so a warp that drew heavy units takes fewer of them.
 __device__ __forceinline__ long long bat_next_chunk(unsigned long long* q, long long c0) {
     unsigned long long t = 0;
     if (lane_id() == 0) t = atomicAdd(q, 1ull);
@@ -89,9 +113,9 @@ __device__ __forceinline__ long long bat_brow_len(const InstDesc& I, int k) {
 }
 
 // ---------------------------------------------------------------------------
-// prepare: one warp per 32-row chunk of one instance (chunks dealt from a
-// queue), lane l owning row i0 + l of A_b and of B_b.
-//  * flops: the entries of the chunk's rows of A with at most PREP_SHORT
+// prepare: one warp per unit (BatUnits, dealt from a queue), lane l owning row
+// i0 + l of A_b and of B_b.
+//  * flops: the entries of the unit's rows of A with at most PREP_SHORT
 //    entries are numbered across the rows and read 32 at a time, four
 //    rounds in flight (coalesced); each entry's B row length goes to its row
 //    by a segmented sum over the lanes.  A longer row is then summed by the
@@ -102,21 +126,80 @@ __device__ __forceinline__ long long bat_brow_len(const InstDesc& I, int k) {
 //    a dense-B instance into its dense copy and pattern bits, cleared first.
 // ---------------------------------------------------------------------------
 constexpr int PREP_SHORT = 256;
+// Rows of more entries than this are summed by k_bat_long, a warp per
+// PREP_LONG entries (a hub of 20,000 entries in one warp was a tail of 100 us).
+constexpr int PREP_LONG = 1024;
 
-__global__ void __launch_bounds__(256) k_bat_prepare(const InstDesc* __restrict__ inst, int count, long long c0,
-                                                     long long c1, long long* __restrict__ flops,
-                                                     int* __restrict__ heavy, BatchCtl* ctl) {
+__device__ __forceinline__ void bat_list_heavy(const InstDesc& I, long long i, long long f, int* heavy, BatchCtl* ctl) {
+    if (f > 0 && f >= I.heavy_min) heavy[atomicAdd(&ctl->nheavy, 1ull)] = (int)(I.row_off + i);
+}
+
+// This lane's share of the products of entries [e0, e1) of A, the warp's
+// entries eight loads per lane in flight.
+__device__ __forceinline__ long long bat_sum_entries(const InstDesc& I, long long e0, long long e1, bool& bad) {
+    long long sum = 0;
+    for (long long e = e0 + lane_id(); e < e1; e += 256) {
+        int k[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) k[u] = e + 32 * u < e1 ? __ldg(I.A_col + e + 32 * u) : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (e + 32 * u < e1) {
+                if ((unsigned)k[u] < (unsigned)I.n) sum += bat_brow_len(I, k[u]);
+                else bad = true;
+            }
+        }
+    }
+    return sum;
+}
+
+// The queued parts of long rows: (row, part), a warp each.  The row's products
+// are added up in flops; parts finished are counted above bit 44 of it (a row
+// has at most 2^31 entries of at most 1024 products), and the last part leaves
+// the sum alone and lists the row if it is heavy.
+constexpr int LONG_SHIFT = 44;
+__global__ void __launch_bounds__(256) k_bat_long(const InstDesc* __restrict__ inst, int count,
+                                                  unsigned long long* flops, const long long* __restrict__ items,
+                                                  long long item_cap, int* __restrict__ heavy, BatchCtl* ctl) {
+    const int lane = lane_id();
+    const long long n = min((long long)ctl->nlong, item_cap);
+    bool bad = false;
+    for (long long x = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n;
+         x += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const long long g = items[x] >> 24, part = items[x] & 0xFFFFFF;
+        const InstDesc& I = inst[inst_of(inst, count, g)];
+        const long long i = g - I.row_off;
+        const long long a0 = clampll(__ldg(I.A_rowptr + i), 0, I.annz), a1 = clampll(__ldg(I.A_rowptr + i + 1), a0, I.annz);
+        const long long e0 = a0 + part * PREP_LONG, e1 = e0 + PREP_LONG < a1 ? e0 + PREP_LONG : a1;
+        const long long sum = warp_sum(bat_sum_entries(I, e0, e1, bad));
+        if (lane == 0) {
+            const unsigned long long parts = (unsigned long long)(a1 - a0 + PREP_LONG - 1) / PREP_LONG;
+            const unsigned long long before = atomicAdd(flops + g, (unsigned long long)sum + (1ull << LONG_SHIFT));
+            if ((before >> LONG_SHIFT) == parts - 1) {
+                const long long f = (long long)(before & ((1ull << LONG_SHIFT) - 1)) + sum;
+                flops[g] = (unsigned long long)f;
+                bat_list_heavy(I, i, f, heavy, ctl);
+            }
+        }
+    }
+    if (bad) atomicOr(&ctl->err, ERR_A_COL);
+}
+
+__global__ void __launch_bounds__(256) k_bat_prepare(const InstDesc* __restrict__ inst, int count,
+                                                     BatUnits un, long long* __restrict__ flops,
+                                                     int* __restrict__ heavy, BatchCtl* ctl, long long* items,
+                                                     long long item_cap) {
     __shared__ long long s_f[8][32];
     const int lane = lane_id(), warp = warp_id();
     long long* wf = s_f[warp];
     wf[lane] = 0;
     __syncwarp();
-    bool bad_a = false, bad_b = false;
-    for (long long c = bat_next_chunk(&ctl->l_prep, c0); c < c1; c = bat_next_chunk(&ctl->l_prep, c0)) {
-        const InstDesc& I = inst[inst_of_chunk(inst, count, c)];
-        const long long i0 = (c - I.chunk_off) * 32;
+    bool bad_a = false, bad_b = false, bad_cap = false;
+    for (long long u = bat_next_chunk(&ctl->l_prep, un.u0); u < un.u1; u = bat_next_chunk(&ctl->l_prep, un.u0)) {
+        const InstDesc& I = inst[inst_of_chunk(inst, count, un.chunk(u))];
+        const long long i0 = un.row0(I, u);
         const long long i = i0 + lane;
-        const bool act = i < I.n;
+        const bool act = lane < un.rows && i < I.n;
         long long a0 = 0, a1 = 0;
         if (act) {
             a0 = clampll(__ldg(I.A_rowptr + i), 0, I.annz);
@@ -158,30 +241,26 @@ __global__ void __launch_bounds__(256) k_bat_prepare(const InstDesc* __restrict_
         long long f = wf[lane];
         wf[lane] = 0;
         // long rows, one at a time by the whole warp
-        unsigned longs = __ballot_sync(FULL, a1 - a0 > PREP_SHORT);
+        const bool queued = a1 - a0 > PREP_LONG;
+        unsigned longs = __ballot_sync(FULL, a1 - a0 > PREP_SHORT && !queued);
         while (longs) {
             const int src = __ffs(longs) - 1;
             longs &= longs - 1;
             const long long la0 = shfl64(a0, src), la1 = shfl64(a1, src);
-            long long sum = 0;
-            for (long long e = la0 + lane; e < la1; e += 256) {
-                int k[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) k[u] = e + 32 * u < la1 ? __ldg(I.A_col + e + 32 * u) : 0;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (e + 32 * u < la1) {
-                        if ((unsigned)k[u] < (unsigned)I.n) sum += bat_brow_len(I, k[u]);
-                        else bad_a = true;
-                    }
-                }
-            }
-            sum = warp_sum(sum);
+            const long long sum = warp_sum(bat_sum_entries(I, la0, la1, bad_a));
             if (lane == src) f = sum;
         }
         if (act) {
-            flops[I.row_off + i] = f;
-            if (f > 0 && f >= I.heavy_min) heavy[atomicAdd(&ctl->nheavy, 1ull)] = (int)(I.row_off + i);
+            flops[I.row_off + i] = f;  // 0 for a queued row, whose parts are added later
+            if (!queued) bat_list_heavy(I, i, f, heavy, ctl);
+        }
+        if (queued) {
+            const long long parts = (a1 - a0 + PREP_LONG - 1) / PREP_LONG;
+            const long long at = (long long)atomicAdd(&ctl->nlong, (unsigned long long)parts);
+            for (long long q = 0; q < parts; ++q) {
+                if (at + q < item_cap) items[at + q] = ((I.row_off + i) << 24) | q;
+                else bad_cap = true;
+            }
         }
         // the chunk's rows of B into the copies
         long long bs = 0;
@@ -190,7 +269,7 @@ __global__ void __launch_bounds__(256) k_bat_prepare(const InstDesc* __restrict_
         if (act) padded_row<2>(I.B_rowptr, I.bnnz, (int)I.d, (int)i, bs, blen, g0);
         const bool dense = I.accum == BAT_DENSE_B && I.Bd;
         if (dense) {  // cleared before the entries land
-            const long long nr = I.n - i0 < 32 ? I.n - i0 : 32;
+            const long long nr = I.n - i0 < un.rows ? (I.n > i0 ? I.n - i0 : 0) : un.rows;
             float4* r4 = reinterpret_cast<float4*>(I.Bd + (size_t)i0 * I.Wd);
             for (long long x = lane; x < nr * (I.Wd >> 2); x += 32) r4[x] = make_float4(0.f, 0.f, 0.f, 0.f);
             unsigned* bw = I.Bbits + (size_t)i0 * (I.Wd >> 5);
@@ -242,6 +321,7 @@ __global__ void __launch_bounds__(256) k_bat_prepare(const InstDesc* __restrict_
     }
     if (bad_a) atomicOr(&ctl->err, ERR_A_COL);
     if (bad_b) atomicOr(&ctl->err, ERR_B_COL);
+    if (bad_cap) atomicOr(&ctl->err, ERR_C_ROW);  // row pointers of A that do not ascend
 }
 
 // Ascending bitonic sort of one key per lane across the warp, carrying val.
@@ -261,15 +341,15 @@ __device__ __forceinline__ void warp_sort_asc(int& key, int& val) {
     }
 }
 
-// Light rows of one 32-row chunk of instance I, sorted by products
+// Light rows of one unit of `rows` rows of instance I, sorted by products
 // (heaviest first) so that the four rows a warp takes side by side have
 // nearly equal lengths: returns the count L; sorted position t of the warp
 // holds row base + srt (lanes >= L hold no row).
 __device__ __forceinline__ int chunk_light_sorted(const InstDesc& I, const long long* __restrict__ flops,
-                                                  long long i0, int& srt) {
+                                                  long long i0, int rows, int& srt) {
     const int lane = lane_id();
     const long long i = i0 + lane;
-    const long long f = i < I.n ? __ldg(flops + I.row_off + i) : 0;
+    const long long f = lane < rows && i < I.n ? __ldg(flops + I.row_off + i) : 0;
     const bool light = f > 0 && f < I.heavy_min;
     int key = light ? -(int)(f < (1LL << 30) ? f : (1LL << 30)) : 0x7FFFFFFF;
     srt = lane;
@@ -301,7 +381,13 @@ __device__ __forceinline__ BatRow bat_row(const InstDesc& I, long long i0, int s
     return b;
 }
 
-// Whether global row g (lane's row of a 32-row chunk) is a light row: it
+// A group of four rows whose longest has this many entries of A or more is
+// taken row by row, the row's entries shared out over the four slots: in one
+// slot a row is a serial chain (0.3 us an entry), and at the block threshold of
+// 4096 products one of short rows of B was most of the pass.
+constexpr int BAT_TEAM = 64;
+
+// Whether global row g (lane's row of a unit) is a light row: it
 // has products and fewer than its instance's threshold.
 __device__ __forceinline__ bool bat_light(const InstDesc* inst, int count, const long long* flops, long long g,
                                           long long g1, int& b) {
@@ -326,9 +412,10 @@ struct AddByte {
 // ---------------------------------------------------------------------------
 // symbolic: row counts into each C_b's row pointers (C_b.rowptr[i + 1])
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict__ inst, int count, long long c0,
-                                                      long long c1, const long long* __restrict__ flops,
-                                                      const int* __restrict__ heavy, BatchCtl* ctl, int Wmax) {
+__global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict__ inst, int count,
+                                                      BatUnits un, const long long* __restrict__ flops,
+                                                      const int* __restrict__ heavy, BatchCtl* ctl,
+                                                      unsigned long long* __restrict__ part, int Wmax) {
     __shared__ __align__(16) unsigned char s_hb[1024];  // the block's byte marks (heavy rows)
     // four slots of byte marks per warp (light rows), Wmax + 32 bytes each
     // (the pad puts the slots' words on different banks)
@@ -348,7 +435,8 @@ __global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict
         __syncthreads();
         if (h >= nheavy) break;
         const long long g = heavy[h];
-        const InstDesc& I = inst[inst_of(inst, count, g)];
+        const int b = inst_of(inst, count, g);
+        const InstDesc& I = inst[b];
         const long long i = g - I.row_off;
         const NumParams p = inst_params(I);
         const long long a0 = clampll(I.A_rowptr[i], 0, I.annz), a1 = clampll(I.A_rowptr[i + 1], a0, I.annz);
@@ -372,7 +460,10 @@ __global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict
                 reinterpret_cast<unsigned*>(s_hb)[x] = 0u;
             }
             cnt = warp_sum(cnt);
-            if (lane == 0) I.C_rowptr[i + 1] = cnt;
+            if (lane == 0) {
+                I.C_rowptr[i + 1] = cnt;
+                atomicAdd(part + bat_tile(I, b, i), (unsigned long long)cnt);
+            }
         }
         __syncthreads();
     }
@@ -380,18 +471,20 @@ __global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict
     // chunk's rows sorted by products), each marking its own bytes
     const int lanes = lane & 7, slot = lane >> 3;
     unsigned char* mym = s_marks + (size_t)(warp * 4 + slot) * mstride;
-    for (long long c = bat_next_chunk(&ctl->l_sym, c0); c < c1; c = bat_next_chunk(&ctl->l_sym, c0)) {
-        const InstDesc& I = inst[inst_of_chunk(inst, count, c)];
-        const long long i0 = (c - I.chunk_off) * 32;
+    for (long long u = bat_next_chunk(&ctl->l_sym, un.u0); u < un.u1; u = bat_next_chunk(&ctl->l_sym, un.u0)) {
+        const int b = inst_of_chunk(inst, count, un.chunk(u));
+        const InstDesc& I = inst[b];
+        const long long i0 = un.row0(I, u);
         {
             const long long i = i0 + lane;
-            if (i < I.n && __ldg(flops + I.row_off + i) <= 0) I.C_rowptr[i + 1] = 0;
+            if (lane < un.rows && i < I.n && __ldg(flops + I.row_off + i) <= 0) I.C_rowptr[i + 1] = 0;
         }
         int srt;
-        const int L = chunk_light_sorted(I, flops, i0, srt);
+        const int L = chunk_light_sorted(I, flops, i0, un.rows, srt);
         const NumParams p = inst_params(I);
         const int nw = I.W >> 5;
-        // pipelined over the chunk's groups: the next group's row bounds load
+        int sum = 0;  // this lane's part of the unit's counts
+        // pipelined over the unit's groups: the next group's row bounds load
         // before this group's walk, its first entries of A before the count
         BatRow cur = bat_row(I, i0, srt, L, 0, false);
         int k0, k1;
@@ -401,6 +494,38 @@ __global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict
         for (int t = 0; t < L; t += 4) {
             const BatRow nxt = bat_row(I, i0, srt, L, t + 4, false);
             const int lmax = (int)__reduce_max_sync(FULL, (unsigned)cur.len);
+            if (lmax >= BAT_TEAM) {  // row by row, all slots marking slot 0's bytes
+                unsigned char* tm = s_marks + (size_t)warp * 4 * mstride;
+                for (int h = 0; h < 4 && t + h < L; ++h) {
+                    long long a0 = shfl64(cur.a0, 8 * h);
+                    int len = __shfl_sync(FULL, cur.len, 8 * h);
+                    const long long i = shfl64(cur.i, 8 * h);
+                    team_share(slot, 4, a0, len);
+                    int q0, q1;
+                    float y0, y1;
+                    rg_load_a(p, a0 + lanes, lanes < len, q0, y0);
+                    rg_load_a(p, a0 + 8 + lanes, 8 + lanes < len, q1, y1);
+                    const int lm = (int)__reduce_max_sync(FULL, (unsigned)len);
+                    rgp_tile<8, 2>(p, I.Bq, AddByte{tm}, a0, len, lm, err, q0, y0, q1, y1);
+                    __syncwarp();
+                    int cnt = 0;
+                    unsigned* mw = reinterpret_cast<unsigned*>(tm);
+                    for (int w = lane; w < nw * 8; w += 32) {
+                        cnt += __popc(mw[w]);
+                        mw[w] = 0u;
+                    }
+                    cnt = warp_sum(cnt);
+                    if (lane == 0) {
+                        I.C_rowptr[i + 1] = cnt;
+                        sum += cnt;
+                    }
+                    __syncwarp();
+                }
+                rg_load_a(p, nxt.a0 + lanes, lanes < nxt.len, k0, x0);
+                rg_load_a(p, nxt.a0 + 8 + lanes, 8 + lanes < nxt.len, k1, x1);
+                cur = nxt;
+                continue;
+            }
             rgp_tile<8, 2>(p, I.Bq, AddByte{mym}, cur.a0, cur.len, lmax, err, k0, x0, k1, x1);
             rg_load_a(p, nxt.a0 + lanes, lanes < nxt.len, k0, x0);
             rg_load_a(p, nxt.a0 + 8 + lanes, 8 + lanes < nxt.len, k1, x1);
@@ -414,57 +539,61 @@ __global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict
             cnt += __shfl_xor_sync(FULL, cnt, 1);
             cnt += __shfl_xor_sync(FULL, cnt, 2);
             cnt += __shfl_xor_sync(FULL, cnt, 4);
-            if (cur.i >= 0 && lanes == 0) I.C_rowptr[cur.i + 1] = cnt;
+            if (cur.i >= 0 && lanes == 0) {
+                I.C_rowptr[cur.i + 1] = cnt;
+                sum += cnt;
+            }
             __syncwarp();
             cur = nxt;
         }
+        sum = warp_sum(sum);
+        if (lane == 0 && sum) atomicAdd(part + bat_tile(I, b, i0), (unsigned long long)sum);
     }
 }
 
 // ---------------------------------------------------------------------------
-// scan: one block of 1024 threads per instance, in place over C_b.rowptr
+// scan: a block of 1024 threads per BAT_TILE rows of an instance, `tiles` blocks
+// for each (as many as the largest needs), in place over C_b.rowptr, from the sums of the tiles before it (one block per
+// instance took 168 us for 200,000 rows)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_bat_scan(const InstDesc* __restrict__ inst, BatchCtl* ctl) {
+__global__ void __launch_bounds__(1024) k_bat_scan(const InstDesc* __restrict__ inst, BatchCtl* ctl,
+                                                   const unsigned long long* __restrict__ part, unsigned tiles) {
     __shared__ long long s_w[32];
-    __shared__ long long s_carry;
-    const InstDesc& I = inst[blockIdx.x];
+    __shared__ long long s_before[32];
+    const int b = (int)(blockIdx.x / tiles), tile = (int)(blockIdx.x - b * tiles);
+    const InstDesc& I = inst[b];
+    const long long t0 = (long long)tile * BAT_TILE;
+    if (t0 >= I.n && t0 > 0) return;
     long long* rp = I.C_rowptr;
     const int tid = threadIdx.x, lane = lane_id(), warp = warp_id();
-    if (tid == 0) {
-        s_carry = 0;
-        rp[0] = 0;
+    if (t0 == 0 && tid == 0) rp[0] = 0;
+    constexpr int ITEMS = BAT_TILE / 1024;
+    long long v[ITEMS], t = 0, before = 0;
+    for (int x = tid; x < tile; x += 1024) before += (long long)part[bat_tile(I, b, 0) + x];
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+        const long long x = t0 + 1 + (long long)tid * ITEMS + u;
+        t += x <= I.n ? rp[x] : 0;
+        v[u] = t;  // running sum inside the thread
+    }
+    const long long wi = warp_incl_scan(t);
+    before = warp_sum(before);
+    if (lane == 31) s_w[warp] = wi;
+    if (lane == 0) s_before[warp] = before;
+    __syncthreads();
+    if (warp == 0) {
+        const long long y = s_w[lane];
+        const long long all = warp_sum(s_before[lane]);
+        s_w[lane] = all + warp_incl_scan(y) - y;
     }
     __syncthreads();
-    constexpr int ITEMS = 4;
-    for (long long base = 1; base <= I.n; base += 1024LL * ITEMS) {
-        long long v[ITEMS];
-        long long t = 0;
+    const long long base = s_w[warp] + wi - t;
 #pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const long long x = base + (long long)tid * ITEMS + u;
-            v[u] = x <= I.n ? rp[x] : 0;
-            t += v[u];
-            v[u] = t;  // running sum inside the thread
-        }
-        const long long wi = warp_incl_scan(t);
-        if (lane == 31) s_w[warp] = wi;
-        __syncthreads();
-        if (warp == 0) {
-            const long long y = warp_incl_scan(s_w[lane]);
-            s_w[lane] = y;
-        }
-        __syncthreads();
-        const long long before = s_carry + (warp ? s_w[warp - 1] : 0) + wi - t;
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const long long x = base + (long long)tid * ITEMS + u;
-            if (x <= I.n) rp[x] = before + v[u];
-        }
-        __syncthreads();
-        if (tid == 0) s_carry += s_w[31];
-        __syncthreads();
+    for (int u = 0; u < ITEMS; ++u) {
+        const long long x = t0 + 1 + (long long)tid * ITEMS + u;
+        if (x <= I.n) rp[x] = base + v[u];
+        if (x == I.n && base + v[u] > I.cap) atomicOr(&ctl->err, ERR_CAPACITY);
     }
-    if (tid == 0 && s_carry > I.cap) atomicOr(&ctl->err, ERR_CAPACITY);
 }
 
 // ---------------------------------------------------------------------------
@@ -523,8 +652,8 @@ __host__ __device__ inline int bat_per_warp(int Wmax, bool values) {
 // block, or the dense-B form), then light rows (one warp each, in row
 // order).  Dynamic shared memory per warp: Wmax + 8 floats of accumulator
 // and Wmax/32 + 1 bitmap words.
-__global__ void __launch_bounds__(256, 3) k_bat_numeric(const InstDesc* __restrict__ inst, int count, long long c0,
-                                                        long long c1, const long long* __restrict__ flops,
+__global__ void __launch_bounds__(256, 3) k_bat_numeric(const InstDesc* __restrict__ inst, int count,
+                                                        BatUnits un, const long long* __restrict__ flops,
                                                         const int* __restrict__ heavy, BatchCtl* ctl, int Wmax,
                                                         bool values) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -623,20 +752,20 @@ __global__ void __launch_bounds__(256, 3) k_bat_numeric(const InstDesc* __restri
         if (tid == 0 && out + tot != out_end) atomicOr(err, ERR_C_ROW);
         __syncthreads();
     }
-    // light rows, by 32-row chunks of one instance.  Plus-times with every
+    // light rows, by units of one instance.  Plus-times with every
     // width <= 256: four rows per warp in row groups (eight lanes, private
     // accumulators that start RG_EMPTY, rows sorted by products); dense-B
     // instances one row per warp in registers; otherwise one row per warp on
     // the warp's shared accumulator.
     const int lanes = lane & 7, slot = lane >> 3;
-    for (long long c = bat_next_chunk(&ctl->l_num, c0); c < c1; c = bat_next_chunk(&ctl->l_num, c0)) {
-        const InstDesc& I = inst[inst_of_chunk(inst, count, c)];
-        const long long i0 = (c - I.chunk_off) * 32;
+    for (long long u = bat_next_chunk(&ctl->l_num, un.u0); u < un.u1; u = bat_next_chunk(&ctl->l_num, un.u0)) {
+        const InstDesc& I = inst[inst_of_chunk(inst, count, un.chunk(u))];
+        const long long i0 = un.row0(I, u);
         const NumParams p = inst_params(I);
         const bool dense = I.accum == BAT_DENSE_B && I.Bd && I.C_val;
         if (rg && !dense) {
             int srt;
-            const int L = chunk_light_sorted(I, flops, i0, srt);
+            const int L = chunk_light_sorted(I, flops, i0, un.rows, srt);
             const int Wi = I.W;
             float* myacc = wacc + (size_t)slot * (Wi + 8);
             for (int t = 0; t < L; t += 4) {
@@ -644,6 +773,23 @@ __global__ void __launch_bounds__(256, 3) k_bat_numeric(const InstDesc* __restri
                 const int lmax = (int)__reduce_max_sync(FULL, (unsigned)cur.len);
                 int k0, k1;
                 float x0, x1;
+                if (lmax >= BAT_TEAM) {  // row by row, shared by the slots
+                    for (int h = 0; h < 4 && t + h < L; ++h) {
+                        long long a0 = shfl64(cur.a0, 8 * h), out = shfl64(cur.out, 8 * h);
+                        const long long out_end = shfl64(cur.out_end, 8 * h);
+                        int len = __shfl_sync(FULL, cur.len, 8 * h);
+                        team_share(slot, 4, a0, len);
+                        rg_load_a(p, a0 + lanes, lanes < len, k0, x0);
+                        rg_load_a(p, a0 + 8 + lanes, 8 + lanes < len, k1, x1);
+                        const int lm = (int)__reduce_max_sync(FULL, (unsigned)len);
+                        rgp_tile<8, 2>(p, I.Bq, AddPlain{myacc}, a0, len, lm, err, k0, x0, k1, x1);
+                        rg_emit_team<8>(wacc, Wi, out, out_end, I.C_col, I.C_val);
+                        if (lanes == 0) myacc[Wi] = __uint_as_float(RG_EMPTY);
+                        if (lane == 0 && out != out_end) atomicOr(err, ERR_C_ROW);
+                        __syncwarp();
+                    }
+                    continue;
+                }
                 rg_load_a(p, cur.a0 + lanes, lanes < cur.len, k0, x0);
                 rg_load_a(p, cur.a0 + 8 + lanes, 8 + lanes < cur.len, k1, x1);
                 rgp_tile<8, 2>(p, I.Bq, AddPlain{myacc}, cur.a0, cur.len, lmax, err, k0, x0, k1, x1);
@@ -657,7 +803,7 @@ __global__ void __launch_bounds__(256, 3) k_bat_numeric(const InstDesc* __restri
             continue;
         }
         const long long g = I.row_off + i0 + lane;
-        const long long f = i0 + lane < I.n ? __ldg(flops + g) : 0;
+        const long long f = lane < un.rows && i0 + lane < I.n ? __ldg(flops + g) : 0;
         unsigned rows = __ballot_sync(FULL, f > 0 && f < I.heavy_min);
         while (rows) {
             const int src = __ffs(rows) - 1;
@@ -844,7 +990,8 @@ __device__ __forceinline__ void bat_scatter_dc(const InstDesc& I, long long i, f
 }
 
 __global__ void __launch_bounds__(256, 4) k_bat_backward(const InstDesc* __restrict__ inst, int count, long long g0,
-                                                         long long g1, const long long* __restrict__ flops,
+                                                         long long g1, int urows,
+                                                         const long long* __restrict__ flops,
                                                          const int* __restrict__ heavy, BatchCtl* ctl, int Wmax) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_item;
@@ -876,17 +1023,17 @@ __global__ void __launch_bounds__(256, 4) k_bat_backward(const InstDesc* __restr
         bat_scatter_dc(I, i, trow, tid, blockDim.x, true);
         __syncthreads();
     }
-    const long long nchunks = (g1 - g0 + 31) / 32;
-    for (long long ch = bat_next_chunk(&ctl->l_bwd, 0); ch < nchunks; ch = bat_next_chunk(&ctl->l_bwd, 0)) {
-        const long long g = g0 + ch * 32 + lane;
-        int b;
-        unsigned rows = __ballot_sync(FULL, bat_light(inst, count, flops, g, g1, b));
+    const long long nunits = (g1 - g0 + urows - 1) / urows;
+    for (long long ch = bat_next_chunk(&ctl->l_bwd, 0); ch < nunits; ch = bat_next_chunk(&ctl->l_bwd, 0)) {
+        const long long g = g0 + ch * urows + lane;
+        int b = 0;
+        unsigned rows = __ballot_sync(FULL, lane < urows && bat_light(inst, count, flops, g, g1, b));
         while (rows) {
             const int src = __ffs(rows) - 1;
             rows &= rows - 1;
             const InstDesc& I = inst[__shfl_sync(FULL, b, src)];
             if (!I.dC) continue;
-            const long long i = g0 + ch * 32 + src - I.row_off;
+            const long long i = g0 + ch * urows + src - I.row_off;
             bat_scatter_dc(I, i, wrow, lane, 32, false);
             __syncwarp();
             const long long a0 = clampll(I.A_rowptr[i], 0, I.annz), a1 = clampll(I.A_rowptr[i + 1], a0, I.annz);
@@ -923,32 +1070,64 @@ __global__ void __launch_bounds__(256) k_batch_bounds(const InstDesc* __restrict
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+// Rows of a unit: as many as leave every resident warp (32 per SM) about
+// BAT_UNITS units, in a chunk or a part of it.
+constexpr int BAT_UNITS = 2;
+static int unit_rows(long long chunks, int sms) {
+    int rows = 32;
+    while (rows > 4 && chunks * (32 / rows) < 32LL * sms * BAT_UNITS) rows /= 2;
+    return rows;
+}
+
+static BatUnits bat_units(long long c0, long long c1, int sms) {
+    BatUnits un;
+    un.rows = unit_rows(c1 - c0, sms);
+    un.shift = 0;
+    while ((un.rows << un.shift) < 32) ++un.shift;
+    un.u0 = c0 << un.shift;
+    un.u1 = c1 << un.shift;
+    return un;
+}
+
 cudaError_t launch_bat_prepare(const InstDesc* inst, int count, long long c0, long long c1, long long* flops,
-                               int* heavy, BatchCtl* ctl, int sms, cudaStream_t st) {
+                               int* heavy, BatchCtl* ctl, long long* items, long long item_cap, int sms,
+                               cudaStream_t st) {
     if (c1 <= c0) return cudaSuccess;
+    const BatUnits un = bat_units(c0, c1, sms);
     long long grid = persistent_grid((const void*)k_bat_prepare, 256, 0, sms);
-    if (grid > (c1 - c0 + 7) / 8) grid = (c1 - c0 + 7) / 8;
+    if (grid > (un.u1 - un.u0 + 7) / 8) grid = (un.u1 - un.u0 + 7) / 8;
     count_launch();
-    k_bat_prepare<<<(unsigned)grid, 256, 0, st>>>(inst, count, c0, c1, flops, heavy, ctl);
+    k_bat_prepare<<<(unsigned)grid, 256, 0, st>>>(inst, count, un, flops, heavy, ctl, items, item_cap);
+    if (item_cap <= 0) return cudaGetLastError();  // no instance has that many entries
+    grid = (item_cap + 7) / 8 < 8LL * sms ? (item_cap + 7) / 8 : 8LL * sms;
+    count_launch();
+    k_bat_long<<<(unsigned)grid, 256, 0, st>>>(inst, count, (unsigned long long*)flops, items, item_cap, heavy, ctl);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bat_symbolic(const InstDesc* inst, int count, long long c0, long long c1, long long,
-                                const long long* flops, const int* heavy, BatchCtl* ctl, int Wmax, int sms,
-                                cudaStream_t st) {
+                                const long long* flops, const int* heavy, BatchCtl* ctl, unsigned long long* part,
+                                int Wmax, int sms, cudaStream_t st) {
     if (c1 <= c0) return cudaSuccess;
     if (Wmax < 32 || Wmax > 1024 || (Wmax & 31)) return cudaErrorInvalidValue;
     const size_t smem = 8 * 4 * (size_t)(Wmax + 32);
     const int grid = persistent_grid((const void*)k_bat_symbolic, 256, smem, sms);
     count_launch();
-    k_bat_symbolic<<<grid, 256, smem, st>>>(inst, count, c0, c1, flops, heavy, ctl, Wmax);
+    k_bat_symbolic<<<grid, 256, smem, st>>>(inst, count, bat_units(c0, c1, sms), flops, heavy, ctl, part, Wmax);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bat_scan(const InstDesc* inst, int count, BatchCtl* ctl, cudaStream_t st) {
+long long bat_long_capacity(long long annz) { return annz > PREP_LONG ? 2 * (annz / PREP_LONG) : 0; }
+
+long long bat_tiles(long long chunks, int count) { return chunks / 128 + count + 1; }
+
+cudaError_t launch_bat_scan(const InstDesc* inst, int count, long long max_rows, BatchCtl* ctl,
+                            const unsigned long long* part, cudaStream_t st) {
     if (count < 1) return cudaSuccess;
+    const long long tiles = max_rows > BAT_TILE ? (max_rows + BAT_TILE - 1) / BAT_TILE : 1;
+    if (tiles * count > INT_MAX) return cudaErrorInvalidValue;
     count_launch();
-    k_bat_scan<<<count, 1024, 0, st>>>(inst, ctl);
+    k_bat_scan<<<(unsigned)(tiles * count), 1024, 0, st>>>(inst, ctl, part, (unsigned)tiles);
     return cudaGetLastError();
 }
 
@@ -964,7 +1143,7 @@ cudaError_t launch_bat_numeric(const InstDesc* inst, int count, long long c0, lo
         return e;
     const int grid = persistent_grid((const void*)k_bat_numeric, 256, smem, sms);
     count_launch();
-    k_bat_numeric<<<grid, 256, smem, st>>>(inst, count, c0, c1, flops, heavy, ctl, Wmax, values != 0);
+    k_bat_numeric<<<grid, 256, smem, st>>>(inst, count, bat_units(c0, c1, sms), flops, heavy, ctl, Wmax, values != 0);
     return cudaGetLastError();
 }
 
@@ -986,7 +1165,7 @@ cudaError_t launch_bat_backward(const InstDesc* inst, int count, long long g0, l
         return e;
     const int grid = persistent_grid((const void*)k_bat_backward, 256, smem, sms);
     count_launch();
-    k_bat_backward<<<grid, 256, smem, st>>>(inst, count, g0, g1, flops, heavy, ctl, Wmax);
+    k_bat_backward<<<grid, 256, smem, st>>>(inst, count, g0, g1, unit_rows((g1 - g0) / 32, sms), flops, heavy, ctl, Wmax);
     return cudaGetLastError();
 }
 

@@ -231,18 +231,26 @@ struct InstDesc {
 // (l_*), and the error flags.  The forward zeroes all of it, the backward
 // q_bwd and l_bwd.
 struct BatchCtl {
-    unsigned long long nheavy, q_sym, q_num, q_bwd, l_bwd, l_sym, l_num, l_prep, err;
+    unsigned long long nheavy, q_sym, q_num, q_bwd, l_bwd, l_sym, l_num, l_prep, err, nlong;
 };
 // 32-row chunks [c0, c1) of the batch's chunk numbering over the instances
 // inst[0..count) (every chunk lies in one instance).
+// items: room for item_cap parts of very long rows, at least
+// bat_long_capacity(entries of A) summed over the instances.
+long long bat_long_capacity(long long annz);
 cudaError_t launch_bat_prepare(const InstDesc* inst, int count, long long c0, long long c1, long long* flops,
-                               int* heavy, BatchCtl* ctl, int sms, cudaStream_t st);
+                               int* heavy, BatchCtl* ctl, long long* items, long long item_cap, int sms,
+                               cudaStream_t st);
 // symbolic / numeric: 32-row chunks [c0, c1) of the batch's chunk numbering
 // (every chunk lies in one instance); `values` = plus-times
 cudaError_t launch_bat_symbolic(const InstDesc* inst, int count, long long c0, long long c1, long long unused,
-                                const long long* flops, const int* heavy, BatchCtl* ctl, int Wmax, int sms,
-                                cudaStream_t st);
-cudaError_t launch_bat_scan(const InstDesc* inst, int count, BatchCtl* ctl, cudaStream_t st);
+                                const long long* flops, const int* heavy, BatchCtl* ctl, unsigned long long* part,
+                                int Wmax, int sms, cudaStream_t st);
+// part: bat_tiles(chunks of the whole batch, count) sums, cleared before the
+// symbolic pass, which fills them for the scan.
+long long bat_tiles(long long chunks, int count);
+cudaError_t launch_bat_scan(const InstDesc* inst, int count, long long max_rows, BatchCtl* ctl,
+                            const unsigned long long* part, cudaStream_t st);
 cudaError_t launch_bat_numeric(const InstDesc* inst, int count, long long c0, long long c1, long long values,
                                const long long* flops, const int* heavy, BatchCtl* ctl, int Wmax, int sms,
                                cudaStream_t st);
