@@ -126,13 +126,26 @@ struct BwdOp {
     }
 };
 
-// dC row i scattered into the dense row g (or cleared again).
+// dC row i scattered into the dense row g (or cleared again), U entries per
+// thread in flight.
+template <int U>
 __device__ __forceinline__ void scatter_dc(const BwdParams& p, long long c0, long long c1, float* g, bool clear,
                                            int tid, int nthr, unsigned long long* err) {
-    for (long long e = c0 + tid; e < c1; e += nthr) {
-        const int c = __ldg(p.Ci + e);
-        if ((unsigned)c < (unsigned)p.d) g[c] = clear ? 0.0f : __ldg(p.dC + e);
-        else if (!clear) atomicOr(err, ERR_C_ROW);
+    for (long long e = c0 + tid; e < c1; e += U * nthr) {
+        int cc[U];
+        float vv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long eu = e + u * nthr;
+            cc[u] = eu < c1 ? __ldg(p.Ci + eu) : 0;
+            vv[u] = !clear && eu < c1 ? __ldg(p.dC + eu) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (e + u * nthr >= c1) break;
+            if ((unsigned)cc[u] < (unsigned)p.d) g[cc[u]] = vv[u];
+            else if (!clear) atomicOr(err, ERR_C_ROW);
+        }
     }
 }
 
@@ -219,7 +232,7 @@ __device__ __forceinline__ void backward_range_cta(const BwdParams& p, const BA&
     unsigned long long* err = &p.hdr->err;
     const long long c0 = clampll(__ldg(p.Cp + row), 0, p.nnzC);
     const long long c1 = clampll(__ldg(p.Cp + row + 1), c0, p.nnzC);
-    scatter_dc(p, c0, c1, g, false, threadIdx.x, blockDim.x, err);
+    scatter_dc<1>(p, c0, c1, g, false, threadIdx.x, blockDim.x, err);
     __syncthreads();
     const int nw = blockDim.x >> 5;
     const SegWhole seg{p.Bp, p.nnzB, p.d};
@@ -229,7 +242,7 @@ __device__ __forceinline__ void backward_range_cta(const BwdParams& p, const BA&
         bwd_chunk<G>(p, load_chunk(e0, nv, p.Ai, p.Ax, p.nB, seg, err), nv, e0, op, sdA);
     }
     __syncthreads();
-    scatter_dc(p, c0, c1, g, true, threadIdx.x, blockDim.x, err);
+    scatter_dc<1>(p, c0, c1, g, true, threadIdx.x, blockDim.x, err);
     __syncthreads();
 }
 
@@ -259,7 +272,7 @@ struct BwdRowBody {
             pc1 = clampll(__ldg(p.Cp + next_row + 1), pc0, p.nnzC);
             pref_row = next_row;
         }
-        scatter_dc(p, c0, c1, g, false, lane_id(), 32, err);
+        scatter_dc<4>(p, c0, c1, g, false, lane_id(), 32, err);
         __syncwarp();
         const SegWhole seg{p.Bp, p.nnzB, p.d};
         BwdOp<BA> op{ba, g, sdA, p.dA, p.dB, p.dA != nullptr, p.d, err, {0.0f, 0.0f}};
@@ -271,7 +284,7 @@ struct BwdRowBody {
     }
     __device__ __forceinline__ void finish(int) {
         __syncwarp();
-        scatter_dc(p, c0, c1, g, true, lane_id(), 32, err);
+        scatter_dc<4>(p, c0, c1, g, true, lane_id(), 32, err);
         __syncwarp();
     }
 };
@@ -365,13 +378,125 @@ __device__ __forceinline__ void brg_seg(const BwdParams& p, int k, bool ok, long
     else atomicOr(err, ERR_A_COL);
 }
 
+// One unit of the light rows: R rows, a slot each (`my` is this slot's place in
+// the class order), or (TEAM) one row whose entries the slots share; the whole
+// warp then scatters its row of dC into slot 0's dense row.
+template <int RG, bool TEAM>
+__device__ __forceinline__ void brg_unit(const BwdParams& p, float* fsm, unsigned my, unsigned end) {
+    constexpr int R = 32 / RG;
+    const int warp = warp_id(), lane = lane_id();
+    const int g = lane / RG, gl = lane % RG;
+    unsigned long long* err = &p.hdr->err;
+    const int4* P4 = reinterpret_cast<const int4*>(p.Bpk);
+    const long long* mark = p.s.flops;
+    float* gr = fsm + (size_t)(warp * R + (TEAM ? 0 : g)) * p.dpad;
+    const int tl = TEAM ? lane : gl;
+    constexpr int tn = TEAM ? 32 : RG;  // lanes on one row of dC
+    long long a0 = 0, a1 = 0, c0 = 0, c1 = 0;
+    if (my < end) {
+        const int row = __ldg(p.perm + my);
+        a0 = clampll(__ldg(p.Ap + row), 0, p.nnzA);
+        a1 = clampll(__ldg(p.Ap + row + 1), a0, p.nnzA);
+        if (is_split_row(mark, row, a1 - a0)) {
+            a1 = a0;  // done by split parts
+        } else {
+            c0 = clampll(__ldg(p.Cp + row), 0, p.nnzC);
+            c1 = clampll(__ldg(p.Cp + row + 1), c0, p.nnzC);
+        }
+    }
+    int len = (int)(a1 - a0);
+    if (TEAM) team_share(g, R, a0, len);
+    // first two chunks of A while dC is scattered
+    int k0, k1;
+    float x0, x1;
+    brg_load_a(p, a0 + gl, gl < len, k0, x0);
+    brg_load_a(p, a0 + RG + gl, RG + gl < len, k1, x1);
+    // the row of dC into the dense row, eight entries per lane in flight
+    // (the row is read once, from DRAM: a chain of single loads would
+    // wait out one memory latency per entry)
+    for (long long e = c0 + tl; e < c1; e += 8 * tn) {
+        int cc[8];
+        float vv[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const long long eu = e + u * tn;
+            cc[u] = eu < c1 ? __ldg(p.Ci + eu) : 0;
+            vv[u] = eu < c1 ? __ldg(p.dC + eu) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (e + u * tn < c1) {
+                if ((unsigned)cc[u] < (unsigned)p.d) gr[cc[u]] = vv[u];
+                else atomicOr(err, ERR_C_ROW);
+            }
+        }
+    }
+    long long sg;
+    int L;
+    brg_seg(p, k0, gl < len, sg, L, err);
+    __syncwarp();
+    const int lmax = (int)__reduce_max_sync(FULL, (unsigned)len);
+    BrgSeg nxt = brg_seg_of(shfl64(sg, g * RG), __shfl_sync(FULL, L, g * RG), __shfl_sync(FULL, x0, g * RG));
+    int4 nv = make_int4(0, 0, 0, 0);
+    brg_fetch(P4, nxt, gl, nv);
+    for (int e = 0; e < lmax; e += RG) {
+        int k2;
+        float x2;
+        long long ns;
+        int nL;
+        brg_load_a(p, a0 + e + 2 * RG + gl, e + 2 * RG + gl < len, k2, x2);
+        brg_seg(p, k1, e + RG + gl < len, ns, nL, err);
+        const int nu = lmax - e < RG ? lmax - e : RG;
+        float mine = 0.0f;  // dA of entry e + gl of this slot's row
+        for (int u = 0; u < nu; ++u) {
+            const BrgSeg cur = nxt;
+            const int4 cv = nv;
+            long long s2;
+            int L2;
+            float a2;
+            if (u + 1 < nu) {
+                s2 = shfl64(sg, g * RG + u + 1);
+                L2 = __shfl_sync(FULL, L, g * RG + u + 1);
+                a2 = __shfl_sync(FULL, x0, g * RG + u + 1);
+            } else {
+                s2 = shfl64(ns, g * RG);
+                L2 = __shfl_sync(FULL, nL, g * RG);
+                a2 = __shfl_sync(FULL, x1, g * RG);
+            }
+            nxt = brg_seg_of(s2, L2, a2);
+            brg_fetch(P4, nxt, gl, nv);
+            float part = 0.0f;
+            if (2 * gl < cur.span) part = brg_apply(p, cur, gl, cv, gr, err);
+            for (int q = gl + RG; 2 * q < cur.span; q += RG) {
+                int4 w = make_int4(0, 0, 0, 0);
+                brg_fetch(P4, cur, q, w);
+                part += brg_apply(p, cur, q, w, gr, err);
+            }
+#pragma unroll
+            for (int o = RG / 2; o >= 1; o >>= 1) part += __shfl_xor_sync(FULL, part, o, RG);
+            if (gl == u) mine = part;
+        }
+        if (p.dA && e + gl < len) p.dA[a0 + e + gl] = mine;
+        sg = ns;
+        L = nL;
+        x0 = x1;
+        k1 = k2;
+        x1 = x2;
+    }
+    __syncwarp();
+    // clear the whole dense row with 16-byte stores (dpad is a multiple
+    // of 32, rows 16-byte aligned): cheaper than revisiting the row's
+    // entries of C
+    for (int c = 4 * tl; c < p.dpad; c += 4 * tn) *reinterpret_cast<float4*>(gr + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncwarp();
+}
+
 template <int RG>
 __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
     extern __shared__ __align__(16) float fsm[];
     __shared__ LightUnits s_lu;
     constexpr int R = 32 / RG;
-    const int nw = blockDim.x >> 5, warp = warp_id(), lane = lane_id(), tid = threadIdx.x;
-    const int g = lane / RG, gl = lane % RG;
+    const int nw = blockDim.x >> 5, warp = warp_id(), tid = threadIdx.x;
     for (int i = tid; i < nw * R * p.dpad; i += blockDim.x) fsm[i] = 0.0f;
     if (tid < 32) {  // one warp; its lanes store the same values
         LightUnits lu;
@@ -380,114 +505,10 @@ __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
     }
     __syncthreads();
     const LightUnits& lu = s_lu;
-    unsigned long long* err = &p.hdr->err;
-    const int4* P4 = reinterpret_cast<const int4*>(p.Bpk);
-    const long long* mark = p.s.flops;
-    for (unsigned un = blockIdx.x * nw + warp; un < lu.units; un += gridDim.x * nw) {
-        // a unit is R rows, a slot each, or one row whose entries the slots
-        // share: the whole warp then scatters its row of dC into slot 0's
-        const bool team = lu.team(un);
-        float* gr = fsm + (size_t)(warp * R + (team ? 0 : g)) * p.dpad;
-        const int tl = team ? lane : gl, tn = team ? 32 : RG;  // lanes on one row of dC
-        const unsigned my = lu.row_at(un, g, R);
-        long long a0 = 0, a1 = 0, c0 = 0, c1 = 0;
-        if (my < lu.end) {
-            const int row = __ldg(p.perm + my);
-            a0 = clampll(__ldg(p.Ap + row), 0, p.nnzA);
-            a1 = clampll(__ldg(p.Ap + row + 1), a0, p.nnzA);
-            if (is_split_row(mark, row, a1 - a0)) {
-                a1 = a0;  // done by split parts
-            } else {
-                c0 = clampll(__ldg(p.Cp + row), 0, p.nnzC);
-                c1 = clampll(__ldg(p.Cp + row + 1), c0, p.nnzC);
-            }
-        }
-        int len = (int)(a1 - a0);
-        if (team) team_share(g, R, a0, len);
-        // first two chunks of A while dC is scattered
-        int k0, k1;
-        float x0, x1;
-        brg_load_a(p, a0 + gl, gl < len, k0, x0);
-        brg_load_a(p, a0 + RG + gl, RG + gl < len, k1, x1);
-        // the row of dC into the dense row, eight entries per lane in flight
-        // (the row is read once, from DRAM: a chain of single loads would
-        // wait out one memory latency per entry)
-        for (long long e = c0 + tl; e < c1; e += 8 * tn) {
-            int cc[8];
-            float vv[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const long long eu = e + u * tn;
-                cc[u] = eu < c1 ? __ldg(p.Ci + eu) : 0;
-                vv[u] = eu < c1 ? __ldg(p.dC + eu) : 0.0f;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                if (e + u * tn < c1) {
-                    if ((unsigned)cc[u] < (unsigned)p.d) gr[cc[u]] = vv[u];
-                    else atomicOr(err, ERR_C_ROW);
-                }
-            }
-        }
-        long long sg;
-        int L;
-        brg_seg(p, k0, gl < len, sg, L, err);
-        __syncwarp();
-        const int lmax = (int)__reduce_max_sync(FULL, (unsigned)len);
-        BrgSeg nxt = brg_seg_of(shfl64(sg, g * RG), __shfl_sync(FULL, L, g * RG), __shfl_sync(FULL, x0, g * RG));
-        int4 nv = make_int4(0, 0, 0, 0);
-        brg_fetch(P4, nxt, gl, nv);
-        for (int e = 0; e < lmax; e += RG) {
-            int k2;
-            float x2;
-            long long ns;
-            int nL;
-            brg_load_a(p, a0 + e + 2 * RG + gl, e + 2 * RG + gl < len, k2, x2);
-            brg_seg(p, k1, e + RG + gl < len, ns, nL, err);
-            const int nu = lmax - e < RG ? lmax - e : RG;
-            float mine = 0.0f;  // dA of entry e + gl of this slot's row
-            for (int u = 0; u < nu; ++u) {
-                const BrgSeg cur = nxt;
-                const int4 cv = nv;
-                long long s2;
-                int L2;
-                float a2;
-                if (u + 1 < nu) {
-                    s2 = shfl64(sg, g * RG + u + 1);
-                    L2 = __shfl_sync(FULL, L, g * RG + u + 1);
-                    a2 = __shfl_sync(FULL, x0, g * RG + u + 1);
-                } else {
-                    s2 = shfl64(ns, g * RG);
-                    L2 = __shfl_sync(FULL, nL, g * RG);
-                    a2 = __shfl_sync(FULL, x1, g * RG);
-                }
-                nxt = brg_seg_of(s2, L2, a2);
-                brg_fetch(P4, nxt, gl, nv);
-                float part = 0.0f;
-                if (2 * gl < cur.span) part = brg_apply(p, cur, gl, cv, gr, err);
-                for (int q = gl + RG; 2 * q < cur.span; q += RG) {
-                    int4 w = make_int4(0, 0, 0, 0);
-                    brg_fetch(P4, cur, q, w);
-                    part += brg_apply(p, cur, q, w, gr, err);
-                }
-#pragma unroll
-                for (int o = RG / 2; o >= 1; o >>= 1) part += __shfl_xor_sync(FULL, part, o, RG);
-                if (gl == u) mine = part;
-            }
-            if (p.dA && e + gl < len) p.dA[a0 + e + gl] = mine;
-            sg = ns;
-            L = nL;
-            x0 = x1;
-            k1 = k2;
-            x1 = x2;
-        }
-        __syncwarp();
-        // clear the whole dense row with 16-byte stores (dpad is a multiple
-        // of 32, rows 16-byte aligned): cheaper than revisiting the row's
-        // entries of C
-        for (int c = 4 * tl; c < p.dpad; c += 4 * tn) *reinterpret_cast<float4*>(gr + c) = make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncwarp();
-    }
+    unsigned un = blockIdx.x * nw + warp;
+    for (; un < lu.nteam; un += gridDim.x * nw) brg_unit<RG, true>(p, fsm, lu.nheavy + un, lu.end);
+    for (; un < lu.units; un += gridDim.x * nw)
+        brg_unit<RG, false>(p, fsm, lu.row_at(un, lane_id() / RG, R), lu.end);
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -495,7 +516,7 @@ __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
 // without the light-row walk the kernel fits six blocks per SM, and more
 // resident warps hide more of its gather latency (300 -> 272 us at scale 20).
 template <int G, bool PACKED, bool HEAVY>
-__global__ void __launch_bounds__(256, HEAVY ? 6 : 5) k_backward(BwdParams p) {
+__global__ void __launch_bounds__(256, HEAVY ? 6 : 4) k_backward(BwdParams p) {
     // a light-row kernel launched behind this one may start on SMs this grid
     // frees (the two handle disjoint rows; dB is only added to atomically)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
