@@ -50,3 +50,26 @@ def test_units(n, d, per_row, copies, tuning):
     rA, bA, rB, bB = oracle.backward(A, B, Cp, Ci, dC.astype(np.float64))
     assert np.all(np.abs(dA.cpu().numpy() - rA) <= REL * bA)
     assert np.all(np.abs(dB.cpu().numpy() - rB) <= REL * bB)
+
+
+@pytest.mark.parametrize("n,d,per_row,copies", [(1100, 513, 6.0, 3), (1100, 1024, 3.0, 1), (1300, 700, 12.0, 2),
+                                                (1500, 2050, 7.0, 1)])
+@pytest.mark.parametrize("tuning", [None, {"cta_min_flops": 1 << 20}, {"warps_per_cta": 1}, {"bwd_group": 1},
+                                    {"pack_b": 2}])
+def test_rows_of_a_whole_warp(n, d, per_row, copies, tuning):
+    test_units(n, d, per_row, copies, tuning)
+
+
+@pytest.mark.parametrize("n,d,per_row,want", [(3000, 64, 4.0, 1024), (3000, 512, 4.6, 2048), (3000, 513, 4.6, 1024),
+                                              (3000, 513, 4.4, 1024), (3000, 513, 9.0, 4096),
+                                              (1 << 20, 513, 4.6, 4096), ((1 << 20) - 1, 513, 4.6, 1024),
+                                              (1 << 20, 512, 4.6, 2048)])
+def test_line_of_the_heavy_rows(n, d, per_row, want):
+    nnz = int(n * per_row + 1)
+    rowptr = np.minimum(np.arange(n + 1, dtype=np.int64) * -(-nnz // n), nnz)
+    lens = np.diff(rowptr)
+    B = CSR(n, d, rowptr, (np.arange(nnz) - np.repeat(rowptr[:-1], lens)).astype(np.int32))
+    B.val = np.ones(nnz, np.float32)
+    A = CSR(n, n, np.zeros(n + 1, np.int64), np.zeros(0, np.int32))
+    A.val = np.zeros(0, np.float32)
+    assert Plan(DeviceCSR.from_host(A), DeviceCSR.from_host(B)).tuning["cta_min_flops"] == want
