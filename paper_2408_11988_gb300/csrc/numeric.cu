@@ -747,9 +747,9 @@ struct LightRows {
 // then light rows (team = warp, in natural row order, pipelined: while row
 // r is walked and read out, the row pointers of B for row r + 1's first
 // chunk, the entries of A of row r + 2 and the bounds of row r + 3 are in
-// flight).  Shared memory per warp: W + 8 floats of accumulator and
-// W/32 + 1 bitmap words (zero between items: every read-out resets what it
-// emitted).
+// flight).  Shared memory per warp: W + 8 floats of accumulator, W/32 + 1
+// bitmap words (zero between items: every read-out resets what it emitted)
+// and WIDE_LIST columns for the read-out.
 __global__ void __launch_bounds__(256, 4) k_numeric_wide(NumParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_item, s_nheavy, s_nrows;
@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(256, 4) k_numeric_wide(NumParams p) {
     __shared__ int s_wcnt[MAX_DENSE_W / 32 + 1];
     const int nwarps = blockDim.x >> 5, warp = warp_id(), lane = lane_id(), tid = threadIdx.x;
     const int ld = p.W + 8, nw = p.W >> 5, bmw = nw + 1;
-    const int per_warp = ld + bmw;  // 4-byte words
+    const int per_warp = ld + bmw + WIDE_LIST / 2;  // 4-byte words
     for (int i = tid; i < nwarps * per_warp; i += blockDim.x) reinterpret_cast<unsigned*>(smem)[i] = 0u;
     if (tid < 32) {  // one warp; its lanes store the same values
         long long nh, nr;
@@ -775,6 +775,7 @@ __global__ void __launch_bounds__(256, 4) k_numeric_wide(NumParams p) {
     // the warps' accumulators column by column
     float* wacc = reinterpret_cast<float*>(smem) + (size_t)warp * per_warp;
     unsigned* wbm = reinterpret_cast<unsigned*>(wacc) + ld;
+    unsigned short* list = reinterpret_cast<unsigned short*>(wbm + bmw);
     const AddShared wadd{wacc, wbm};
     float* acc0 = reinterpret_cast<float*>(smem);  // warp 0's accumulator takes the sum
     unsigned* bm0 = reinterpret_cast<unsigned*>(smem) + ld;
@@ -883,7 +884,7 @@ __global__ void __launch_bounds__(256, 4) k_numeric_wide(NumParams p) {
         wide_chunk_walk(p.Bq, wadd, W, g0, np, ca, r0.len < 32 ? r0.len : 32);
         if (r0.len > 32) wide_range(p, wadd, r0.a0 + 32, r0.a0 + r0.len, 32, err);  // a long light row
         __syncwarp();
-        const int tot = wide_emit(wacc, wbm, nw, out, out_end, p.Ci, p.Cx, 0, 1, err);
+        const int tot = wide_emit_row(wacc, wbm, list, nw, out, out_end, p.Ci, p.Cx, err);
         if (lane == 0 && out + tot != out_end) atomicOr(err, ERR_C_ROW);
         __syncwarp();
         if (lane < nw) wbm[lane] = 0u;
@@ -898,7 +899,7 @@ __global__ void __launch_bounds__(256, 4) k_numeric_wide(NumParams p) {
 }
 
 size_t numeric_wide_smem(int W, int warps) {
-    return (size_t)warps * 4 * (size_t)((W + 8) + (W / 32 + 1));
+    return (size_t)warps * 4 * (size_t)((W + 8) + (W / 32 + 1) + WIDE_LIST / 2);
 }
 
 template <bool VALUES, int G, bool PACKED>
