@@ -4,6 +4,8 @@
 #include <atomic>
 #include <climits>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -229,7 +231,7 @@ __device__ __forceinline__ void split_row(long long i, long long alen, long long
 // running sums come from one load of the histogram and a scan in shared
 // memory, a warp's lane taking 13 classes (as a loop of loads and warp scans
 // they were 10 of the kernel's 14 us for a small product).
-constexpr int SCATTER_ROWS = 8;  // rows per thread
+template <int SCATTER_ROWS>  // rows per thread
 __global__ void __launch_bounds__(256) k_scatter(long long n, long long* flops, int* __restrict__ perm, WsHeader* hdr,
                                                  const long long* __restrict__ Ap, long long nnzA, Sched s,
                                                  long long item_cap) {
@@ -342,16 +344,23 @@ cudaError_t launch_row_flops(const DevCsr& A, const DevCsr& B, const Sched& s, c
     return cudaGetLastError();
 }
 
+// Rows below which a thread of k_scatter takes one row instead of eight: few
+// rows in few blocks wait for the shared-memory ranks of their own block
+// (2^14 rows, the two passes of a product: 49.2 -> 47.2 us).
+constexpr long long SCATTER_FEW = 1LL << 18;
+
 cudaError_t launch_reclassify(long long n, const Sched& s, long long* Cp_next, cudaStream_t st, const DevCsr* A) {
     if (n == 0) return cudaSuccess;
     long long cb = (n + 255) / 256;
     if (cb > 152 * 16) cb = 152 * 16;
     count_launch();
     k_classify<<<(unsigned)cb, 256, 0, st>>>(n, s.flops, Cp_next, s.hdr);
-    const long long sb = (n + 256LL * SCATTER_ROWS - 1) / (256LL * SCATTER_ROWS);
+    const int rows = n < SCATTER_FEW ? 1 : 8;
+    const long long sb = (n + 256LL * rows - 1) / (256LL * rows);
     count_launch();
-    k_scatter<<<(unsigned)sb, 256, 0, st>>>(n, s.flops, s.perm, s.hdr, A ? A->rowptr : nullptr, A ? A->nnz : 0, s,
-                                            A ? split_item_capacity(A->nnz) : 0);
+    const auto scatter = rows == 1 ? k_scatter<1> : k_scatter<8>;
+    scatter<<<(unsigned)sb, 256, 0, st>>>(n, s.flops, s.perm, s.hdr, A ? A->rowptr : nullptr, A ? A->nnz : 0, s,
+                                          A ? split_item_capacity(A->nnz) : 0);
     return cudaGetLastError();
 }
 
@@ -1080,6 +1089,34 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(long long* x, long 
     }
 }
 
+// Up to SCAN_CLUSTER tiles: one launch, a cluster of blocks that exchange their
+// tiles' sums through distributed shared memory (2^14 rows, the two passes of
+// a product: 49.2 us with a launch for the sums, 47.2 so).
+constexpr int SCAN_CLUSTER = 8;
+
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_cluster(long long* x, long long n) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ long long s_sum;
+    const unsigned rank = cl.block_rank();
+    const long long base = (long long)rank * SCAN_TILE + (long long)threadIdx.x * SCAN_PER_THREAD;
+    long long v[SCAN_PER_THREAD];
+    long long run = 0;
+#pragma unroll
+    for (int u = 0; u < SCAN_PER_THREAD; ++u) v[u] = base + u < n ? x[base + u] : 0;
+#pragma unroll
+    for (int u = 0; u < SCAN_PER_THREAD; ++u) v[u] = run += v[u];
+    long long tot;
+    long long ex = block_excl_scan<SCAN_THREADS>(run, tot);
+    if (threadIdx.x == 0) s_sum = tot;
+    cl.sync();
+    for (unsigned r = 0; r < rank; ++r) ex += *cl.map_shared_rank(&s_sum, r);
+#pragma unroll
+    for (int u = 0; u < SCAN_PER_THREAD; ++u)
+        if (base + u < n) x[base + u] = ex + v[u];
+    cl.sync();  // a block's sum stays until every block has read it
+}
+
 // Tiles up to which every block of k_scan_apply sums the tiles before its own
 // (at most four loads a thread) instead of waiting for a kernel of one block.
 constexpr long long SCAN_FEW = 4 * SCAN_THREADS;
@@ -1087,6 +1124,22 @@ constexpr long long SCAN_FEW = 4 * SCAN_THREADS;
 cudaError_t launch_scan_inplace(long long* x, long long n, long long* partial, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const long long nb = (n + SCAN_TILE - 1) / SCAN_TILE;
+    if (nb > 1 && nb <= SCAN_CLUSTER) {
+        const unsigned blocks = nb <= 2 ? 2 : nb <= 4 ? 4 : SCAN_CLUSTER;
+        cudaLaunchConfig_t lc{};
+        lc.gridDim = dim3(blocks);
+        lc.blockDim = dim3(SCAN_THREADS);
+        lc.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = blocks;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+        count_launch();
+        return cudaLaunchKernelEx(&lc, k_scan_cluster, x, n);
+    }
     if (nb > 1) {
         count_launch();
         k_scan_reduce<<<(unsigned)nb, SCAN_THREADS, 0, st>>>(x, n, partial);
