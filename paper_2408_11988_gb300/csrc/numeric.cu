@@ -612,7 +612,7 @@ __device__ __forceinline__ void rgcta_tile(const NumParams& p, const int4* P4, f
 // Split parts, then heavy rows, in row groups (plus-times, padded packed B).
 // Shared memory: S accumulators of W + 8 floats (the slots), then W floats
 // for the summed tile.  Launched ahead of k_numeric_light, which takes the
-// light rows.
+// light rows, and possibly beside k_numeric_tiny: block 0 ends after it.
 template <int RG>
 __global__ void __launch_bounds__(256, 5) k_numeric_rgcta(NumParams p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -622,7 +622,10 @@ __global__ void __launch_bounds__(256, 5) k_numeric_rgcta(NumParams p) {
     __shared__ int s_last;
     constexpr int R = 32 / RG;
     const int tid = threadIdx.x, S = (blockDim.x >> 5) * R, ld = p.W + 8;
-    if (nothing_heavy(p.hdr, p.cta_class)) return;
+    if (nothing_heavy(p.hdr, p.cta_class)) {
+        end_after_kernel_before();
+        return;
+    }
     float* racc = reinterpret_cast<float*>(smem);
     float* sum = racc + (size_t)S * ld;
     for (int i = tid; i < S * ld + p.W; i += blockDim.x) reinterpret_cast<unsigned*>(racc)[i] = RG_EMPTY;
@@ -680,6 +683,7 @@ __global__ void __launch_bounds__(256, 5) k_numeric_rgcta(NumParams p) {
         if (out != out_end && tid == 0) atomicOr(err, ERR_C_ROW);
     }
     if (bad) atomicOr(err, ERR_B_COL);
+    end_after_kernel_before();
 }
 
 // A light row as the pipeline holds it: its row id (-1: none), first entry
@@ -747,7 +751,8 @@ struct LightRows {
 // then light rows (team = warp, in natural row order, pipelined: while row
 // r is walked and read out, the row pointers of B for row r + 1's first
 // chunk, the entries of A of row r + 2 and the bounds of row r + 3 are in
-// flight).  Shared memory per warp: W + 8 floats of accumulator, W/32 + 1
+// flight).  May run beside k_numeric_tiny, which takes other rows: block 0
+// ends after it.  Shared memory per warp: W + 8 floats of accumulator, W/32 + 1
 // bitmap words (zero between items: every read-out resets what it emitted)
 // and WIDE_LIST columns for the read-out.
 __global__ void __launch_bounds__(256, 4) k_numeric_wide(NumParams p) {
@@ -896,6 +901,7 @@ __global__ void __launch_bounds__(256, 4) k_numeric_wide(NumParams p) {
         np = np1;
         ca = ca1;
     }
+    end_after_kernel_before();
 }
 
 size_t numeric_wide_smem(int W, int warps) {
@@ -1065,6 +1071,7 @@ size_t numeric_rgcta_smem(int W, int warps, int rg) {
     return numeric_light_smem(W, warps, rg) + 4 * (size_t)W;  // the slots, then the summed tile
 }
 
+// p.tiny_max: behind k_numeric_tiny.
 template <int RG>
 static cudaError_t launch_rgcta(const NumParams& p, int warps, int sms, cudaStream_t st) {
     const void* k = (const void*)k_numeric_rgcta<RG>;
@@ -1076,6 +1083,7 @@ static cudaError_t launch_rgcta(const NumParams& p, int warps, int sms, cudaStre
         return e;
     const int grid = persistent_grid(k, 32 * warps, smem, sms);
     count_launch();
+    if (p.tiny_max) return launch_beside(k_numeric_rgcta<RG>, grid, 32 * warps, smem, st, p);
     k_numeric_rgcta<RG><<<grid, 32 * warps, smem, st>>>(p);
     return cudaGetLastError();
 }
@@ -1093,8 +1101,7 @@ static cudaError_t launch_wide(NumParams p, int warps, int sms, cudaStream_t st)
         return e;
     const int grid = persistent_grid(k, 32 * warps, smem, sms);
     count_launch();
-    k_numeric_wide<<<grid, 32 * warps, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_beside(k_numeric_wide, grid, 32 * warps, smem, st, p);
 }
 
 template <bool VALUES, int G, bool PACKED>
@@ -1135,18 +1142,9 @@ static cudaError_t launch_light_k(const NumParams& p, int warps, int sms, cudaSt
     if (smem > 48 * 1024 &&
         (e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
         return e;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(persistent_grid(k, 32 * warps, smem, sms));
-    lc.blockDim = dim3(32 * warps);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
+    const int grid = persistent_grid(k, 32 * warps, smem, sms);
     count_launch();
-    return cudaLaunchKernelEx(&lc, k_numeric_light<RG, PADDED>, p);
+    return launch_beside(k_numeric_light<RG, PADDED>, grid, 32 * warps, smem, st, p);
 }
 
 template <int RG>

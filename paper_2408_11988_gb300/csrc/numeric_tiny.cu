@@ -148,6 +148,8 @@ __device__ __forceinline__ void tiny_process(const NumParams& p, const int2* __r
 // rows go through a two-stage pipeline: the next row's gathers are issued
 // before the current row is sorted and written.
 __global__ void __launch_bounds__(256, 4) k_numeric_tiny(NumParams p) {
+    // the kernel for the other rows may start on SMs this grid frees
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = lane_id();
     unsigned long long* err = &p.hdr->err;
     const int2* Q = reinterpret_cast<const int2*>(p.Bq);
