@@ -50,7 +50,6 @@ __global__ void __launch_bounds__(256) k_flops_rows(long long n, const long long
                                                     Seg segB, int nB, long long* __restrict__ flops,
                                                     long long* __restrict__ items, long long item_cap,
                                                     WsHeader* hdr, int rows) {
-    __shared__ long long s_f[256];
     const int lane = lane_id();
     // rows per warp: 32, or fewer where there are too few for every warp
     const long long i = lane < rows ? ((long long)blockIdx.x * 8 + warp_id()) * rows + lane : n;
@@ -64,24 +63,29 @@ __global__ void __launch_bounds__(256) k_flops_rows(long long n, const long long
         if (a1 - a0 <= SHORT_ROW) len = (int)(a1 - a0);
         else nchunks = (a1 - a0 + LONG_CHUNK - 1) / LONG_CHUNK;
     }
-    long long* wf = s_f + (threadIdx.x & ~31);
-    wf[lane] = 0;
-    __syncwarp();
-    // The short rows of the warp's rows hold consecutive entries of A: they
-    // are numbered across the rows and read 32 at a time (coalesced); each
-    // entry's B row length goes to its row by a segmented sum over the lanes
-    // (the row of entry p is the last lane whose first number is <= p).
+    // The short rows of the warp's rows are numbered across the rows and read
+    // 32 entries at a time (coalesced).  Entry p of these is at first + p
+    // where the rows follow each other in A; past a long row its row is the
+    // last lane whose first number is <= p.  A running sum of B's row lengths
+    // over the lanes then gives every row (a lane) its part of the round as a
+    // difference of two places (mod 2^32: at most 32 rows of B of at most d
+    // entries are an int).  Against a segmented sum over each entry's row, us:
+    // 2^14 rows of 8 entries 6.6 -> 4.5, 2^20 rows of 8 entries 47 -> 40, 2^20
+    // rows of an R-MAT graph 70 -> 67 (bound by the gather); four rounds in
+    // flight instead of two gain nothing.
     const int incl = warp_incl_scan(len), excl = incl - len;
     const int total = __shfl_sync(FULL, incl, 31);
     const long long shift = a0 - excl;  // entry of number p in row q: shift(q) + p
-    constexpr int U = 4;  // rounds of 32 entries in flight
+    const long long first = shfl64(a0, 0);
+    const bool follow = __all_sync(FULL, len == 0 || shift == first);
+    constexpr int U = 2;  // rounds of 32 entries in flight
+    long long f = 0;
     for (int p0 = 0; p0 < total; p0 += 32 * U) {
-        int q[U], k[U], v[U];
+        int k[U], v[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int p = p0 + 32 * u + lane;
-            q[u] = owner_lane(excl, p);
-            const long long e = shfl64(shift, q[u]) + p;
+            const long long e = (follow ? first : shfl64(shift, owner_lane(excl, p))) + p;
             k[u] = p < total ? __ldg(Ai + e) : -1;
             if (p < total && (unsigned)k[u] >= (unsigned)nB) atomicOr(err, ERR_A_COL);
         }
@@ -95,21 +99,20 @@ __global__ void __launch_bounds__(256) k_flops_rows(long long n, const long long
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            // sum over this lane's run of equal q, from this lane on (at most
-            // 32 rows of B of at most d entries: an int)
-            int sum = v[u];
+            unsigned run = (unsigned)v[u];
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_down_sync(FULL, sum, o);
-                const int qo = __shfl_down_sync(FULL, q[u], o);
-                if (lane + o < 32 && qo == q[u]) sum += t;
+                const unsigned t = __shfl_up_sync(FULL, run, o);
+                if (lane >= o) run += t;
             }
-            const int qp = __shfl_up_sync(FULL, q[u], 1);
-            if (p0 + 32 * u + lane < total && (lane == 0 || qp != q[u])) wf[q[u]] += sum;  // one lane per row and round
-            __syncwarp();
+            int beg = excl - p0 - 32 * u, end = beg + len;  // this lane's row in the round
+            beg = beg > 0 ? beg : 0;
+            end = end < 32 ? end : 32;
+            const unsigned upto = __shfl_sync(FULL, run, (end - 1) & 31), before = __shfl_sync(FULL, run, (beg - 1) & 31);
+            if (end > beg) f += upto - (beg ? before : 0u);
         }
     }
-    if (i < n) flops[i] = nchunks ? 0 : wf[lane];
+    if (i < n) flops[i] = nchunks ? 0 : f;
     // reserve item slots: one atomic per warp
     long long cincl = warp_incl_scan(nchunks);
     const long long tot = __shfl_sync(FULL, cincl, 31);
