@@ -68,7 +68,11 @@ typedef int32_t ts_status;
 /* Accumulator kinds (paper Sec. III-C: SPA for d <= 1024, hash above). */
 #define TS_ACC_AUTO 0
 #define TS_ACC_DENSE 1   /* shared-memory dense accumulator + occupancy flags   */
-#define TS_ACC_HASH 2    /* shared-memory open-addressing hash accumulator      */
+#define TS_ACC_HASH 2    /* shared-memory open-addressing hash accumulator.
+                          * Chosen automatically (d > 4096) it stands for
+                          * sparse accumulation: up to d = 32768 a row's columns
+                          * are ranked by their bitmap and summed by rank; asked
+                          * for, it is the hash table                           */
 #define TS_ACC_COPIES 3  /* dense accumulator, one private copy per lane group
                           * and no atomics (plus-times; the boolean semiring
                           * uses TS_ACC_DENSE)                                  */
@@ -100,7 +104,10 @@ typedef struct ts_csr_desc {
  *                 concatenation of its tiles (B column tiling).
  *  cta_min_flops  rows with at least this many products (rounded up to the
  *                 next boundary of the row classes, eighths of an octave of
- *                 products) run CTA-per-row; lighter rows warp-per-row.
+ *                 products) run CTA-per-row; lighter rows several a warp, a
+ *                 row's entries shared by the warp's slots where they are many
+ *                 (or one a warp, where d is large).  Automatic: 1024 to 4096,
+ *                 by B's mean row length, d and the number of rows.
  *  warps_per_cta  warps per thread block (1..8).
  *  hash_slots     slots of a warp's hash table (power of two, >= 64).
  *  group          how a warp spreads the products of 32 entries of A over its
@@ -321,7 +328,7 @@ TS_API ts_status msbfs_step(const ts_csr_desc* A, const ts_csr_desc* F, uint32_t
  *   W(r, j) = npos - (npos + nneg) * sigmoid(z_i . z_j)   (i = r0 + r),
  *     npos = [A(i, j) stored], nneg = occurrences of j in the row's s
  *     negative samples neg[r*s .. r*s+s) (device int32, vertex ids);
- *   G = W * Z (this library's plus-times TS-SpGEMM);
+ *   G = W * Z (the plus-times product, each row summed as it is gathered);
  *   U_i = z_i + lr * G_r;  new row i = the k entries of U_i of largest
  *     magnitude (ties: smaller column), ascending columns.
  * Every row of the batch is computed from the old Z; the new rows then
@@ -396,7 +403,8 @@ TS_API ts_status msbfs_emit(const ts_csr_desc* F_next, int64_t F_next_capacity, 
  * another and scheduled together (rows with products at or above their
  * instance's heavy threshold one block each from a list, the others one warp
  * each).  Forward: four launches (row flops with the packed and dense copies
- * of B, row counts, per-instance scan, numeric); backward: two (clear dA/dB,
+ * of B, row counts, scan, numeric), five where an instance may hold a row of
+ * more than 1024 entries (their flops in parts); backward: two (clear dA/dB,
  * gradients).  Every instance has its own tuning in its descriptor: the
  * accumulator (the shared accumulator with occupancy bits over one column
  * tile of d_b padded to 32, or the dense-B form for d_b <= 256) and the

@@ -127,7 +127,9 @@ struct BwdOp {
 };
 
 // dC row i scattered into the dense row g (or cleared again), U entries per
-// thread in flight.
+// thread in flight: four for a warp's light row, where the row of dC comes
+// from DRAM and C's columns are read again to clear; one for a block's row
+// (its registers are capped at 40).
 template <int U>
 __device__ __forceinline__ void scatter_dc(const BwdParams& p, long long c0, long long c1, float* g, bool clear,
                                            int tid, int nthr, unsigned long long* err) {
@@ -515,6 +517,11 @@ __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
 // HEAVY: split parts and heavy rows only (light rows run in k_backward_light);
 // without the light-row walk the kernel fits six blocks per SM, and more
 // resident warps hide more of its gather latency (300 -> 272 us at scale 20).
+// With it the kernel takes 61 registers at four blocks.  At five (48, spilled)
+// and with one load of dC in flight the backward of 2^24 rows, d = 1024, 1%,
+// took 23.8 ms, at five with four in flight 21.5, so 20.4; two or four steps of
+// quads in flight spill and cost 1.1 - 1.6 times, reading B's own arrays instead
+// of the packed copy 1.1 times (more sectors for the same entries).
 template <int G, bool PACKED, bool HEAVY>
 __global__ void __launch_bounds__(256, HEAVY ? 6 : 4) k_backward(BwdParams p) {
     // a light-row kernel launched behind this one may start on SMs this grid
