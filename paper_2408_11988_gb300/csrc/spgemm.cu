@@ -233,9 +233,11 @@ __device__ __forceinline__ void split_row(long long i, long long alen, long long
 // rows of many entries are cut into split items on the way.  The classes'
 // running sums come from one load of the histogram and a scan in shared
 // memory, a warp's lane taking 13 classes (as a loop of loads and warp scans
-// they were 10 of the kernel's 14 us for a small product).
+// they were 10 of the kernel's 14 us for a small product).  Four blocks per SM:
+// left alone the kernel takes 105 registers, two blocks (symbolic call, us:
+// 2^22 rows 1698 -> 1680, 2^24 rows 8555 -> 8487).
 template <int SCATTER_ROWS>  // rows per thread
-__global__ void __launch_bounds__(256) k_scatter(long long n, long long* flops, int* __restrict__ perm, WsHeader* hdr,
+__global__ void __launch_bounds__(256, 4) k_scatter(long long n, long long* flops, int* __restrict__ perm, WsHeader* hdr,
                                                  const long long* __restrict__ Ap, long long nnzA, Sched s,
                                                  long long item_cap) {
     __shared__ unsigned s_cnt[NUM_CLASSES];
