@@ -193,13 +193,16 @@ static bool dense_b_auto(bool vals, long long d, long long nB, long long nnzB) {
 // chain, which a pass over few rows ends by waiting for and one over many
 // hides.  All three passes at 1024 / 2048 / 4096, B rows of 7 entries: 2^16
 // rows, d = 600: 359 / 359 / 445; 2^18, d = 700: 815 / 881 / 858; 2^21,
-// d = 1024: 5653 / 5636 / 5404.
-static long long auto_cta_min_flops(long long d, long long nB, long long nnzB) {
+// d = 1024: 5653 / 5636 / 5404.  That is the wide kernel's (plus-times, one
+// tile); the others' light rows wait less (2^18 rows, boolean, symbolic +
+// numeric, d = 700: 435 / 420 / 416; tiles of 256, d = 1024: 707 / 678 / 681)
+// and change lines at fewer rows.
+static long long auto_cta_min_flops(long long d, long long nB, long long nnzB, bool wide) {
     const double avg = nB > 0 ? (double)nnzB / (double)nB : 0.0;
     if (avg <= 0.0 || avg >= 9.0) return 4096;
     if (avg < 4.5) return 1024;
     if (d <= 512) return 2048;
-    return nB >= (1LL << 20) ? 4096 : 1024;
+    return nB >= (wide ? 1LL << 20 : 1LL << 17) ? 4096 : 1024;
 }
 
 static ts_status resolve_tuning(long long d, const ts_tuning& force, ts_tuning& t,
@@ -210,7 +213,7 @@ static ts_status resolve_tuning(long long d, const ts_tuning& force, ts_tuning& 
                           : (dense_b_auto(vals, d, nB, nnzB) ? TS_ACC_DENSE_B
                                                               : (dpad <= 4096 ? TS_ACC_DENSE : TS_ACC_HASH));
     t.col_tile = force.col_tile ? force.col_tile : (int)std::min<long long>(dpad, 1024);
-    t.cta_min_flops = force.cta_min_flops ? force.cta_min_flops : auto_cta_min_flops(dpad, nB, nnzB);
+    t.cta_min_flops = force.cta_min_flops ? force.cta_min_flops : auto_cta_min_flops(dpad, nB, nnzB, vals && dpad <= 1024 && t.col_tile >= dpad);
     t.warps_per_cta = force.warps_per_cta ? force.warps_per_cta : 8;
     t.hash_slots = force.hash_slots ? force.hash_slots : 1024;
     t.group = force.group ? force.group : auto_group(nB, nnzB, 0);

@@ -13,7 +13,7 @@ from synth import CSR
 
 pytestmark = pytest.mark.gpu
 
-from paper_2408_11988_gb300 import DeviceCSR, Plan
+from paper_2408_11988_gb300 import OR_SELECT2ND, DeviceCSR, Plan
 
 ENTRIES = [0, 1, 2, 3, 4, 5, 7, 8, 9, 15, 16, 17, 31, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 513, 1023, 1025]
 
@@ -60,11 +60,7 @@ def test_rows_of_a_whole_warp(n, d, per_row, copies, tuning):
     test_units(n, d, per_row, copies, tuning)
 
 
-@pytest.mark.parametrize("n,d,per_row,want", [(3000, 64, 4.0, 1024), (3000, 512, 4.6, 2048), (3000, 513, 4.6, 1024),
-                                              (3000, 513, 4.4, 1024), (3000, 513, 9.0, 4096),
-                                              (1 << 20, 513, 4.6, 4096), ((1 << 20) - 1, 513, 4.6, 1024),
-                                              (1 << 20, 512, 4.6, 2048)])
-def test_line_of_the_heavy_rows(n, d, per_row, want):
+def _line(n, d, per_row, **plan):
     nnz = int(n * per_row + 1)
     rowptr = np.minimum(np.arange(n + 1, dtype=np.int64) * -(-nnz // n), nnz)
     lens = np.diff(rowptr)
@@ -72,4 +68,18 @@ def test_line_of_the_heavy_rows(n, d, per_row, want):
     B.val = np.ones(nnz, np.float32)
     A = CSR(n, n, np.zeros(n + 1, np.int64), np.zeros(0, np.int32))
     A.val = np.zeros(0, np.float32)
-    assert Plan(DeviceCSR.from_host(A), DeviceCSR.from_host(B)).tuning["cta_min_flops"] == want
+    return Plan(DeviceCSR.from_host(A), DeviceCSR.from_host(B), **plan).tuning["cta_min_flops"]
+
+
+@pytest.mark.parametrize("n,want", [((1 << 17) - 1, 1024), (1 << 17, 4096)])
+@pytest.mark.parametrize("d,plan", [(600, {"semiring": OR_SELECT2ND}), (600, {"tuning": {"col_tile": 256}}), (1025, {})])
+def test_line_without_the_wide_kernel(n, want, d, plan):
+    assert _line(n, d, 4.6, **plan) == want
+
+
+@pytest.mark.parametrize("n,d,per_row,want", [(3000, 64, 4.0, 1024), (3000, 512, 4.6, 2048), (3000, 513, 4.6, 1024),
+                                              (3000, 513, 4.4, 1024), (3000, 513, 9.0, 4096),
+                                              (1 << 20, 513, 4.6, 4096), ((1 << 20) - 1, 513, 4.6, 1024),
+                                              (1 << 20, 512, 4.6, 2048)])
+def test_line_of_the_heavy_rows(n, d, per_row, want):
+    assert _line(n, d, per_row) == want
