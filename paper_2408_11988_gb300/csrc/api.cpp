@@ -458,7 +458,7 @@ static ts_status read_errors(void* ws, const Layout& L, cudaStream_t st, const c
                     (err & ERR_A_COL) ? "column of A out of range; " : "",
                     (err & ERR_B_COL) ? "column of B out of range; " : "",
                     (err & ERR_C_ROW) ? "C row does not match its rowptr; " : "",
-                    (err & ERR_HASH_FULL) ? "hash table overflow; " : "");
+                    (err & ERR_HASH_FULL) ? "row too wide for its hash table or ranked values; " : "");
     return TS_OK;
 }
 

@@ -32,7 +32,7 @@ inline int class_at_least(long long min_flops) {
 constexpr unsigned long long ERR_A_COL = 1ull;     // column of A outside [0, n)
 constexpr unsigned long long ERR_B_COL = 2ull;     // column of B outside [0, d)
 constexpr unsigned long long ERR_C_ROW = 4ull;     // row of C longer/shorter than its rowptr
-constexpr unsigned long long ERR_HASH_FULL = 8ull; // hash table overflow (row too wide)
+constexpr unsigned long long ERR_HASH_FULL = 8ull; // row too wide for its hash table or its ranked values
 constexpr unsigned long long ERR_CAPACITY = 16ull; // output capacity exceeded
 
 // Rows of A with more than SPLIT_ENTRIES entries are cut into work items of

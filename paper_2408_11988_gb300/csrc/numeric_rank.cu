@@ -188,13 +188,18 @@ struct RankRow {
             return;
         }
         __syncwarp();
-        for (int j = lane; j < total; j += 32) {
+        // the row's class promises at most RANK_WARP products; the columns walked
+        // here can still be more (patterns that changed after the symbolic pass,
+        // row pointers of A that do not ascend), and the values end at RANK_WARP
+        const int held = VALUES && total > RANK_WARP ? RANK_WARP : total;
+        for (int j = lane; j < held; j += 32) {
             if (out + j < out_end) {
                 n.Ci[out + j] = rank_column(bits, pre, p.top, p.dw, j);
                 if (VALUES) n.Cx[out + j] = vals[j];
             }
             if (VALUES) vals[j] = 0.0f;
         }
+        if (lane == 0 && held < total) atomicOr(&n.hdr->err, ERR_HASH_FULL);
         if (lane == 0 && out + total != out_end) atomicOr(&n.hdr->err, ERR_C_ROW);
         __syncwarp();
         for (int w = lane; w < p.dw; w += 32) bits[w] = 0u;
