@@ -283,17 +283,17 @@ __global__ void __launch_bounds__(256) k_f2v_rows(F2vParams p) {
     }
     const long long units = LONG ? min((long long)__ldcg(&ctl->items), p.item_cap) : p.b;
     for (long long x = gw; x < units; x += gws) {
-        const long long r = LONG ? p.ws.items[x] >> 24 : x;
+        const long long r = LONG ? item_row(p.ws.items[x]) : x;
         const long long i = p.r0 + r;
         const long long a0 = clampll(__ldg(p.Ap + i), 0, p.nnzA), a1 = clampll(__ldg(p.Ap + i + 1), a0, p.nnzA);
         const long long len = a1 - a0, terms = len + p.s;
-        const int nch = (int)((terms + F2V_CHUNK - 1) / F2V_CHUNK);
+        const long long nch = (terms + F2V_CHUNK - 1) / F2V_CHUNK;
         if (!LONG && nch > 1) {  // queued; its sum starts empty
             unsigned long long at = 0;
             if (lane == 0) at = atomicAdd(&ctl->items, (unsigned long long)nch);
             at = __shfl_sync(FULL, at, 0);
-            for (int c = lane; c < nch; c += 32) {
-                if ((long long)at + c < p.item_cap) p.ws.items[at + c] = (r << 24) | c;
+            for (long long c = lane; c < nch; c += 32) {
+                if ((long long)at + c < p.item_cap) p.ws.items[at + c] = queue_item(r, c);
                 else atomicOr(&ctl->err, ERR_CAPACITY);
             }
             for (int c = lane; c < p.d; c += 32) p.ws.G[r * p.d + c] = __uint_as_float(F2V_EMPTY);
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(256) k_f2v_rows(F2vParams p) {
         __syncwarp();
         f2v_scatter(p, i, z);
         __syncwarp();
-        const long long t0 = LONG ? (p.ws.items[x] & 0xFFFFFF) * (long long)F2V_CHUNK : 0;
+        const long long t0 = LONG ? item_chunk(p.ws.items[x]) * F2V_CHUNK : 0;
         f2v_terms<KL>(p, r, a0, len, t0, t0 + F2V_CHUNK < terms ? t0 + F2V_CHUNK : terms, z, g);
         __syncwarp();
         if (LONG) {

@@ -41,6 +41,18 @@ constexpr unsigned long long ERR_CAPACITY = 16ull; // output capacity exceeded
 constexpr int SPLIT_ENTRIES = 1024;
 constexpr int MAX_SPLIT_ROWS = 8192;
 
+// Queue items of rows cut into chunks, for queues whose chunks are so short that
+// 24 bits do not number those of the longest row (2^31 - 1 entries): the row in
+// the upper half of the word, the chunk in the lower.
+#ifdef __CUDACC__
+#define TS_BOTH __host__ __device__
+#else
+#define TS_BOTH
+#endif
+TS_BOTH inline long long queue_item(long long row, long long chunk) { return (row << 32) | chunk; }
+TS_BOTH inline long long item_row(long long item) { return item >> 32; }
+TS_BOTH inline long long item_chunk(long long item) { return item & 0xFFFFFFFFll; }
+
 // Workspace header (offset 0 of every workspace).
 struct WsHeader {
     unsigned long long heavy_ctr;     // next heavy row (dynamic CTA scheduling)
