@@ -338,7 +338,8 @@ TS_API ts_status msbfs_step(const ts_csr_desc* A, const ts_csr_desc* F, uint32_t
  * Synchronises `stream`.  Errors: TS_ERR_INVALID_ARG (shapes, batch range,
  * NULL), TS_ERR_UNSUPPORTED (d > 4096, k > d, s > 32, n >= 2^31),
  * TS_ERR_WORKSPACE_TOO_SMALL, TS_ERR_BAD_CSR (device checks: columns out of
- * range, Z not k entries per row), TS_ERR_CUDA.
+ * range, Z not k entries per row, row pointers of A that do not ascend; Z is
+ * left as it was), TS_ERR_CUDA.
  */
 TS_API ts_status f2v_workspace_size(int64_t n, int64_t d, int64_t nnz_A, int64_t b, int32_t s, int32_t k,
                                     size_t* bytes);

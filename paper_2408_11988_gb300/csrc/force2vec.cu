@@ -327,8 +327,12 @@ __global__ void __launch_bounds__(256) k_f2v_rows(F2vParams p) {
     }
 }
 
+// The staged rows into Z, unless a check failed: then some of them may not have
+// been finished, and Z stays as it was.
 __global__ void __launch_bounds__(256) k_f2v_commit(long long r0, long long b, int k, const int* __restrict__ Sc,
-                                                    const float* __restrict__ Sv, int* Zc, float* Zv) {
+                                                    const float* __restrict__ Sv, int* Zc, float* Zv,
+                                                    const F2vCtl* ctl) {
+    if (__ldg(&ctl->err)) return;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < b * k;
          t += (long long)gridDim.x * blockDim.x) {
         Zc[r0 * k + t] = Sc[t];
@@ -392,7 +396,7 @@ cudaError_t launch_f2v_step(const DevCsr& A, const DevCsr& Z, int k, long long r
     if (blocks > 152 * 16) blocks = 152 * 16;
     count_launch();
     k_f2v_commit<<<(unsigned)blocks, 256, 0, st>>>(r0, b, k, p.ws.Sc, p.ws.Sv, const_cast<int*>(Z.col),
-                                                   const_cast<float*>(Z.val));
+                                                   const_cast<float*>(Z.val), p.ws.ctl);
     return cudaGetLastError();
 }
 
