@@ -331,7 +331,8 @@ TS_API ts_status msbfs_step(const ts_csr_desc* A, const ts_csr_desc* F, uint32_t
  *   G = W * Z (the plus-times product, each row summed as it is gathered);
  *   U_i = z_i + lr * G_r;  new row i = the k entries of U_i of largest
  *     magnitude (ties: smaller column), ascending columns.
- * Every row of the batch is computed from the old Z; the new rows then
+ * The sums are taken in an order that the arguments fix: the same step gives
+ * the same bits.  Every row of the batch is computed from the old Z; the new rows then
  * overwrite Z's batch rows in place (Z.col and Z.val are written).  U_out:
  * optional device float32[b*d] receiving the dense U before sparsification
  * (NULL: not written).  ws: f2v_workspace_size bytes, 256-byte aligned.

@@ -262,7 +262,8 @@ cudaError_t launch_batch_bounds(const InstDesc* inst, int count, const long long
 
 // Sparse Force2Vec step (force2vec.cu): the new rows computed, then written
 // into Z's batch rows.  ws: f2v_bytes, 256-byte aligned, beginning with an
-// F2vCtl that the step clears.
+// F2vCtl that the step clears.  Rows are summed in an order that b, d and the
+// rows' lengths fix.
 struct F2vCtl {
     unsigned long long err;    // ERR_* bits
     unsigned long long items;  // chunks of long rows queued
