@@ -154,10 +154,13 @@ __device__ __forceinline__ long long bat_sum_entries(const InstDesc& I, long lon
 }
 
 // The queued parts of long rows: (row, part), a warp each.  The row's products
-// are added up in flops; parts finished are counted above bit 44 of it (a row
-// has at most 2^31 entries of at most 1024 products), and the last part leaves
-// the sum alone and lists the row if it is heavy.
-constexpr int LONG_SHIFT = 44;
+// are added up in flops; parts finished are counted above bit 42 of it, and the
+// last part leaves the sum alone and lists the row if it is heavy.  A row has
+// fewer than 2^31 entries of at most 1024 products: the sum stays below 2^41 and
+// the parts are at most 2^21.
+constexpr int LONG_SHIFT = 42;
+static_assert((1ull << 31) * 1024 < (1ull << LONG_SHIFT) && (1ull << 31) / PREP_LONG < (1ull << (64 - LONG_SHIFT)),
+              "the longest row's parts and products fit the word");
 __global__ void __launch_bounds__(256) k_bat_long(const InstDesc* __restrict__ inst, int count,
                                                   unsigned long long* flops, const long long* __restrict__ items,
                                                   long long item_cap, int* __restrict__ heavy, BatchCtl* ctl) {

@@ -60,3 +60,16 @@ def test_queue_items_round_trip(tmp_path):
     out = subprocess.run([str(exe)], input="\n".join("%d %d" % p for p in pairs), capture_output=True, text=True,
                          check=True).stdout.split("\n")
     assert [tuple(map(int, x.split())) for x in out if x] == [(1, r, c) for r, c in pairs]
+
+
+def test_batched_long_rows_count_their_parts():
+    # one 64-bit word per row: the products added so far below bit LONG_SHIFT,
+    # the parts finished above it; neither may run into the other or out of the
+    # word for the longest row over rows of B of 1024 entries
+    text = source("batched.cu")
+    part, shift = constant("PREP_LONG", text), constant("LONG_SHIFT", text)
+    parts, products = -(-LONGEST // part), LONGEST * 1024
+    assert products < 2**shift
+    word = (parts << shift) + products
+    assert word < 2**64
+    assert (word >> shift, word & (2**shift - 1)) == (parts, products)
