@@ -1054,7 +1054,7 @@ extern "C" ts_status msbfs_search(const ts_csr_desc* A, int64_t d, const int32_t
     if (d < 1 || !sources_dev || !levels || start < 0 || max_steps < 0 || !steps || (max_steps > 0 && !frontier_nnz))
         return fail(TS_ERR_INVALID_ARG, "%s: NULL or negative argument", fn);
     if (d > 256) return fail(TS_ERR_UNSUPPORTED, "%s: d above 256", fn);
-    if (start + max_steps > INT32_MAX) return fail(TS_ERR_OVERFLOW, "%s: levels are 32-bit", fn);
+    if (start > INT32_MAX || max_steps > INT32_MAX - start) return fail(TS_ERR_OVERFLOW, "%s: levels are 32-bit", fn);
     const size_t need = msbfs_search_bytes(A->nrows, A->nnz, (int)d);
     if (!ws || ws_bytes < need)
         return fail(TS_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes, %zu needed", fn, ws_bytes, need);
