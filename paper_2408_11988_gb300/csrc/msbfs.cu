@@ -1026,6 +1026,8 @@ cudaError_t launch_msbfs_search(const DevCsr& A, int d, const int* src, int* lev
                 n, A.rowptr, A.col, A.nnz, &w.ctl->err);
         }
         if ((e = cudaGetLastError())) return e;
+        // no level follows that the call would wait for: the caller may free ws
+        if (max_steps == 0) return cudaStreamSynchronize(st);
     }
     BfsParams p = {};
     p.Ap = A.rowptr;
