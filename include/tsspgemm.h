@@ -68,11 +68,13 @@ typedef int32_t ts_status;
 /* Accumulator kinds (paper Sec. III-C: SPA for d <= 1024, hash above). */
 #define TS_ACC_AUTO 0
 #define TS_ACC_DENSE 1   /* shared-memory dense accumulator + occupancy flags   */
-#define TS_ACC_HASH 2    /* shared-memory open-addressing hash accumulator.
-                          * Chosen automatically (d > 4096) it stands for
-                          * sparse accumulation: up to d = 32768 a row's columns
-                          * are ranked by their bitmap and summed by rank; asked
-                          * for, it is the hash table                           */
+#define TS_ACC_HASH 2    /* shared-memory open-addressing hash accumulator, or
+                          * (hash_slots = TS_HASH_RANKED) a row's columns ranked
+                          * by their bitmap and summed by rank, without a table.
+                          * Chosen automatically for d > 4096: ranked up to
+                          * d = 32768, hashed above.  Asked for without
+                          * hash_slots, it is the hash table                    */
+#define TS_HASH_RANKED (-1)
 #define TS_ACC_COPIES 3  /* dense accumulator, one private copy per lane group
                           * and no atomics (plus-times; the boolean semiring
                           * uses TS_ACC_DENSE)                                  */
@@ -109,7 +111,10 @@ typedef struct ts_csr_desc {
  *                 (or one a warp, where d is large).  Automatic: 1024 to 4096,
  *                 by B's mean row length, d and the number of rows.
  *  warps_per_cta  warps per thread block (1..8).
- *  hash_slots     slots of a warp's hash table (power of two, >= 64).
+ *  hash_slots     TS_ACC_HASH: slots of a warp's hash table (power of two, 64 to
+ *                 8192), or TS_HASH_RANKED (4096 < d <= 32768; for any other d
+ *                 it is the default table of 1024).  A plan that ranks reports
+ *                 TS_HASH_RANKED, so that its tuning makes the same plan again.
  *  group          how a warp spreads the products of 32 entries of A over its
  *                 lanes: 1 = one product per lane across entries (any mix of
  *                 B row lengths); 4, 8, 16 or 32 = that many lanes walk one

@@ -31,6 +31,7 @@ ACC_DENSE = 1
 ACC_HASH = 2
 ACC_COPIES = 3
 ACC_DENSE_B = 4
+HASH_RANKED = -1  # hash_slots of a plan that ranks a row's columns
 
 
 class CsrDesc(ctypes.Structure):

@@ -215,7 +215,11 @@ static ts_status resolve_tuning(long long d, const ts_tuning& force, ts_tuning& 
     t.col_tile = force.col_tile ? force.col_tile : (int)std::min<long long>(dpad, 1024);
     t.cta_min_flops = force.cta_min_flops ? force.cta_min_flops : auto_cta_min_flops(dpad, nB, nnzB, vals && dpad <= 1024 && t.col_tile >= dpad);
     t.warps_per_cta = force.warps_per_cta ? force.warps_per_cta : 8;
-    t.hash_slots = force.hash_slots ? force.hash_slots : 1024;
+    // ranked columns where they fit, unless a hash table is asked for (by its
+    // kind or its size); a reported TS_HASH_RANKED asks for them again
+    const bool rank = t.accum == TS_ACC_HASH && numeric_rank_fits(d) &&
+                      (force.hash_slots ? force.hash_slots == TS_HASH_RANKED : !force.accum);
+    t.hash_slots = rank ? TS_HASH_RANKED : force.hash_slots && force.hash_slots != TS_HASH_RANKED ? force.hash_slots : 1024;
     t.group = force.group ? force.group : auto_group(nB, nnzB, 0);
     t.sym_group = force.sym_group ? force.sym_group : auto_group(nB, nnzB, 1);
     t.bwd_group = force.bwd_group ? force.bwd_group : auto_group(nB, nnzB, 2);
@@ -260,8 +264,8 @@ static ts_status resolve_tuning(long long d, const ts_tuning& force, ts_tuning& 
     if (t.cta_min_flops < 1) return fail(TS_ERR_INVALID_ARG, "tuning: cta_min_flops must be >= 1");
     if (t.warps_per_cta < 1 || t.warps_per_cta > 8)
         return fail(TS_ERR_INVALID_ARG, "tuning: warps_per_cta must be in [1, 8]");
-    if (t.hash_slots < 64 || (t.hash_slots & (t.hash_slots - 1)) || t.hash_slots > 8192)
-        return fail(TS_ERR_INVALID_ARG, "tuning: hash_slots must be a power of two in [64, 8192]");
+    if (!rank && (t.hash_slots < 64 || (t.hash_slots & (t.hash_slots - 1)) || t.hash_slots > 8192))
+        return fail(TS_ERR_INVALID_ARG, "tuning: hash_slots must be a power of two in [64, 8192], or TS_HASH_RANKED");
     return TS_OK;
 }
 
@@ -577,8 +581,7 @@ static ts_status run_numeric(ts_plan* plan, const ts_csr_desc* A, const ts_csr_d
                                          (const long long*)C->rowptr, C->col, (float*)C->val, C->nnz, st, bq),
                     fn);
         }
-    } else if (plan->force.accum != TS_ACC_HASH && numeric_rank_fits(plan->d)) {
-        // the hash accumulator chosen, not asked for: ranked columns where they fit
+    } else if (plan->cur.hash_slots == TS_HASH_RANKED) {
         TS_CUDA(launch_numeric_rank(dA, dB, plan->d, vals, sc, cfg, (const long long*)C->rowptr, C->col,
                                     (float*)C->val, C->nnz, st),
                 fn);
@@ -769,6 +772,12 @@ extern "C" ts_status ts_plan_autotune(ts_plan* plan, const ts_csr_desc* A, const
                     if (acc == TS_ACC_COPIES && (!vals || dpad > 4096)) continue;
                     if (acc == TS_ACC_DENSE_B && (!vals || dpad > 256)) continue;
                     c.accum = acc;
+                    c.hash_slots = best.hash_slots;
+                    if (acc == TS_ACC_HASH && !plan->force.hash_slots && numeric_rank_fits(plan->d)) {
+                        c.hash_slots = TS_HASH_RANKED;
+                        cands.push_back(c);
+                        c.hash_slots = 1024;
+                    }
                     cands.push_back(c);
                 }
                 break;
