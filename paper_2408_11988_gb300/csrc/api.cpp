@@ -1329,8 +1329,8 @@ static ts_status bat_forward(ts_batched_plan* plan, char* w, const BLayout& L, i
     TS_CUDA(launch_bat_prepare(inst, nb, c0, c1, flops, heavy, ctl, (long long*)(w + L.items), L.item_cap, sms, st), fn);
     if (!numeric) return TS_OK;
     TS_CUDA(launch_bat_symbolic(inst, nb, c0, c1, 0, flops, heavy, ctl, part, plan->Wmax, sms, st), fn);
-    TS_CUDA(launch_bat_scan(inst, nb, *std::max_element(plan->n.begin() + b0, plan->n.begin() + b0 + nb), ctl, part, st),
-            fn);
+    const int last = b0 + nb - 1;
+    TS_CUDA(launch_bat_scan(inst, nb, bat_tile_span(c0, plan->chunk_off[last], nb, plan->n[last]), ctl, part, st), fn);
     TS_CUDA(launch_bat_numeric(inst, nb, c0, c1, bat_vals(plan) ? 1 : 0, flops, heavy, ctl, plan->Wmax, sms, st),
             fn);
     return TS_OK;

@@ -89,11 +89,10 @@ struct BatUnits {
     }
 };
 
-// Sums of C's row counts over 4096 rows of an instance, for the scan: where row
-// i of instance b keeps its sum.
-constexpr int BAT_TILE = 4096;
+// Sums of C's row counts over BAT_TILE rows of an instance, for the scan: where
+// row i of instance b keeps its sum.
 __device__ __forceinline__ long long bat_tile(const InstDesc& I, int b, long long i) {
-    return (I.chunk_off >> 7) + b + i / BAT_TILE;  // instances' tiles do not meet: 128 chunks a tile, one spare each
+    return bat_first_tile(I.chunk_off, b) + i / BAT_TILE;
 }
 
 // This warp's next unit from queue q: units are dealt c0, c0 + 1,
@@ -555,18 +554,23 @@ __global__ void __launch_bounds__(256) k_bat_symbolic(const InstDesc* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// scan: a block of 1024 threads per BAT_TILE rows of an instance, `tiles` blocks
-// for each (as many as the largest needs), in place over C_b.rowptr, from the sums of the tiles before it (one block per
-// instance took 168 us for 200,000 rows)
+// scan: a block of 1024 threads per tile of BAT_TILE rows, in place over
+// C_b.rowptr, from the sums of the tiles before it (one block per instance took
+// 168 us for 200,000 rows; as many blocks for every instance as the largest
+// needs are mostly empty where one is much larger than the others: a graph of
+// 300,000 rows beside 3,000 of 50 had 222,000 blocks, 3,100 now: forward 1020 ->
+// 408 us)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_bat_scan(const InstDesc* __restrict__ inst, BatchCtl* ctl,
-                                                   const unsigned long long* __restrict__ part, unsigned tiles) {
+__global__ void __launch_bounds__(1024) k_bat_scan(const InstDesc* __restrict__ inst, int count, BatchCtl* ctl,
+                                                   const unsigned long long* __restrict__ part) {
     __shared__ long long s_w[32];
     __shared__ long long s_before[32];
-    const int b = (int)(blockIdx.x / tiles), tile = (int)(blockIdx.x - b * tiles);
+    const long long at = bat_first_tile(__ldg(&inst[0].chunk_off), 0) + blockIdx.x;
+    const int b = bat_inst_of_tile([&](int k) { return __ldg(&inst[k].chunk_off); }, count, at);
     const InstDesc& I = inst[b];
+    const int tile = (int)(at - bat_first_tile(I.chunk_off, b));
     const long long t0 = (long long)tile * BAT_TILE;
-    if (t0 >= I.n && t0 > 0) return;
+    if (t0 >= I.n && t0 > 0) return;  // an instance's spare tile
     long long* rp = I.C_rowptr;
     const int tid = threadIdx.x, lane = lane_id(), warp = warp_id();
     if (t0 == 0 && tid == 0) rp[0] = 0;
@@ -1122,15 +1126,14 @@ cudaError_t launch_bat_symbolic(const InstDesc* inst, int count, long long c0, l
 
 long long bat_long_capacity(long long annz) { return annz > PREP_LONG ? 2 * (annz / PREP_LONG) : 0; }
 
-long long bat_tiles(long long chunks, int count) { return chunks / 128 + count + 1; }
+long long bat_tiles(long long chunks, int count) { return bat_first_tile(chunks, count) + 1; }
 
-cudaError_t launch_bat_scan(const InstDesc* inst, int count, long long max_rows, BatchCtl* ctl,
+cudaError_t launch_bat_scan(const InstDesc* inst, int count, long long tiles, BatchCtl* ctl,
                             const unsigned long long* part, cudaStream_t st) {
     if (count < 1) return cudaSuccess;
-    const long long tiles = max_rows > BAT_TILE ? (max_rows + BAT_TILE - 1) / BAT_TILE : 1;
-    if (tiles * count > INT_MAX) return cudaErrorInvalidValue;
+    if (tiles > INT_MAX) return cudaErrorInvalidValue;  // 2^43 rows
     count_launch();
-    k_bat_scan<<<(unsigned)(tiles * count), 1024, 0, st>>>(inst, ctl, part, (unsigned)tiles);
+    k_bat_scan<<<(unsigned)tiles, 1024, 0, st>>>(inst, count, ctl, part);
     return cudaGetLastError();
 }
 

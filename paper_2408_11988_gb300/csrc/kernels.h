@@ -249,7 +249,8 @@ cudaError_t launch_bat_symbolic(const InstDesc* inst, int count, long long c0, l
 // part: bat_tiles(chunks of the whole batch, count) sums, cleared before the
 // symbolic pass, which fills them for the scan.
 long long bat_tiles(long long chunks, int count);
-cudaError_t launch_bat_scan(const InstDesc* inst, int count, long long max_rows, BatchCtl* ctl,
+// tiles: bat_tile_span of these instances.
+cudaError_t launch_bat_scan(const InstDesc* inst, int count, long long tiles, BatchCtl* ctl,
                             const unsigned long long* part, cudaStream_t st);
 cudaError_t launch_bat_numeric(const InstDesc* inst, int count, long long c0, long long c1, long long values,
                                const long long* flops, const int* heavy, BatchCtl* ctl, int Wmax, int sms,
