@@ -517,13 +517,18 @@ __global__ void __launch_bounds__(256, 5) k_backward_light(BwdParams p) {
 // HEAVY: split parts and heavy rows only (light rows run in k_backward_light);
 // without the light-row walk the kernel fits six blocks per SM, and more
 // resident warps hide more of its gather latency (300 -> 272 us at scale 20).
-// With it the kernel takes 61 registers at four blocks.  At five (48, spilled)
-// and with one load of dC in flight the backward of 2^24 rows, d = 1024, 1%,
-// took 23.8 ms, at five with four in flight 21.5, so 20.4; two or four steps of
-// quads in flight spill and cost 1.1 - 1.6 times, reading B's own arrays instead
-// of the packed copy 1.1 times (more sectors for the same entries).
-template <int G, bool PACKED, bool HEAVY>
-__global__ void __launch_bounds__(256, HEAVY ? 6 : 4) k_backward(BwdParams p) {
+// With it the kernel runs four blocks (quads: 61 registers) or five (48).  Quads
+// and the groups of 1 and 4 spill at five: the backward of 2^24 rows, d = 1024, 1%,
+// took 23.8 ms with one load of dC in flight, at five with four in flight 21.5, so
+// 20.4; two or four steps of quads in flight spill and cost 1.1 - 1.6 times, reading
+// B's own arrays instead of the packed copy 1.1 times (more sectors for the same
+// entries).  Groups of 8, 16 and 32 spill little (56 bytes) and hide more at five
+// where shared memory leaves room for them (bwd_kernel), us, four / five: 2^20 rows, d =
+// 1024, 16 lanes 1374 / 1247; d = 128 on B's own arrays 1400 / 1259 (1364 with one
+// load of dC in flight); where it does not, 48 registers only cost: 2^18 rows, d =
+// 4096, 16 lanes 1769 / 1879.
+template <int G, bool PACKED, bool HEAVY, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS) k_backward(BwdParams p) {
     // a light-row kernel launched behind this one may start on SMs this grid
     // frees (the two handle disjoint rows; dB is only added to atomically)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -689,9 +694,13 @@ size_t backward_smem(long long d, int warps) {
     return sizeof(float) * (size_t)warps * (size_t)(dpad + 32);
 }
 
+// smem: dynamic shared memory of a block.
 template <int G, bool PACKED>
-static const void* bwd_kernel(bool heavy_only) {
-    return heavy_only ? (const void*)k_backward<G, PACKED, true> : (const void*)k_backward<G, PACKED, false>;
+static const void* bwd_kernel(bool heavy_only, size_t smem) {
+    if (heavy_only) return (const void*)k_backward<G, PACKED, true, 6>;
+    if constexpr (G >= 8)  // five blocks beside what each takes for itself
+        if (5 * (smem + 2048) <= 228 * 1024) return (const void*)k_backward<G, PACKED, false, 5>;
+    return (const void*)k_backward<G, PACKED, false, 4>;
 }
 
 cudaError_t launch_backward(const DevCsr& A, const DevCsr& B, long long d, const long long* Cp,
@@ -759,13 +768,13 @@ cudaError_t launch_backward(const DevCsr& A, const DevCsr& B, long long d, const
     switch (cfg.group) {
         case 2:  // quads: packed B and a 16-byte aligned dB only
             if (!pk || (dB && (reinterpret_cast<uintptr_t>(dB) & 15))) return cudaErrorInvalidValue;
-            k = bwd_kernel<2, true>(rg);
+            k = bwd_kernel<2, true>(rg, smem);
             break;
-        case 1: k = pk ? bwd_kernel<1, true>(rg) : bwd_kernel<1, false>(rg); break;
-        case 4: k = pk ? bwd_kernel<4, true>(rg) : bwd_kernel<4, false>(rg); break;
-        case 8: k = pk ? bwd_kernel<8, true>(rg) : bwd_kernel<8, false>(rg); break;
-        case 16: k = pk ? bwd_kernel<16, true>(rg) : bwd_kernel<16, false>(rg); break;
-        case 32: k = pk ? bwd_kernel<32, true>(rg) : bwd_kernel<32, false>(rg); break;
+        case 1: k = pk ? bwd_kernel<1, true>(rg, smem) : bwd_kernel<1, false>(rg, smem); break;
+        case 4: k = pk ? bwd_kernel<4, true>(rg, smem) : bwd_kernel<4, false>(rg, smem); break;
+        case 8: k = pk ? bwd_kernel<8, true>(rg, smem) : bwd_kernel<8, false>(rg, smem); break;
+        case 16: k = pk ? bwd_kernel<16, true>(rg, smem) : bwd_kernel<16, false>(rg, smem); break;
+        case 32: k = pk ? bwd_kernel<32, true>(rg, smem) : bwd_kernel<32, false>(rg, smem); break;
         default: return cudaErrorInvalidValue;
     }
     if (smem > 48 * 1024 &&
