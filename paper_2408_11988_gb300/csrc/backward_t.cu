@@ -56,8 +56,10 @@ __device__ __forceinline__ long long row_holding(const long long* __restrict__ A
     return lo;
 }
 
-// row_of[e] = row of entry e: a warp per ROW_TILE entries (a warp per row left
-// the longest row as a tail: 43 us for 500,009 rows).
+// row_of[e] = row of entry e, or -1 for an entry of no row (before the first
+// row pointer or behind the last: A's arrays may hold more than its rows do): a
+// warp per ROW_TILE entries (a warp per row left the longest row as a tail: 43 us
+// for 500,009 rows).
 __global__ void __launch_bounds__(256) k_row_of(long long n, const long long* __restrict__ Ap, long long nnzA,
                                                 int* __restrict__ row_of) {
     const int lane = lane_id();
@@ -65,8 +67,9 @@ __global__ void __launch_bounds__(256) k_row_of(long long n, const long long* __
     if (e0 >= nnzA) return;
     const long long e1 = e0 + ROW_TILE < nnzA ? e0 + ROW_TILE : nnzA;
     long long r = row_holding(Ap, n, e0), e = e0;
-    while (e < e1) {
-        // rows r .. r + 31: lane l holds the end of row r + l
+    for (; e < e1 && r < n; r += 32) {
+        // rows r .. r + 31: lane l holds the bounds of row r + l
+        const long long beg = r + lane < n ? clampll(__ldg(Ap + r + lane), 0, nnzA) : nnzA;
         const long long end = r + lane < n ? clampll(__ldg(Ap + r + lane + 1), 0, nnzA) : nnzA;
         const long long upto = shfl64(end, 31) < e1 ? shfl64(end, 31) : e1;
         for (long long x = e + lane; x - lane < upto; x += 32) {
@@ -74,12 +77,12 @@ __global__ void __launch_bounds__(256) k_row_of(long long n, const long long* __
 #pragma unroll
             for (int s = 16; s >= 1; s >>= 1)
                 if (shfl64(end, q + s - 1) <= x) q += s;
-            if (x < upto) row_of[x] = (int)(r + q < n ? r + q : n - 1);
+            const long long starts = shfl64(beg, q);
+            if (x < upto) row_of[x] = r + q < n && starts <= x ? (int)(r + q) : -1;
         }
         if (upto > e) e = upto;
-        r += 32;
-        if (r >= n) break;
     }
+    for (long long x = e + lane; x < e1; x += 32) row_of[x] = -1;
 }
 
 // Per tile of RS_TILE keys, the count of each digit: cnt[digit * nb + tile].
