@@ -449,18 +449,39 @@ __global__ void __launch_bounds__(PULL_T_THREADS) k_t_pull(TParams p) {
 
 static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
+// Layout of the workspace.
+struct TWs {
+    int *row_of, *k0, *k1, *v0, *v1;
+    long long* cnt;      // the sort's counters, then the long columns' items
+    size_t cnt_bytes;
+    long long* spart;    // their scan's partial sums
+    long long* ATp;
+    float* part;         // the long columns' sums: every row of B once and one more row per full chunk
+    long long part_cap;
+};
+
+static size_t t_ws(char* base, long long n, long long nnzA, long long nnzB, long long d, TWs* out) {
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* p = base + off;
+        off += al256(bytes);
+        return p;
+    };
+    TWs w;
+    for (int** a : {&w.row_of, &w.k0, &w.k1, &w.v0, &w.v1}) *a = (int*)take(sizeof(int) * (size_t)nnzA);
+    const size_t counts = (size_t)((nnzA + RS_TILE - 1) / RS_TILE) << RS_BITS;
+    w.cnt_bytes = sizeof(long long) * counts;
+    w.cnt = (long long*)take(w.cnt_bytes);
+    w.spart = (long long*)take(sizeof(long long) * scan_partial_count((long long)counts));
+    w.ATp = (long long*)take(sizeof(long long) * (size_t)(n + 1));
+    w.part_cap = nnzB + d * (nnzA / TCH + 1);
+    w.part = (float*)take(sizeof(float) * (size_t)w.part_cap);
+    if (out) *out = w;
+    return off;
+}
+
 size_t backward_t_bytes(long long n, long long nnzA, long long nnzB, long long d) {
-    const long long nb = (nnzA + 2047) / 2048;
-    const long long hist = 256 * nb;
-    size_t s = 0;
-    s += al256(sizeof(int) * (size_t)nnzA) * 5;                 // row_of, keys x2, vals x2
-    s += al256(sizeof(long long) * (size_t)(hist + 1));          // radix counts, then the long columns' items
-    s += al256(sizeof(long long) * (size_t)((hist + 4095) / 4096 + 2));  // scan partials
-    s += al256(sizeof(long long) * (size_t)(n + 1)) * 3;         // ATp, and room kept
-    s += al256(sizeof(long long) * (size_t)((n + 1 + 4095) / 4096 + 2));
-    // partial sums: every row of B once plus one more row per full chunk
-    s += al256(sizeof(float) * (size_t)(nnzB + (long long)d * (nnzA / TCH + 1)));
-    return s;
+    return t_ws(nullptr, n, nnzA, nnzB, d, nullptr);
 }
 
 template <class Places>
@@ -492,51 +513,28 @@ cudaError_t launch_backward_t(const DevCsr& A, const DevCsr& B, long long d, con
     const long long n = A.nrows, m = A.nnz;
     if (!dB || B.nnz == 0) return cudaSuccess;
     if (m == 0) return cudaMemsetAsync(dB, 0, sizeof(float) * B.nnz, st);
-    char* w = (char*)ws;
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        char* p = w + off;
-        off += al256(bytes);
-        return p;
-    };
     const long long nb = (m + RS_TILE - 1) / RS_TILE;
-    const size_t cnt_bytes = sizeof(long long) * (size_t)(256 * ((m + 2047) / 2048) + 1);  // >= 1024 nb counts
-    int* row_of = (int*)take(sizeof(int) * m);
-    int* k0 = (int*)take(sizeof(int) * m);
-    int* k1 = (int*)take(sizeof(int) * m);
-    int* v0 = (int*)take(sizeof(int) * m);
-    int* v1 = (int*)take(sizeof(int) * m);
-    long long* cnt = (long long*)take(cnt_bytes);
-    const size_t npart = (cnt_bytes / sizeof(long long) - 1 + 4095) / 4096 + 2;
-    long long* spart = (long long*)take(sizeof(long long) * npart);
-    long long* ATp = (long long*)take(sizeof(long long) * (n + 1));
-    take(sizeof(long long) * (n + 1));
-    take(sizeof(long long) * (n + 1));
-    take(sizeof(long long) * ((n + 1 + 4095) / 4096 + 2));
-    const long long part_cap = B.nnz + d * (m / TCH + 1);
-    float* part = (float*)take(sizeof(float) * part_cap);
+    TWs w;
+    t_ws((char*)ws, n, m, B.nnz, d, &w);
     const unsigned g256 = (unsigned)std::min<long long>((m + 256) / 256, 152LL * 16);
     count_launch();
-    k_row_of<<<(unsigned)((m + 8LL * ROW_TILE - 1) / (8LL * ROW_TILE)), 256, 0, st>>>(n, A.rowptr, m, row_of);
+    k_row_of<<<(unsigned)((m + 8LL * ROW_TILE - 1) / (8LL * ROW_TILE)), 256, 0, st>>>(n, A.rowptr, m, w.row_of);
     int bits = 1;
     while ((1LL << bits) < n) ++bits;
-    // passes of equal digits, of at most RS_BITS bits, and no more digits than
-    // the counters have room for
-    int most = RS_BITS;
-    while (most > 8 && (size_t)nb << most > cnt_bytes / sizeof(long long) - 1) --most;
-    const int passes = (bits + most - 1) / most, width = (bits + passes - 1) / passes;
+    // passes of equal digits, of at most RS_BITS bits
+    const int passes = (bits + RS_BITS - 1) / RS_BITS, width = (bits + passes - 1) / passes;
     const size_t smem = sizeof(int) * (size_t)std::max(RS_STAGE, RS_WARPS << width);
     if ((e = cudaFuncSetAttribute((const void*)k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
         return e;
     const int *kin = A.col, *vin = nullptr;
-    int *kout = k0, *vout = v0, *kalt = k1, *valt = v1;
+    int *kout = w.k0, *vout = w.v0, *kalt = w.k1, *valt = w.v1;
     for (int shift = 0; shift < bits; shift += width) {
         const int nd = 1 << (bits - shift < width ? bits - shift : width);
         count_launch();
-        k_rs_count<<<(unsigned)nb, RS_THREADS, 0, st>>>(kin, m, shift, nd, cnt, nb);
-        if ((e = launch_scan_inplace(cnt, nd * nb, spart, st))) return e;
+        k_rs_count<<<(unsigned)nb, RS_THREADS, 0, st>>>(kin, m, shift, nd, w.cnt, nb);
+        if ((e = launch_scan_inplace(w.cnt, nd * nb, w.spart, st))) return e;
         count_launch();
-        k_rs_scatter<<<(unsigned)nb, RS_THREADS, smem, st>>>(kin, vin, kout, vout, m, shift, nd, cnt, nb);
+        k_rs_scatter<<<(unsigned)nb, RS_THREADS, smem, st>>>(kin, vin, kout, vout, m, shift, nd, w.cnt, nb);
         kin = kout;
         vin = vout;
         std::swap(kout, kalt);
@@ -544,17 +542,17 @@ cudaError_t launch_backward_t(const DevCsr& A, const DevCsr& B, long long d, con
     }
     // kin, vin: columns and entry indices sorted by column (stable)
     count_launch();
-    k_col_ptr<<<g256, 256, 0, st>>>(kin, m, n, (unsigned)((1ull << bits) - 1), ATp);
+    k_col_ptr<<<g256, 256, 0, st>>>(kin, m, n, (unsigned)((1ull << bits) - 1), w.ATp);
     // rows and values of the sorted entries (into the free sort buffers)
     int* ti = kout;
     float* ta = reinterpret_cast<float*>(vout);
     count_launch();
-    k_t_gather<<<g256, 256, 0, st>>>(m, vin, row_of, A.val, ti, ta);
+    k_t_gather<<<g256, 256, 0, st>>>(m, vin, w.row_of, A.val, ti, ta);
     if ((e = cudaMemsetAsync(&hdr->scratch[4], 0, 2 * sizeof(long long), st))) return e;
     TParams p;
     p.n = n;
     p.d = (int)d;
-    p.ATp = ATp;
+    p.ATp = w.ATp;
     p.ti = ti;
     p.ta = ta;
     p.Bp = B.rowptr;
@@ -565,10 +563,10 @@ cudaError_t launch_backward_t(const DevCsr& A, const DevCsr& B, long long d, con
     p.dC = dC;
     p.nnzC = nnzC;
     p.dB = dB;
-    p.part = part;
-    p.part_cap = part_cap;
-    p.items = (TItem*)cnt;  // the sort is done with its counters
-    p.item_cap = (long long)(cnt_bytes / sizeof(TItem));
+    p.part = w.part;
+    p.part_cap = w.part_cap;
+    p.items = (TItem*)w.cnt;  // the sort is done with its counters
+    p.item_cap = (long long)(w.cnt_bytes / sizeof(TItem));
     p.nitems = (unsigned long long*)&hdr->scratch[4];
     p.hdr = hdr;
     // the bitmaps: in the room given, or in row_of's (no longer needed)
@@ -576,7 +574,7 @@ cudaError_t launch_backward_t(const DevCsr& A, const DevCsr& B, long long d, con
     const size_t need = sizeof(unsigned) * (size_t)n * words;
     unsigned* place = dw > 8 ? nullptr
                       : bits_room && bits_bytes >= need ? (unsigned*)bits_room
-                      : sizeof(int) * (size_t)m >= need ? (unsigned*)row_of : nullptr;
+                      : sizeof(int) * (size_t)m >= need ? (unsigned*)w.row_of : nullptr;
     p.bits = place;
     if (!place) return launch_pulls<SearchPlaces>(p, m, st);
     switch (words) {
