@@ -15,6 +15,7 @@
 #include "../../include/tsspgemm.h"
 #include "kernels.h"
 #include "layout.h"
+#include "queues.h"
 
 using namespace ts;
 

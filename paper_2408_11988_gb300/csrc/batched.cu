@@ -28,6 +28,7 @@
 #include "common.cuh"
 #include "denseb.cuh"
 #include "kernels.h"
+#include "queues.h"
 #include "numeric.cuh"
 #include "rowgroup.cuh"
 #include "wide.cuh"

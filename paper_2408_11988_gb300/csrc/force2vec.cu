@@ -34,6 +34,7 @@
 // more than 32 terms 108, and 670 against 602 us for 65,536 rows.)
 #include "common.cuh"
 #include "kernels.h"
+#include "queues.h"
 
 namespace ts {
 

@@ -14,7 +14,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 PROGRAM = textwrap.dedent(r"""
     #include <cstdio>
     #include <vector>
-    #include "layout.h"
+    #include "queues.h"
     using namespace ts;
     // reads: chunk offset of the first instance, their number, their rows; prints the blocks, then (instance,
     // tile) of each block that has rows or is its instance's first

@@ -15,7 +15,7 @@ LONGEST = 2**31 - 1
 
 PROGRAM = textwrap.dedent(r"""
     #include <cstdio>
-    #include "layout.h"
+    #include "queues.h"
     using namespace ts;
     int main() {
         long long r, c;
