@@ -910,8 +910,8 @@ static cudaError_t launch_pull(BfsParams p, const DevCsr& F, unsigned* fb, const
 // of every level).  A level that starts with an empty frontier ends at once.
 // Buffers by level: frontier bitmaps modulo 2, non-empty bits modulo 3 (one
 // is read, one added to, one cleared), counters modulo 2 * BFS_GROUP.
-// The 128-source search of the scale-20 graph: 2.11 -> 1.26 ms (steps as
-// above, from Python); the trees of 50 sources, 300,007 vertices: 1.09 -> 0.64.
+// The 128-source search of the scale-20 graph: 2.11 -> 1.29 ms (steps as
+// above, from Python); the trees of 50 sources, 300,007 vertices: 1.09 -> 0.68.
 // ---------------------------------------------------------------------------
 constexpr int BFS_GROUP = 4;
 

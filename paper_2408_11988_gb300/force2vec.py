@@ -1,8 +1,8 @@
 """Sparse Force2Vec training on the f2v_step kernels (paper Sec. IV, sparse
 embedding): minibatch SGD with attractive forces along the graph's edges and
-repulsive forces from negative samples, the force product run as this
-library's TS-SpGEMM, and each updated row sparsified to its k largest
-entries.  This module only marshals tensors to the C ABI."""
+repulsive forces from negative samples, each row's forces summed as they are
+gathered (the product W * Z without forming W), and each updated row sparsified
+to its k largest entries.  This module only marshals tensors to the C ABI."""
 from __future__ import annotations
 
 import ctypes

@@ -1,4 +1,5 @@
-"""Multi-source BFS (paper Alg. 3) on the msbfs_init / msbfs_step kernels."""
+"""Multi-source BFS (paper Alg. 3): the whole search by msbfs_search for up to 256
+sources, level by level by msbfs_init and msbfs_step above."""
 from __future__ import annotations
 
 import ctypes
